@@ -16,6 +16,7 @@
 // (diagonal) or scale one side only (diagonal with a 1 on the other side).
 #pragma once
 
+#include "k_fx.cuh"
 #include "qs_debug.cuh"
 #include "qs_internal.cuh"
 
@@ -60,7 +61,11 @@ template <> struct Vec<double, 2> {
     __device__ __forceinline__ static void st(double2 *p, const double2 *v) { p[0] = v[0]; p[1] = v[1]; }
 };
 
-// Device copy of a gate: index map in the index width, matrix in the state's precision.
+// Device copy of a gate: index map in the index width, matrix in the state's precision
+// (complex128: also in limbs, k_fx.cuh).
+struct NoFx {};
+template <typename Real> struct FxOf { using T = NoFx; };
+template <> struct FxOf<double> { using T = FxMat; };
 template <typename Real, typename Idx> struct DevGate {
     Idx mask[kMaxSeg];
     Idx ins;
@@ -69,6 +74,7 @@ template <typename Real, typename Idx> struct DevGate {
     Idx cvals;
     int32_t shift[kMaxSeg];
     Real m[8];  // a, b, c, d as (re, im)
+    typename FxOf<Real>::T fx;
 };
 
 template <typename Idx, int NS, typename G>
@@ -117,6 +123,62 @@ __device__ __forceinline__ void pair_update(T2 &x, T2 &y, const Real *m) {
     } else if (OP == OP_DIAG) {
         x = cmul<T2, Real>(m[0], m[1], x);
         y = cmul<T2, Real>(m[6], m[7], y);
+    }
+}
+
+// The update of one pair (one-sided: one amplitude) with the gate's matrix. complex64: float32
+// arithmetic. complex128: fixed point where the numbers allow it, float64 arithmetic otherwise
+// (k_fx.cuh); a pair of zeros needs neither.
+template <int OP, typename Idx>
+__device__ __forceinline__ void gate_pair(float2 &x, float2 &y, const DevGate<float, Idx> &g) {
+    pair_update<OP == OP_GENW ? (int)OP_GEN : OP, float2, float>(x, y, g.m);
+}
+template <typename Idx>
+__device__ __forceinline__ void gate_side(float2 &x, const DevGate<float, Idx> &g) {
+    x = cmul<float2, float>(g.m[0], g.m[1], x);
+}
+template <typename Idx>
+__device__ __forceinline__ void gate_side(double2 &x, const DevGate<double, Idx> &g) {
+    if (!fx::mul<0>(x, g.fx) && (fx::nonzero(x.x) || fx::nonzero(x.y))) x = cmul<double2, double>(g.m[0], g.m[1], x);
+}
+template <int OP, typename Idx>
+__device__ __forceinline__ void gate_pair(double2 &x, double2 &y, const DevGate<double, Idx> &g) {
+    if (OP == OP_SWAP) {
+        pair_update<OP, double2, double>(x, y, g.m);
+    } else if (OP == OP_GEN || OP == OP_GENW) {
+        if (!(OP == OP_GEN ? fx::gen(x, y, g.fx) : fx::genw(x, y, g.fx)) &&
+            (fx::nonzero(x.x) || fx::nonzero(x.y) || fx::nonzero(y.x) || fx::nonzero(y.y)))
+            pair_update<OP_GEN, double2, double>(x, y, g.m);
+    } else if (OP == OP_REAL) {
+        if (!fx::real(x.x, y.x, g.fx) && (fx::nonzero(x.x) || fx::nonzero(y.x))) {
+            const double nx = fma(g.m[0], x.x, g.m[2] * y.x);
+            y.x = fma(g.m[4], x.x, g.m[6] * y.x);
+            x.x = nx;
+        }
+        if (!fx::real(x.y, y.y, g.fx) && (fx::nonzero(x.y) || fx::nonzero(y.y))) {
+            const double nx = fma(g.m[0], x.y, g.m[2] * y.y);
+            y.y = fma(g.m[4], x.y, g.m[6] * y.y);
+            x.y = nx;
+        }
+    } else if (OP == OP_DIAG) {
+        if (!fx::mul<0>(x, g.fx) && (fx::nonzero(x.x) || fx::nonzero(x.y))) x = cmul<double2, double>(g.m[0], g.m[1], x);
+        if (!fx::mul<3>(y, g.fx) && (fx::nonzero(y.x) || fx::nonzero(y.y))) y = cmul<double2, double>(g.m[6], g.m[7], y);
+    }
+}
+// Masked comparator: the class of the matrix is read at run time, so that it runs the arithmetic
+// of the reduced schedule (the two give the same bits).
+template <typename Idx>
+__device__ __forceinline__ void gate_pair_any(float2 &x, float2 &y, const DevGate<float, Idx> &g, int) {
+    pair_update<OP_GEN, float2, float>(x, y, g.m);
+}
+template <typename Idx>
+__device__ __forceinline__ void gate_pair_any(double2 &x, double2 &y, const DevGate<double, Idx> &g, int side) {
+    switch (g.fx.form) {
+    case FX_GEN: gate_pair<OP_GEN>(x, y, g); break;
+    case FX_GENW: gate_pair<OP_GENW>(x, y, g); break;
+    case FX_REAL: gate_pair<OP_REAL>(x, y, g); break;
+    case FX_DIAG: gate_pair<OP_DIAG>(x, y, g); break;
+    default: gate_side(side ? y : x, g); break;
     }
 }
 
@@ -201,17 +263,23 @@ k_gate(typename CxT<Real>::T *__restrict__ psi, const DevGate<Real, Idx> g, Idx 
             if (!on[k]) continue;
             if (LAY == LAY_ADJ) {
 #pragma unroll
-                for (int i = 0; i < R; ++i) pair_update<OP, T2, Real>(x[k][2 * i], x[k][2 * i + 1], g.m);
+                for (int i = 0; i < R; ++i) {
+                    if (MASKED) gate_pair_any(x[k][2 * i], x[k][2 * i + 1], g, side);
+                    else gate_pair<OP>(x[k][2 * i], x[k][2 * i + 1], g);
+                }
                 Vec<Real, A>::st(psi + lo[k], x[k]);
                 QS_DBG_WRITE(lo[k], A);
             } else if (OP == OP_SIDE) {
 #pragma unroll
-                for (int i = 0; i < R; ++i) x[k][i] = cmul<T2, Real>(g.m[0], g.m[1], x[k][i]);
+                for (int i = 0; i < R; ++i) gate_side(x[k][i], g);
                 Vec<Real, R>::st(psi + (lo[k] | (side ? g.tbit : (Idx)0)), x[k]);
                 QS_DBG_WRITE(lo[k] | (side ? g.tbit : (Idx)0), R);
             } else {
 #pragma unroll
-                for (int i = 0; i < R; ++i) pair_update<OP, T2, Real>(x[k][i], y[k][i], g.m);
+                for (int i = 0; i < R; ++i) {
+                    if (MASKED) gate_pair_any(x[k][i], y[k][i], g, side);
+                    else gate_pair<OP>(x[k][i], y[k][i], g);
+                }
                 Vec<Real, R>::st(psi + lo[k], x[k]);
                 Vec<Real, R>::st(psi + (lo[k] | g.tbit), y[k]);
                 QS_DBG_WRITE(lo[k], R);

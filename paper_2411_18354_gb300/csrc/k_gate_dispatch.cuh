@@ -25,6 +25,13 @@ DevGate<Real, Idx> make_dev(const GatePlan &p, uint64_t cmask, uint64_t cvals) {
     return g;
 }
 
+inline void set_fx(DevGate<float, uint32_t> &, const FxMat &) {}
+inline void set_fx(DevGate<float, uint64_t> &, const FxMat &) {}
+template <typename Idx>
+void set_fx(DevGate<double, Idx> &g, const FxMat &fx) {
+    g.fx = fx;
+}
+
 template <typename K>
 int occupancy_of(K kern) {
     int occ = 0;
@@ -34,9 +41,11 @@ int occupancy_of(K kern) {
 }
 
 template <typename Real, typename Idx, int NS, int LAY, int R, int OP, bool MASKED>
-cudaError_t go(void *psi, const GatePlan &p, uint64_t cmask, uint64_t cvals, cudaStream_t st) {
-    // units in flight per thread: 2 with a vector on each side, 4 with one vector per unit
-    constexpr int UNR = (LAY == LAY_ADJ || OP == OP_SIDE) ? 4 : 2;
+cudaError_t go(void *psi, const GatePlan &p, const FxMat &fx, uint64_t cmask, uint64_t cvals, cudaStream_t st) {
+    // units in flight per thread: 2 with a vector on each side, 4 with one vector per unit;
+    // complex128 has one 16-byte vector per amplitude and more arithmetic to hide them behind
+    constexpr int UNR = sizeof(Real) == 8 ? (OP == OP_GEN || OP == OP_SIDE || OP == OP_SWAP ? 2 : 1)
+                                          : (LAY == LAY_ADJ || OP == OP_SIDE) ? 4 : 2;
     auto kern = k_gate<Real, Idx, NS, LAY, R, OP, MASKED, UNR>;
     static const int occ = occupancy_of(kern);
     const uint64_t per_block = (uint64_t)kGateThreads * UNR;
@@ -58,21 +67,24 @@ cudaError_t go(void *psi, const GatePlan &p, uint64_t cmask, uint64_t cvals, cud
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = dependent ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, reinterpret_cast<T2 *>(psi), make_dev<Real, Idx>(p, cmask, cvals),
-                              (Idx)p.units, p.side);
+    DevGate<Real, Idx> g = make_dev<Real, Idx>(p, cmask, cvals);
+    set_fx(g, fx);
+    return cudaLaunchKernelEx(&cfg, kern, reinterpret_cast<T2 *>(psi), g, (Idx)p.units, p.side);
 }
 
 template <typename Real, typename Idx, int NS, bool MASKED>
-cudaError_t by_shape(void *psi, const GatePlan &p, uint64_t cmask, uint64_t cvals, cudaStream_t st) {
+cudaError_t by_shape(void *psi, const GatePlan &p, const FxMat &fx, uint64_t cmask, uint64_t cvals, cudaStream_t st) {
     constexpr bool F = sizeof(Real) == 4;
-    const int op = MASKED ? (int)OP_GEN : p.op;
+    int op = MASKED ? (int)OP_GEN : p.op;
+    if (!F && !MASKED && op == OP_GEN && fx.form == FX_GENW) op = OP_GENW;
 #define QS_OPS(LAY, R)                                                                        \
     switch (op) {                                                                             \
-        case OP_GEN: return go<Real, Idx, NS, LAY, R, OP_GEN, MASKED>(psi, p, cmask, cvals, st); \
-        case OP_REAL: if (!MASKED) return go<Real, Idx, NS, LAY, R, OP_REAL, false>(psi, p, cmask, cvals, st); break; \
-        case OP_SWAP: if (!MASKED) return go<Real, Idx, NS, LAY, R, OP_SWAP, false>(psi, p, cmask, cvals, st); break; \
-        case OP_DIAG: if (!MASKED) return go<Real, Idx, NS, LAY, R, OP_DIAG, false>(psi, p, cmask, cvals, st); break; \
-        case OP_SIDE: if (!MASKED && LAY == LAY_SPLIT) return go<Real, Idx, NS, LAY_SPLIT, R, OP_SIDE, false>(psi, p, cmask, cvals, st); break; \
+        case OP_GEN: return go<Real, Idx, NS, LAY, R, OP_GEN, MASKED>(psi, p, fx, cmask, cvals, st); \
+        case OP_GENW: if (!MASKED && !F) return go<Real, Idx, NS, LAY, R, F ? OP_GEN : OP_GENW, false>(psi, p, fx, cmask, cvals, st); break; \
+        case OP_REAL: if (!MASKED) return go<Real, Idx, NS, LAY, R, OP_REAL, false>(psi, p, fx, cmask, cvals, st); break; \
+        case OP_SWAP: if (!MASKED) return go<Real, Idx, NS, LAY, R, OP_SWAP, false>(psi, p, fx, cmask, cvals, st); break; \
+        case OP_DIAG: if (!MASKED) return go<Real, Idx, NS, LAY, R, OP_DIAG, false>(psi, p, fx, cmask, cvals, st); break; \
+        case OP_SIDE: if (!MASKED && LAY == LAY_SPLIT) return go<Real, Idx, NS, LAY_SPLIT, R, OP_SIDE, false>(psi, p, fx, cmask, cvals, st); break; \
         default: break;                                                                       \
     }
     if (p.layout == LAY_SPLIT) {
@@ -86,12 +98,12 @@ cudaError_t by_shape(void *psi, const GatePlan &p, uint64_t cmask, uint64_t cval
 }
 
 template <typename Real, typename Idx, bool MASKED>
-cudaError_t by_nseg(void *psi, const GatePlan &p, uint64_t cmask, uint64_t cvals, cudaStream_t st) {
+cudaError_t by_nseg(void *psi, const GatePlan &p, const FxMat &fx, uint64_t cmask, uint64_t cvals, cudaStream_t st) {
     const int ns = p.map.nseg;
-    if (ns <= 2) return by_shape<Real, Idx, 2, MASKED>(psi, p, cmask, cvals, st);
-    if (ns <= 4) return by_shape<Real, Idx, 4, MASKED>(psi, p, cmask, cvals, st);
-    if (ns <= 10) return by_shape<Real, Idx, 10, MASKED>(psi, p, cmask, cvals, st);
-    return by_shape<Real, Idx, kMaxSeg, MASKED>(psi, p, cmask, cvals, st);
+    if (ns <= 2) return by_shape<Real, Idx, 2, MASKED>(psi, p, fx, cmask, cvals, st);
+    if (ns <= 4) return by_shape<Real, Idx, 4, MASKED>(psi, p, fx, cmask, cvals, st);
+    if (ns <= 10) return by_shape<Real, Idx, 10, MASKED>(psi, p, fx, cmask, cvals, st);
+    return by_shape<Real, Idx, kMaxSeg, MASKED>(psi, p, fx, cmask, cvals, st);
 }
 
 template <typename Real>
@@ -99,11 +111,26 @@ cudaError_t launch(void *psi, const GatePlan &p, bool masked, uint64_t cmask, ui
                    cudaStream_t st) {
     if (p.units == 0) return cudaSuccess;
     const bool narrow = p.n <= 32;  // every amplitude index fits in 32 bits
+    FxMat fx;
+    GatePlan masked_plan;
+    const GatePlan *pp = &p;
+    if (sizeof(Real) == 8) {
+        if (!masked) {
+            make_fx(p.U, p.op, &fx);
+        } else {
+            // the comparator runs the arithmetic of the class its matrix has (k_fx.cuh)
+            masked_plan = p;
+            make_fx_full(p.U, &fx, &masked_plan.side);
+            if (fx.form == FX_SIDE && masked_plan.side)  // the scalar where the kernel reads it
+                for (int i = 0; i < 2; ++i) masked_plan.U[i] = p.U[6 + i];
+            pp = &masked_plan;
+        }
+    }
     if (masked)
-        return narrow ? by_nseg<Real, uint32_t, true>(psi, p, cmask, cvals, st)
-                      : by_nseg<Real, uint64_t, true>(psi, p, cmask, cvals, st);
-    return narrow ? by_nseg<Real, uint32_t, false>(psi, p, cmask, cvals, st)
-                  : by_nseg<Real, uint64_t, false>(psi, p, cmask, cvals, st);
+        return narrow ? by_nseg<Real, uint32_t, true>(psi, *pp, fx, cmask, cvals, st)
+                      : by_nseg<Real, uint64_t, true>(psi, *pp, fx, cmask, cvals, st);
+    return narrow ? by_nseg<Real, uint32_t, false>(psi, *pp, fx, cmask, cvals, st)
+                  : by_nseg<Real, uint64_t, false>(psi, *pp, fx, cmask, cvals, st);
 }
 
 }  // namespace gate_detail

@@ -1,18 +1,23 @@
 // k_adjoint.cu -- adjoint (reverse-sweep) gradient kernels.
 //
 // For E = <psi|O|psi>, psi = U_G ... U_1 |psi_in>, O = sum_i Z_i:
-//   lambda = O psi;  for g = G .. 1:  psi <- U_g^dagger psi;
-//                                     if g has a parameter: grad += 2 Re <lambda| dU_g psi>;
-//                                     lambda <- U_g^dagger lambda.
+//   lambda = O psi;  for g = G .. 1:  if g has a parameter: grad += 2 Re <lambda| dU_g U_g^dagger psi>;
+//                                     psi <- U_g^dagger psi;  lambda <- U_g^dagger lambda.
 // No intermediate state is stored: un-applying a unitary gate recovers the state before
 // it. One kernel does the three steps of one gate on the gate's reduced iteration set
 // (the 2^(n-1-c) control-satisfied pairs, Section III-B of arXiv 2411.18354), reading
-// and writing psi and lambda once. The inner product is summed per thread in the state's
+// and writing psi and lambda once. A parameterised gate is a rotation exp(-i theta P / 2) about
+// P = Y or Z, so dU U^dagger = (-i / 2) P and the inner product is Im <lambda| P psi> / 2, taken from
+// the pair before the un-apply: four products per pair. It is summed per thread in the state's
 // precision, per warp and block in float64, and per block written to a fixed slot; a
 // final pass adds the slots in a fixed order.
+//
+// complex128 un-applies in fixed point (k_fx.cuh): in float64 arithmetic a step took 28 operations
+// per pair, 14 SM clocks against 5.4 of memory time and less from the L2. n = 20 (psi and lambda in
+// the L2), 8-layer ansatz gradient with its 320 rotation steps: 16.6 -> 8.1 ms.
 #include <algorithm>
 
-#include "k_gate.cuh"
+#include "k_gate_dispatch.cuh"
 #include "qs_debug.cuh"
 
 namespace qs {
@@ -21,16 +26,19 @@ constexpr int kAdjMaxBlocks = 1024;
 
 namespace {
 
-template <typename Real> struct DevMat { Real m[8]; };
+enum : int { PAULI_NONE = 0, PAULI_Y = 1, PAULI_Z = 2 };
 
-template <typename Real, typename Idx, int NS, int LAY, int R, int OP, bool PARAM>
+template <typename Real, typename Idx, int NS, int LAY, int R, int OP, int PAULI>
 __global__ void __launch_bounds__(kGateThreads)
 k_adj_step(typename CxT<Real>::T *__restrict__ psi, typename CxT<Real>::T *__restrict__ lam,
-           const DevGate<Real, Idx> g, const DevMat<Real> du, Idx units, double *__restrict__ part) {
+           const DevGate<Real, Idx> g, Idx units, double *__restrict__ part) {
     using T2 = typename CxT<Real>::T;
     constexpr int r = Log2<R>::v;
     constexpr int A = (LAY == LAY_ADJ) ? 2 * R : R;
-    constexpr int DOP = (OP == OP_DIAG) ? OP_DIAG : (OP == OP_REAL) ? OP_REAL : OP_GEN;  // structure of dU
+    // programmatic dependent launch as in k_gate: nothing is touched before the previous kernel
+    // on the stream has completed
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     Real acc = 0;
     const Idx step = (Idx)gridDim.x * kGateThreads;
     for (Idx u = (Idx)blockIdx.x * kGateThreads + threadIdx.x; u < units; u += step) {
@@ -52,13 +60,19 @@ k_adj_step(typename CxT<Real>::T *__restrict__ psi, typename CxT<Real>::T *__res
             T2 &y = (LAY == LAY_ADJ) ? px[2 * i + 1] : py[i];
             T2 &a = (LAY == LAY_ADJ) ? lx[2 * i] : lx[i];
             T2 &b = (LAY == LAY_ADJ) ? lx[2 * i + 1] : ly[i];
-            pair_update<OP, T2, Real>(x, y, g.m);  // psi <- U^dagger psi
-            if (PARAM) {
-                T2 mx = x, my = y;
-                pair_update<DOP, T2, Real>(mx, my, du.m);  // mu = dU psi
-                acc += a.x * mx.x + a.y * mx.y + b.x * my.x + b.y * my.y;  // Re <lambda|mu>
+            if (PAULI == PAULI_Y) {  // Im <l|Y p> = (b . x) - (a . y), real dot products
+                acc = fma(b.x, x.x, acc);
+                acc = fma(b.y, x.y, acc);
+                acc = fma(-a.x, y.x, acc);
+                acc = fma(-a.y, y.y, acc);
+            } else if (PAULI == PAULI_Z) {  // Im(conj(a) x) - Im(conj(b) y)
+                acc = fma(a.x, x.y, acc);
+                acc = fma(-a.y, x.x, acc);
+                acc = fma(-b.x, y.y, acc);
+                acc = fma(b.y, y.x, acc);
             }
-            pair_update<OP, T2, Real>(a, b, g.m);  // lambda <- U^dagger lambda
+            gate_pair<OP>(x, y, g);  // psi <- U^dagger psi
+            gate_pair<OP>(a, b, g);  // lambda <- U^dagger lambda
         }
         if (LAY == LAY_ADJ) {
             Vec<Real, A>::st(psi + lo, px);
@@ -73,7 +87,7 @@ k_adj_step(typename CxT<Real>::T *__restrict__ psi, typename CxT<Real>::T *__res
             Vec<Real, R>::st(lam + (lo | g.tbit), ly);
         }
     }
-    if (PARAM) {
+    if (PAULI != PAULI_NONE) {
         __shared__ double wsum[kGateThreads / 32];
         double v = (double)acc;
 #pragma unroll
@@ -83,7 +97,7 @@ k_adj_step(typename CxT<Real>::T *__restrict__ psi, typename CxT<Real>::T *__res
         if (threadIdx.x == 0) {
             double s = 0.0;
             for (int w = 0; w < kGateThreads / 32; ++w) s += wsum[w];
-            part[blockIdx.x] = s;
+            part[blockIdx.x] = 0.5 * s;
         }
     }
 }
@@ -124,15 +138,20 @@ __global__ void k_slot_sums(const double *__restrict__ part, int nslots, double 
     if (lane == 0) slot_sum[s] = v;
 }
 
-// grad[p] = 2 * sum of slot sums whose parameter is p (slots in gate order).
+// grad[p] = 2 * sum of slot sums whose parameter is p: a warp per parameter, lane l looks at slots
+// l, l + 32, ..., then a fixed-order shuffle reduction (a thread per parameter walking all slots
+// took 55 us at 960 slots, 25 us at 320).
 __global__ void k_grad_gather(const double *__restrict__ slot_sum, const int *__restrict__ slot_param, int nslots,
                               double *__restrict__ grad, int nparams) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= nparams) return;
+    const int p = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int lane = threadIdx.x & 31;
+    if (p >= nparams) return;  // uniform over the warp
     double v = 0.0;
-    for (int s = 0; s < nslots; ++s)
+    for (int s = lane; s < nslots; s += 32)
         if (slot_param[s] == p) v += slot_sum[s];
-    grad[p] = 2.0 * v;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) grad[p] = 2.0 * v;
 }
 
 template <typename K>
@@ -142,44 +161,44 @@ int occ_of(K kern) {
     return o;
 }
 
-template <typename Real, typename Idx, int NS, int LAY, int R, int OP, bool PARAM>
-cudaError_t go(void *psi, void *lam, const GatePlan &p, const double *dU, double *part, cudaStream_t st) {
-    auto kern = k_adj_step<Real, Idx, NS, LAY, R, OP, PARAM>;
+template <typename Real, typename Idx, int NS, int LAY, int R, int OP, int PAULI>
+cudaError_t go(void *psi, void *lam, const GatePlan &p, const FxMat &fx, double *part, cudaStream_t st) {
+    auto kern = k_adj_step<Real, Idx, NS, LAY, R, OP, PAULI>;
     static const int occ = occ_of(kern);
     const uint64_t need = (p.units + kGateThreads - 1) / kGateThreads;
     const uint64_t cap = std::min<uint64_t>((uint64_t)device_sm_count() * occ, (uint64_t)kAdjMaxBlocks);
     const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min(need, cap));
-    DevGate<Real, Idx> g;
-    for (int s = 0; s < kMaxSeg; ++s) {
-        g.mask[s] = (Idx)(s < p.map.nseg ? p.map.mask[s] : 0);
-        g.shift[s] = s < p.map.nseg ? p.map.shift[s] : 0;
-    }
-    g.ins = (Idx)p.map.ins;
-    g.tbit = (Idx)p.tbit;
-    g.cmask = 0;
-    g.cvals = 0;
-    for (int i = 0; i < 8; ++i) g.m[i] = (Real)p.U[i];
-    DevMat<Real> d;
-    for (int i = 0; i < 8; ++i) d.m[i] = dU ? (Real)dU[i] : (Real)0;
+    DevGate<Real, Idx> g = gate_detail::make_dev<Real, Idx>(p, 0, 0);
+    gate_detail::set_fx(g, fx);
     using T2 = typename CxT<Real>::T;
-    kern<<<grid, kGateThreads, 0, st>>>(reinterpret_cast<T2 *>(psi), reinterpret_cast<T2 *>(lam), g, d, (Idx)p.units, part);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kGateThreads);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = (p.units << p.r) <= (uint64_t)grid << 15 ? 1 : 0;  // the rule of k_gate
+    return cudaLaunchKernelEx(&cfg, kern, reinterpret_cast<T2 *>(psi), reinterpret_cast<T2 *>(lam), g, (Idx)p.units,
+                              part);
 }
 
 template <typename Real, typename Idx, int NS>
-cudaError_t by_shape(void *psi, void *lam, const GatePlan &p, const double *dU, double *part, cudaStream_t st) {
+cudaError_t by_shape(void *psi, void *lam, const GatePlan &p, const FxMat &fx, double *part, cudaStream_t st) {
     constexpr bool F = sizeof(Real) == 4;
-    const bool param = dU != nullptr;
-#define QS_ADJ_OPS(LAY, R)                                                                            \
-    if (param) {                                                                                      \
-        if (p.op == OP_GEN) return go<Real, Idx, NS, LAY, R, OP_GEN, true>(psi, lam, p, dU, part, st);   \
-        if (p.op == OP_DIAG) return go<Real, Idx, NS, LAY, R, OP_DIAG, true>(psi, lam, p, dU, part, st); \
-        if (p.op == OP_REAL) return go<Real, Idx, NS, LAY, R, OP_REAL, true>(psi, lam, p, dU, part, st); \
-    } else {                                                                                          \
-        if (p.op == OP_REAL) return go<Real, Idx, NS, LAY, R, OP_REAL, false>(psi, lam, p, dU, part, st); \
-        if (p.op == OP_GEN) return go<Real, Idx, NS, LAY, R, OP_GEN, false>(psi, lam, p, dU, part, st);  \
-        if (p.op == OP_DIAG) return go<Real, Idx, NS, LAY, R, OP_DIAG, false>(psi, lam, p, dU, part, st); \
-        if (p.op == OP_SWAP) return go<Real, Idx, NS, LAY, R, OP_SWAP, false>(psi, lam, p, dU, part, st); \
+    int op = p.op;
+    if (!F && op == OP_GEN && fx.form == FX_GENW) op = OP_GENW;
+#define QS_ADJ_OPS(LAY, R)                                                                                     \
+    if (part) {                                                                                                \
+        if (op == OP_DIAG) return go<Real, Idx, NS, LAY, R, OP_DIAG, PAULI_Z>(psi, lam, p, fx, part, st);       \
+        if (op == OP_REAL) return go<Real, Idx, NS, LAY, R, OP_REAL, PAULI_Y>(psi, lam, p, fx, part, st);       \
+    } else {                                                                                                   \
+        if (op == OP_REAL) return go<Real, Idx, NS, LAY, R, OP_REAL, PAULI_NONE>(psi, lam, p, fx, part, st);    \
+        if (op == OP_GEN) return go<Real, Idx, NS, LAY, R, OP_GEN, PAULI_NONE>(psi, lam, p, fx, part, st);      \
+        if (op == OP_GENW) return go<Real, Idx, NS, LAY, R, F ? OP_GEN : OP_GENW, PAULI_NONE>(psi, lam, p, fx, part, st); \
+        if (op == OP_DIAG) return go<Real, Idx, NS, LAY, R, OP_DIAG, PAULI_NONE>(psi, lam, p, fx, part, st);    \
+        if (op == OP_SWAP) return go<Real, Idx, NS, LAY, R, OP_SWAP, PAULI_NONE>(psi, lam, p, fx, part, st);    \
     }
     if (p.layout == LAY_SPLIT) {
         if (p.r == 0) { QS_ADJ_OPS(LAY_SPLIT, 1) }
@@ -192,24 +211,25 @@ cudaError_t by_shape(void *psi, void *lam, const GatePlan &p, const double *dU, 
 }
 
 template <typename Real>
-cudaError_t adj_step_impl(void *psi, void *lam, const GatePlan &p, const double *dU, double *part, cudaStream_t st) {
+cudaError_t adj_step_impl(void *psi, void *lam, const GatePlan &p, double *part, cudaStream_t st) {
     if (p.units == 0) return cudaSuccess;
     const bool narrow = p.n <= 32;
+    FxMat fx;
+    if (sizeof(Real) == 8) make_fx(p.U, p.op, &fx);
     if (p.map.nseg <= 4)
-        return narrow ? by_shape<Real, uint32_t, 4>(psi, lam, p, dU, part, st)
-                      : by_shape<Real, uint64_t, 4>(psi, lam, p, dU, part, st);
-    return narrow ? by_shape<Real, uint32_t, kMaxSeg>(psi, lam, p, dU, part, st)
-                  : by_shape<Real, uint64_t, kMaxSeg>(psi, lam, p, dU, part, st);
+        return narrow ? by_shape<Real, uint32_t, 4>(psi, lam, p, fx, part, st)
+                      : by_shape<Real, uint64_t, 4>(psi, lam, p, fx, part, st);
+    return narrow ? by_shape<Real, uint32_t, kMaxSeg>(psi, lam, p, fx, part, st)
+                  : by_shape<Real, uint64_t, kMaxSeg>(psi, lam, p, fx, part, st);
 }
 
 }  // namespace
 
 size_t adj_partials_per_slot() { return kAdjMaxBlocks; }
 
-cudaError_t launch_adj_step(int dtype, void *psi, void *lam, const GatePlan &p, const double *dU, double *part,
-                            cudaStream_t st) {
-    return dtype == QS_C64 ? adj_step_impl<float>(psi, lam, p, dU, part, st)
-                           : adj_step_impl<double>(psi, lam, p, dU, part, st);
+// part: the gradient slot of a parameterised gate (a rotation: OP_REAL about Y, OP_DIAG about Z).
+cudaError_t launch_adj_step(int dtype, void *psi, void *lam, const GatePlan &p, double *part, cudaStream_t st) {
+    return dtype == QS_C64 ? adj_step_impl<float>(psi, lam, p, part, st) : adj_step_impl<double>(psi, lam, p, part, st);
 }
 
 cudaError_t launch_obs_sumz(int dtype, const void *psi, void *lam, int n, cudaStream_t st) {
@@ -235,7 +255,7 @@ cudaError_t launch_grad_final(const double *part, int nslots, double *slot_sum, 
         if (e != cudaSuccess) return e;
     }
     if (nparams > 0) {
-        k_grad_gather<<<(nparams + 127) / 128, 128, 0, st>>>(slot_sum, slot_param, nslots, grad, nparams);
+        k_grad_gather<<<(nparams + 7) / 8, 256, 0, st>>>(slot_sum, slot_param, nslots, grad, nparams);
         return cudaGetLastError();
     }
     return cudaSuccess;

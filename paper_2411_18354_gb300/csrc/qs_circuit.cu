@@ -18,8 +18,7 @@
 namespace qs {
 
 size_t adj_partials_per_slot();
-cudaError_t launch_adj_step(int dtype, void *psi, void *lam, const GatePlan &p, const double *dU, double *part,
-                            cudaStream_t st);
+cudaError_t launch_adj_step(int dtype, void *psi, void *lam, const GatePlan &p, double *part, cudaStream_t st);
 cudaError_t launch_obs_sumz(int dtype, const void *psi, void *lam, int n, cudaStream_t st);
 cudaError_t launch_sum_vec(const double *z, int n, double *out, cudaStream_t st);
 cudaError_t launch_grad_final(const double *part, int nslots, double *slot_sum, const int *slot_param,
@@ -357,10 +356,9 @@ static qs_status ensure_device(void **buf, size_t *cap, size_t bytes, cudaStream
 }
 
 // Launch a fused program. Forward: `lam` == nullptr. Adjoint: single gates use the sweep
-// kernel with dus[g] / part + slot * P, passes use the adjoint tile kernel.
+// kernel with part + slot * P, passes use the adjoint tile kernel.
 static qs_status launch_program(qs_state *s, const FusedProgram &prog, const std::vector<GatePlan> &plans,
-                                const void *dev_table, void *lam, const std::vector<const double *> *dus,
-                                const std::vector<int> *slots, double *part, size_t P, cudaStream_t st,
+                                const void *dev_table, void *lam, const std::vector<int> *slots, double *part, size_t P, cudaStream_t st,
                                 const std::vector<JitPass> *jit = nullptr) {
     const TileGroup *groups = dev_table ? table_groups(prog, dev_table) : nullptr;
     const RegGate *gates = dev_table ? table_gates(prog, dev_table) : nullptr;
@@ -382,8 +380,7 @@ static qs_status launch_program(qs_state *s, const FusedProgram &prog, const std
             e = launch_gate(s->dtype, s->psi, plans[op.gate], st);
         } else {
             const int slot = (*slots)[op.gate];
-            e = launch_adj_step(s->dtype, s->psi, lam, plans[op.gate], (*dus)[op.gate],
-                                slot >= 0 ? part + (size_t)slot * P : nullptr, st);
+            e = launch_adj_step(s->dtype, s->psi, lam, plans[op.gate], slot >= 0 ? part + (size_t)slot * P : nullptr, st);
         }
         if (e != cudaSuccess) {
             char what[160];
@@ -955,7 +952,7 @@ qs_status qs_apply_circuit(qs_state *s, const qs_gate *gates, size_t count, cons
                                             s->stream);
             if (e != cudaSuccess) return cuda_fail(e, "qs_apply_circuit: gate table upload");
         }
-        return launch_program(s, prog, plans, s->tile_table, nullptr, nullptr, nullptr, nullptr, 0, s->stream, jp);
+        return launch_program(s, prog, plans, s->tile_table, nullptr, nullptr, nullptr, 0, s->stream, jp);
     }
 
     // CUDA graph not recorded yet (the lookup above missed): record it, keep it, launch it.
@@ -987,7 +984,7 @@ qs_status qs_apply_circuit(qs_state *s, const qs_gate *gates, size_t count, cons
             if (table) cudaFree(table);
             return cuda_fail(e, "cudaStreamBeginCapture");
         }
-        qs_status st = fuse ? launch_program(s, prog, plans, table, nullptr, nullptr, nullptr, nullptr, 0,
+        qs_status st = fuse ? launch_program(s, prog, plans, table, nullptr, nullptr, nullptr, 0,
                                              s->capture_stream, jp)
                             : launch_plans(s, plans, s->capture_stream, masked);
         cudaGraph_t graph = nullptr;
@@ -1036,7 +1033,6 @@ qs_status qs_adjoint_grad(qs_state *s, const qs_gate *gates, size_t count, const
     }
     std::vector<GatePlan> &fwd = ap.fwd, &adj = ap.adj;
     std::vector<int> &slot_of = ap.slot_of, &slot_param = ap.slot_param;
-    std::vector<double> &dus = ap.dus;
     std::vector<const double *> &dusp = ap.dusp;
     FusedProgram &pf = ap.pf, &pa = ap.pa;
     const int nslots = (int)slot_param.size();
@@ -1110,7 +1106,7 @@ qs_status qs_adjoint_grad(qs_state *s, const qs_gate *gates, size_t count, const
     const void *tab_f = s->tile_table;
     const void *tab_a = tab_f ? static_cast<const char *>(tab_f) + bf : nullptr;
     // Forward pass.
-    st = fuse ? launch_program(s, pf, fwd, tab_f, nullptr, nullptr, nullptr, nullptr, 0, stm, use_jit ? &jf : nullptr)
+    st = fuse ? launch_program(s, pf, fwd, tab_f, nullptr, nullptr, nullptr, 0, stm, use_jit ? &jf : nullptr)
               : launch_plans(s, fwd, stm);
     if (st != QS_OK) return st;
     // Energy and lambda = O psi.
@@ -1125,13 +1121,12 @@ qs_status qs_adjoint_grad(qs_state *s, const qs_gate *gates, size_t count, const
     if (e != cudaSuccess) return cuda_fail(e, "qs_adjoint_grad setup");
     // Reverse sweep.
     if (fuse) {
-        st = launch_program(s, pa, adj, tab_a, s->lam, &dusp, &slot_of, part, P, stm, use_jit ? &ja : nullptr);
+        st = launch_program(s, pa, adj, tab_a, s->lam, &slot_of, part, P, stm, use_jit ? &ja : nullptr);
         if (st != QS_OK) return st;
     } else {
         for (size_t ii = count; ii-- > 0;) {
             const int slot = slot_of[ii];
-            e = launch_adj_step(s->dtype, s->psi, s->lam, adj[ii], slot >= 0 ? &dus[8 * slot] : nullptr,
-                                slot >= 0 ? part + (size_t)slot * P : nullptr, stm);
+            e = launch_adj_step(s->dtype, s->psi, s->lam, adj[ii], slot >= 0 ? part + (size_t)slot * P : nullptr, stm);
             if (e != cudaSuccess) return cuda_fail(e, "qs_adjoint_grad sweep launch");
         }
     }

@@ -31,7 +31,7 @@ enum : int { PAULI_NONE = 0, PAULI_Y = 1, PAULI_Z = 2 };
 template <typename Real, typename Idx, int NS, int LAY, int R, int OP, int PAULI>
 __global__ void __launch_bounds__(kGateThreads)
 k_adj_step(typename CxT<Real>::T *__restrict__ psi, typename CxT<Real>::T *__restrict__ lam,
-           const DevGate<Real, Idx> g, Idx units, double *__restrict__ part) {
+           const DevGate<Real, Idx> g, Idx units, int side, double *__restrict__ part) {
     using T2 = typename CxT<Real>::T;
     constexpr int r = Log2<R>::v;
     constexpr int A = (LAY == LAY_ADJ) ? 2 * R : R;
@@ -43,6 +43,26 @@ k_adj_step(typename CxT<Real>::T *__restrict__ psi, typename CxT<Real>::T *__res
     const Idx step = (Idx)gridDim.x * kGateThreads;
     for (Idx u = (Idx)blockIdx.x * kGateThreads + threadIdx.x; u < units; u += step) {
         const Idx lo = deposit<Idx, NS>(u << r, g);
+        if (OP == OP_SIDE) {  // the side that changes
+            const Idx k = lo | (side ? g.tbit : (Idx)0);
+            if (!QS_DBG_OK(k, R)) continue;
+            T2 x[R], a[R];
+            Vec<Real, R>::ld(psi + k, x);
+            Vec<Real, R>::ld(lam + k, a);
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                if (PAULI == PAULI_Z) {  // Im(conj(a) x), doubled below
+                    acc = fma(a[i].x, x[i].y, acc);
+                    acc = fma(-a[i].y, x[i].x, acc);
+                }
+                gate_side(x[i], g);
+                gate_side(a[i], g);
+            }
+            Vec<Real, R>::st(psi + k, x);
+            Vec<Real, R>::st(lam + k, a);
+            QS_DBG_WRITE(k, R);
+            continue;
+        }
         if (LAY == LAY_ADJ ? !QS_DBG_OK(lo, A) : (!QS_DBG_OK(lo, R) || !QS_DBG_OK(lo | g.tbit, R))) continue;
         T2 px[A], py[(LAY == LAY_SPLIT) ? R : 1], lx[A], ly[(LAY == LAY_SPLIT) ? R : 1];
         if (LAY == LAY_ADJ) {
@@ -97,7 +117,8 @@ k_adj_step(typename CxT<Real>::T *__restrict__ psi, typename CxT<Real>::T *__res
         if (threadIdx.x == 0) {
             double s = 0.0;
             for (int w = 0; w < kGateThreads / 32; ++w) s += wsum[w];
-            part[blockIdx.x] = 0.5 * s;
+            // one side of a Z rotation stands for both (Im <lambda|psi> = 0); side 1 counts negative
+            part[blockIdx.x] = OP == OP_SIDE ? (side ? -s : s) : 0.5 * s;
         }
     }
 }
@@ -181,7 +202,7 @@ cudaError_t go(void *psi, void *lam, const GatePlan &p, const FxMat &fx, double 
     cfg.attrs = attr;
     cfg.numAttrs = (p.units << p.r) <= (uint64_t)grid << 15 ? 1 : 0;  // the rule of k_gate
     return cudaLaunchKernelEx(&cfg, kern, reinterpret_cast<T2 *>(psi), reinterpret_cast<T2 *>(lam), g, (Idx)p.units,
-                              part);
+                              p.side, part);
 }
 
 template <typename Real, typename Idx, int NS>
@@ -193,12 +214,16 @@ cudaError_t by_shape(void *psi, void *lam, const GatePlan &p, const FxMat &fx, d
     if (part) {                                                                                                \
         if (op == OP_DIAG) return go<Real, Idx, NS, LAY, R, OP_DIAG, PAULI_Z>(psi, lam, p, fx, part, st);       \
         if (op == OP_REAL) return go<Real, Idx, NS, LAY, R, OP_REAL, PAULI_Y>(psi, lam, p, fx, part, st);       \
+        if (op == OP_SIDE && LAY == LAY_SPLIT)                                                                 \
+            return go<Real, Idx, NS, LAY_SPLIT, R, OP_SIDE, PAULI_Z>(psi, lam, p, fx, part, st);                \
     } else {                                                                                                   \
         if (op == OP_REAL) return go<Real, Idx, NS, LAY, R, OP_REAL, PAULI_NONE>(psi, lam, p, fx, part, st);    \
         if (op == OP_GEN) return go<Real, Idx, NS, LAY, R, OP_GEN, PAULI_NONE>(psi, lam, p, fx, part, st);      \
         if (op == OP_GENW) return go<Real, Idx, NS, LAY, R, F ? OP_GEN : OP_GENW, PAULI_NONE>(psi, lam, p, fx, part, st); \
         if (op == OP_DIAG) return go<Real, Idx, NS, LAY, R, OP_DIAG, PAULI_NONE>(psi, lam, p, fx, part, st);    \
         if (op == OP_SWAP) return go<Real, Idx, NS, LAY, R, OP_SWAP, PAULI_NONE>(psi, lam, p, fx, part, st);    \
+        if (op == OP_SIDE && LAY == LAY_SPLIT)                                                                 \
+            return go<Real, Idx, NS, LAY_SPLIT, R, OP_SIDE, PAULI_NONE>(psi, lam, p, fx, part, st);             \
     }
     if (p.layout == LAY_SPLIT) {
         if (p.r == 0) { QS_ADJ_OPS(LAY_SPLIT, 1) }
@@ -227,7 +252,7 @@ cudaError_t adj_step_impl(void *psi, void *lam, const GatePlan &p, double *part,
 
 size_t adj_partials_per_slot() { return kAdjMaxBlocks; }
 
-// part: the gradient slot of a parameterised gate (a rotation: OP_REAL about Y, OP_DIAG about Z).
+// part: the gradient slot of a parameterised gate (a rotation: OP_REAL about Y, OP_DIAG and OP_SIDE about Z).
 cudaError_t launch_adj_step(int dtype, void *psi, void *lam, const GatePlan &p, double *part, cudaStream_t st) {
     return dtype == QS_C64 ? adj_step_impl<float>(psi, lam, p, part, st) : adj_step_impl<double>(psi, lam, p, part, st);
 }

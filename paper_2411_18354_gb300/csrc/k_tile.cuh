@@ -43,9 +43,7 @@ struct RegGate {
     int32_t pad1;
     uint64_t hmask, hvals;    // non-local controls: the tile predicate (global bits)
     double U[8];              // forward: U; adjoint: U^dagger
-    double D[8];              // adjoint: dU/dtheta (parameterised gates)
     float Uf[8];              // the same, rounded once to float32 for complex64 states
-    float Df[8];
 };
 
 // A register group: which local qubits are in registers, how a row number becomes a local

@@ -16,7 +16,6 @@ template <> struct TileT<float> {
     static constexpr int VEC = 2;
     static constexpr int SW = 4;  // 16 amplitudes of 8 bytes per 128-byte bank row
     __device__ static const float *U(const RegGate &G) { return G.Uf; }
-    __device__ static const float *D(const RegGate &G) { return G.Df; }
 };
 template <> struct TileT<double> {
     using T2 = double2;
@@ -24,7 +23,6 @@ template <> struct TileT<double> {
     static constexpr int VEC = 1;
     static constexpr int SW = 3;  // 8 amplitudes of 16 bytes per bank row
     __device__ static const double *U(const RegGate &G) { return G.U; }
-    __device__ static const double *D(const RegGate &G) { return G.D; }
 };
 
 // Compact copy of a RegGate in shared memory (matrices in the state's precision), staged once
@@ -34,11 +32,11 @@ template <typename Real> struct alignas(16) SGate {
     // crm, crv, meta, pidx -- one 16-byte load; meta = code | cqm << 8 | cqv << 12 | side << 16 |
     // pkind << 17 | (slot + 1) << 20, code = (op * 4 + p) * 2 + (cqm != 0)
     uint32_t crm, crv, meta, pidx;
-    Real u[8], d[8];
+    Real u[8];
 };
 
 template <typename Real>
-__device__ __forceinline__ void param_matrices(int kind, Real c, Real s, bool adjoint, Real *u, Real *d);
+__device__ __forceinline__ void param_matrices(int kind, Real c, Real s, bool adjoint, Real *u);
 
 template <typename Real>
 __device__ __forceinline__ void stage_gate(const RegGate &G, SGate<Real> &S, const Real *cs, bool adjoint) {
@@ -50,10 +48,10 @@ __device__ __forceinline__ void stage_gate(const RegGate &G, SGate<Real> &S, con
     int pkind = G.pkind;
     S.pidx = (uint32_t)G.pidx;
     if (G.pkind != 0 && cs) {  // the state's parameter: matrices built once per pass
-        param_matrices<Real>(G.pkind, cs[2 * G.pidx], cs[2 * G.pidx + 1], adjoint, S.u, S.d);
+        param_matrices<Real>(G.pkind, cs[2 * G.pidx], cs[2 * G.pidx + 1], adjoint, S.u);
         if (G.pkind2 != 0) {  // forward only: a second rotation on the same qubit, u <- u2 u
-            Real u2[8], d2[8], w[8];
-            param_matrices<Real>(G.pkind2, cs[2 * G.pidx2], cs[2 * G.pidx2 + 1], false, u2, d2);
+            Real u2[8], w[8];
+            param_matrices<Real>(G.pkind2, cs[2 * G.pidx2], cs[2 * G.pidx2 + 1], false, u2);
 #pragma unroll
             for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -68,12 +66,8 @@ __device__ __forceinline__ void stage_gate(const RegGate &G, SGate<Real> &S, con
         pkind = 0;
     } else {
         const Real *u = TileT<Real>::U(G);
-        const Real *d = TileT<Real>::D(G);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            S.u[i] = u[i];
-            S.d[i] = d[i];
-        }
+        for (int i = 0; i < 8; ++i) S.u[i] = u[i];
     }
     S.meta = code | ((uint32_t)G.cqm << 8) | ((uint32_t)G.cqv << 12) | ((uint32_t)(G.side & 1) << 16) |
              ((uint32_t)(pkind & 7) << 17) | ((uint32_t)(G.slot + 1) << 20);
@@ -99,59 +93,42 @@ __device__ __forceinline__ void stage_pass(const TilePass &P, const TileGroup *g
 template <typename Real> struct GateRegs {
     uint32_t crm, crv;
     int cqm, cqv, side, slot, code;
-    Real u[8], d[8];
+    Real u[8];
 };
 
 // Parameterised matrices from (c, s) = (cos(theta/2), sin(theta/2)):
-//  RY = [[c, -s], [s, c]]             RY^dagger = [[c, s], [-s, c]]   dRY = 1/2 [[-s, -c], [c, -s]]
+//  RY = [[c, -s], [s, c]]             RY^dagger = [[c, s], [-s, c]]
 //  RZ = diag(c - i s, c + i s)        RZ^dagger = diag(c + i s, c - i s)
-//  dRZ = diag((-s - i c) / 2, (-s + i c) / 2)
 template <typename Real>
-__device__ __forceinline__ void param_matrices(int kind, Real c, Real s, bool adjoint, Real *u, Real *d) {
+__device__ __forceinline__ void param_matrices(int kind, Real c, Real s, bool adjoint, Real *u) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        u[i] = 0;
-        d[i] = 0;
-    }
-    const Real h = (Real)0.5;
+    for (int i = 0; i < 8; ++i) u[i] = 0;
     if (kind == QS_GATE_RY) {
         u[0] = c;
         u[6] = c;
         u[2] = adjoint ? s : -s;
         u[4] = adjoint ? -s : s;
-        d[0] = -h * s;
-        d[2] = -h * c;
-        d[4] = h * c;
-        d[6] = -h * s;
     } else {
         u[0] = c;
         u[6] = c;
         u[1] = adjoint ? s : -s;
         u[7] = adjoint ? -s : s;
-        d[0] = -h * s;
-        d[1] = -h * c;
-        d[6] = -h * s;
-        d[7] = h * c;
     }
 }
 
 // Raw copy of a staged gate (one 16-byte control word and the matrices).
 template <typename Real> struct GateRaw {
     uint4 w;  // crm, crv, meta, pidx
-    Real u[8], d[8];
+    Real u[8];
 };
 
-template <typename Real, bool ADJ>
+template <typename Real>
 __device__ __forceinline__ void fetch_gate(const SGate<Real> &G, GateRaw<Real> &r) {
     using V = typename TileT<Real>::V;  // 16 bytes
     constexpr int PER = 16 / sizeof(Real);
     r.w = *reinterpret_cast<const uint4 *>(&G.crm);
 #pragma unroll
     for (int i = 0; i < 8; i += PER) *reinterpret_cast<V *>(&r.u[i]) = *reinterpret_cast<const V *>(&G.u[i]);
-    if (ADJ) {
-#pragma unroll
-        for (int i = 0; i < 8; i += PER) *reinterpret_cast<V *>(&r.d[i]) = *reinterpret_cast<const V *>(&G.d[i]);
-    }
 }
 
 template <typename Real>
@@ -166,14 +143,10 @@ __device__ __forceinline__ void decode_gate(const GateRaw<Real> &g, GateRegs<Rea
     const int pkind = (int)((meta >> 17) & 7u);
     r.slot = (int)(meta >> 20) - 1;
     if (pkind != 0 && cs) {
-        param_matrices<Real>(pkind, cs[2 * g.w.w], cs[2 * g.w.w + 1], adjoint, r.u, r.d);
+        param_matrices<Real>(pkind, cs[2 * g.w.w], cs[2 * g.w.w + 1], adjoint, r.u);
     } else {
 #pragma unroll
         for (int i = 0; i < 8; ++i) r.u[i] = g.u[i];
-        if (adjoint) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) r.d[i] = g.d[i];
-        }
     }
 }
 
@@ -200,6 +173,17 @@ __device__ __forceinline__ void op_pair(T2 &x, T2 &y, const Real *u, int side) {
     }
 }
 
+// Im <lambda| P psi> of one pair (x, y) of psi and (a, b) of lambda before the un-apply, P the Pauli
+// of the rotation: Y for OP_REAL, Z for OP_DIAG; OP_SIDE is a Z rotation taken on one side, whose
+// other half follows from Im <lambda|psi> = 0 (see plan_adjoint_gates).
+template <int OP, typename T2, typename Real>
+__device__ __forceinline__ Real pauli_dot(const T2 &x, const T2 &y, const T2 &a, const T2 &b, int side) {
+    if (OP == OP_REAL) return (b.x * x.x + b.y * x.y) - (a.x * y.x + a.y * y.y);
+    if (OP == OP_DIAG) return (a.x * x.y - a.y * x.x) - (b.x * y.y - b.y * y.x);
+    if (OP == OP_SIDE) return 2 * (side ? b.y * y.x - b.x * y.y : a.x * x.y - a.y * x.x);
+    return 0;
+}
+
 // All pairs (e, e | 2^P) of the thread's RPT rows for one gate with operation OP; CQ: the
 // gate has controls on group qubits (else every pair of a selected row is updated); UNI: every
 // row is selected (no per-row predicate). RPT independent rows per thread share one decoded
@@ -210,7 +194,6 @@ __device__ __forceinline__ void op_pair(T2 &x, T2 &y, const Real *u, int side) {
 template <int P, int OP, bool ADJ, int GB, bool CQ, int RPT, bool UNI, typename T2, typename Real>
 __device__ __forceinline__ void row_pairs(T2 (&v)[RPT][1 << GB], T2 (&w)[RPT][ADJ ? (1 << GB) : 1],
                                           const GateRegs<Real> &R, const bool (&ok)[RPT], Real &dot) {
-    constexpr int DOP = OP == OP_DIAG ? OP_DIAG : (OP == OP_REAL ? OP_REAL : OP_GEN);
 #pragma unroll
     for (int e = 0; e < (1 << GB); ++e) {
         if ((e >> P) & 1) continue;
@@ -219,15 +202,9 @@ __device__ __forceinline__ void row_pairs(T2 (&v)[RPT][1 << GB], T2 (&w)[RPT][AD
 #pragma unroll
             for (int j = 0; j < RPT; ++j) {
                 if (!UNI && !ok[j]) continue;
+                if (ADJ && R.slot >= 0) dot += pauli_dot<OP, T2, Real>(v[j][e], v[j][e2], w[j][e], w[j][e2], R.side);
                 op_pair<OP, T2, Real>(v[j][e], v[j][e2], R.u, R.side);
-                if (ADJ) {
-                    if (R.slot >= 0) {
-                        T2 mx = v[j][e], my = v[j][e2];
-                        pair_update<DOP, T2, Real>(mx, my, R.d);
-                        dot += w[j][e].x * mx.x + w[j][e].y * mx.y + w[j][e2].x * my.x + w[j][e2].y * my.y;
-                    }
-                    op_pair<OP, T2, Real>(w[j][e], w[j][e2], R.u, R.side);
-                }
+                if (ADJ) op_pair<OP, T2, Real>(w[j][e], w[j][e2], R.u, R.side);
             }
         }
     }
@@ -355,7 +332,7 @@ __device__ __forceinline__ void apply_groups(typename TileT<Real>::T2 *tp, typen
             for (int g = 0; g < gc; ++g) {
                 if (Gr.hctrl && (base & gates[gb + g].hmask) != gates[gb + g].hvals) continue;  // uniform
                 GateRaw<Real> cr;
-                fetch_gate<Real, ADJ>(gates[gb + g], cr);
+                fetch_gate<Real>(gates[gb + g], cr);
                 GateRegs<Real> R;
                 decode_gate<Real>(cr, R, cs, ADJ);
                 Real dot = 0;
@@ -365,7 +342,7 @@ __device__ __forceinline__ void apply_groups(typename TileT<Real>::T2 *tp, typen
                 // uniform: without row controls and with every thread on a row, no predicate
                 row_gate<ADJ, GB, RPT, FOLD, T2, Real>(v, w, R, ok, !(all_rows && R.crm == 0), dot);
                 if (ADJ && R.slot >= 0) {
-                    Real d = dot;
+                    Real d = (Real)0.5 * dot;
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
                     if (lane == 0) acc[R.slot * nwarps + warp].add(d);

@@ -314,25 +314,14 @@ qs_status qs_batch_create(int num_states, const int *n_qubits, const qs_gate *ga
             pid = it->second;
         } else {
             std::vector<GatePlan> fwd(gc), adj(gc);
-            std::vector<const double *> dus(gc, nullptr);
             std::vector<int> slots(gc, -1);
-            static const double kMarker[8] = {0};
             for (size_t i = 0; i < gc; ++i) {
                 if (gs[i].reserved != 0) return set_error(QS_EINVAL, "qs_batch_create: reserved field must be 0");
                 if (!plan_pair(n, dtype, gs[i], (int)np, &fwd[i], &adj[i], err, sizeof(err))) {
                     std::snprintf(e2, sizeof(e2), "qs_batch_create: state %d gate %zu: %s", s, i, err);
                     return set_error(QS_EINVAL, e2);
                 }
-                if (adj[i].op == OP_SIDE) {  // both sides in the sweep (the sweep never skips a side)
-                    double Ud[8];
-                    dagger8(gs[i].U, Ud);
-                    plan_gate(n, dtype, gs[i].target, gs[i].ctrl_mask, gs[i].ctrl_vals, Ud, QS_GATE_U, OP_DIAG, &adj[i],
-                              err, sizeof(err));
-                }
-                if (gs[i].kind == QS_GATE_RY || gs[i].kind == QS_GATE_RZ) {
-                    dus[i] = kMarker;
-                    slots[i] = gs[i].param;
-                }
+                if (gs[i].kind == QS_GATE_RY || gs[i].kind == QS_GATE_RZ) slots[i] = gs[i].param;
             }
             // forward program: two consecutive rotations on the same qubit with the same controls
             // (RY then RZ in the ansatz) become one general gate whose matrix the kernel forms
@@ -364,9 +353,9 @@ qs_status qs_batch_create(int num_states, const int *n_qubits, const qs_gate *ga
             std::iota(seq.begin(), seq.end(), 0);
             FusedProgram pf, pa;
             // the batch kernel runs kGroupBits-qubit groups forward, kGroupBitsAdjoint in the sweep
-            plan_fused(n, dtype, k, seqf, fwdm, nullptr, nullptr, &pf, max_pass_gates, false, kGroupBits);
+            plan_fused(n, dtype, k, seqf, fwdm, nullptr, &pf, max_pass_gates, false, kGroupBits);
             std::reverse(seq.begin(), seq.end());
-            plan_fused(n, dtype, k, seq, adj, &dus, &slots, &pa, max_pass_gates, false, kGroupBitsAdjoint);
+            plan_fused(n, dtype, k, seq, adj, &slots, &pa, max_pass_gates, false, kGroupBitsAdjoint);
             BatchProg bp{};
             bp.small = small;
             bp.n = n;

@@ -57,18 +57,6 @@ static void rot_matrix(int kind, double theta, double U[8]) {
     }
 }
 
-// d/dtheta of the matrices above: dRY = 1/2 [[-s, -c], [c, -s]],
-// dRZ = diag(-i/2 (c - i s), i/2 (c + i s)) = diag((-s - i c)/2, (-s + i c)/2).
-static void rot_derivative(int kind, double theta, double D[8]) {
-    const double c = std::cos(0.5 * theta), s = std::sin(0.5 * theta);
-    std::memset(D, 0, 8 * sizeof(double));
-    if (kind == QS_GATE_RY) {
-        D[0] = -0.5 * s; D[2] = -0.5 * c; D[4] = 0.5 * c; D[6] = -0.5 * s;
-    } else {
-        D[0] = -0.5 * s; D[1] = -0.5 * c; D[6] = -0.5 * s; D[7] = 0.5 * c;
-    }
-}
-
 static void dagger(const double U[8], double D[8]) {
     // [a b; c d]^dagger = [a* c*; b* d*]
     D[0] = U[0]; D[1] = -U[1];
@@ -291,6 +279,41 @@ static void fold_phases(const qs_state *s, std::vector<GatePlan> &plans, int fla
     if (plan_gate(s->n, s->dtype, p.t, 0, 0, U, QS_GATE_U, -1, &q, e2, sizeof(e2))) plans[first] = q;
 }
 
+// The sweep's version of fold_phases (see plan_adjoint_gates): any precision and schedule.
+static void fold_sweep_phases(const qs_state *s, std::vector<GatePlan> &adj) {
+    auto unit = [](double re, double im) { return std::fabs(re * re + im * im - 1.0) <= 1e-12; };
+    int first = -1;  // the first un-applied gate keeps both sides
+    double gr = 1.0, gi = 0.0;
+    char e2[200];
+    for (size_t i = adj.size(); i-- > 0;) {
+        const GatePlan &p = adj[i];
+        if (p.units == 0 || p.op != OP_DIAG || p.ctrl_mask != 0) continue;
+        const double ar = p.Ufull[0], ai = p.Ufull[1], dr = p.Ufull[6], di = p.Ufull[7];
+        if (!unit(ar, ai) || !unit(dr, di)) continue;
+        if (first < 0) {
+            first = (int)i;
+            continue;
+        }
+        const double U[8] = {1.0, 0.0, 0.0, 0.0, 0.0, 0.0, dr * ar + di * ai, di * ar - dr * ai};  // d conj(a)
+        GatePlan q;
+        if (!plan_gate(s->n, s->dtype, p.t, 0, 0, U, QS_GATE_U, OP_SIDE, &q, e2, sizeof(e2))) continue;
+        q.side = 1;  // forced, so that a rotation keeps its structure at every angle
+        q.U[0] = U[6];
+        q.U[1] = U[7];
+        const double nr = gr * ar - gi * ai, ni = gr * ai + gi * ar;
+        gr = nr;
+        gi = ni;
+        adj[i] = q;
+    }
+    if (first < 0) return;
+    GatePlan &p = adj[first];
+    for (int q = 0; q < 8; q += 6) {
+        const double re = p.U[q], im = p.U[q + 1];
+        p.U[q] = p.Ufull[q] = gr * re - gi * im;
+        p.U[q + 1] = p.Ufull[q + 1] = gr * im + gi * re;
+    }
+}
+
 static qs_status launch_plans(qs_state *s, const std::vector<GatePlan> &plans, cudaStream_t st,
                               bool masked = false) {
     for (size_t i = 0; i < plans.size(); ++i) {
@@ -400,18 +423,23 @@ static qs_status launch_program(qs_state *s, const FusedProgram &prog, const std
 }
 
 // Plans of one gradient: the forward gates (same-target runs merged), the sweep's gates
-// (U^dagger, and dU/dtheta for parameterised ones with their gradient slots) and, with
-// QS_FLAG_FUSE, the fused forward and sweep programs.
+// (U^dagger, with the gradient slots of the parameterised ones) and, with QS_FLAG_FUSE, the fused
+// forward and sweep programs.
 struct AdjPlan {
     std::vector<GatePlan> fwd, adj;
     std::vector<int> slot_of, slot_param;
-    std::vector<double> dus;  // 8 doubles per slot
-    std::vector<const double *> dusp;
     FusedProgram pf, pa;
 };
 
-// The per-gate plans of a gradient: forward (then merged), sweep (U^dagger), the parameter
-// slots and derivative matrices.
+// The per-gate plans of a gradient: forward (then merged), sweep (U^dagger) and the parameter
+// slots.
+//
+// In the sweep an uncontrolled diagonal gate of modulus 1, diag(a, d), is the global phase a times
+// diag(1, d / a). A global phase on psi and lambda alike leaves every <lambda| P psi> as it is, so
+// all such gates but one become one-sided (half the amplitudes, half the work) and the one that
+// stays takes the product of their phases, which psi needs to come back as psi_in. The derivative
+// product of a Z rotation then also needs one side only: Im <lambda|psi> = Im <psi|O|psi> is 0 when
+// the sweep starts and every un-apply keeps it, so Im <lambda|Z psi> = 2 Im over one side.
 static bool plan_adjoint_gates(const qs_state *s, const qs_gate *gates, size_t count, const double *theta,
                                size_t n_theta, int flags, AdjPlan *ap, char *err, size_t errlen) {
     std::vector<GatePlan> &fwd = ap->fwd, &adj = ap->adj;
@@ -419,9 +447,7 @@ static bool plan_adjoint_gates(const qs_state *s, const qs_gate *gates, size_t c
     adj.assign(count, GatePlan{});
     ap->slot_of.assign(count, -1);
     std::vector<int> &slot_of = ap->slot_of, &slot_param = ap->slot_param;
-    std::vector<double> &dus = ap->dus;
     slot_param.clear();
-    dus.clear();
     char e2[200];
     for (size_t i = 0; i < count; ++i) {
         const qs_gate &g = gates[i];
@@ -445,22 +471,12 @@ static bool plan_adjoint_gates(const qs_state *s, const qs_gate *gates, size_t c
             std::snprintf(err, errlen, "%s", e2);
             return false;
         }
-        if (adj[i].op == OP_SIDE) {  // the sweep kernels scale both sides
-            GatePlan q;
-            plan_gate(s->n, s->dtype, g.target, g.ctrl_mask, g.ctrl_vals, Ud, QS_GATE_U, OP_DIAG, &q, e2, sizeof(e2));
-            adj[i] = q;
-        }
         if (g.kind == QS_GATE_RY || g.kind == QS_GATE_RZ) {
             slot_of[i] = (int)slot_param.size();
             slot_param.push_back(g.param);
-            double D[8];
-            rot_derivative(g.kind, theta[g.param], D);
-            dus.insert(dus.end(), D, D + 8);
         }
     }
-    ap->dusp.assign(count, nullptr);
-    for (size_t i = 0; i < count; ++i)
-        if (slot_of[i] >= 0) ap->dusp[i] = &dus[8 * slot_of[i]];
+    fold_sweep_phases(s, adj);
     merge_runs(s, fwd, nullptr, flags);  // the forward pass needs no per-gate state
     fold_phases(s, fwd, flags);
     return true;
@@ -472,13 +488,13 @@ static void plan_adjoint_programs(const qs_state *s, int flags, AdjPlan *ap) {
     std::vector<int> seq(ap->fwd.size());
     for (size_t i = 0; i < ap->fwd.size(); ++i) seq[i] = (int)i;
     const bool jit = (flags & QS_FLAG_JIT) != 0;
-    plan_fused(s->n, s->dtype, tile_bits(s->dtype, false), seq, ap->fwd, nullptr, nullptr, &ap->pf, kPassMaxGates, true,
+    plan_fused(s->n, s->dtype, tile_bits(s->dtype, false), seq, ap->fwd, nullptr, &ap->pf, kPassMaxGates, true,
                0, jit);
     seq.resize(count);
     for (size_t i = 0; i < count; ++i) seq[i] = (int)(count - 1 - i);
     // sweep passes keep psi and lambda rows of kGroupBitsAdjoint group qubits in registers
     // (compiled passes too: with 4, their long straight-line groups spill registers)
-    plan_fused(s->n, s->dtype, tile_bits(s->dtype, true, jit), seq, ap->adj, &ap->dusp, &ap->slot_of, &ap->pa,
+    plan_fused(s->n, s->dtype, tile_bits(s->dtype, true, jit), seq, ap->adj, &ap->slot_of, &ap->pa,
                kPassMaxGates, true, 0, jit);
 }
 
@@ -551,17 +567,13 @@ std::vector<uint64_t> adj_signature(const AdjPlan &ap) {
     return sig;
 }
 
-// The matrices of a program's gates from the current plans (and derivative matrices).
-void refresh_matrices(FusedProgram &prog, const std::vector<GatePlan> &plans, const std::vector<const double *> *dusp) {
+// The matrices of a program's gates from the current plans.
+void refresh_matrices(FusedProgram &prog, const std::vector<GatePlan> &plans) {
     for (size_t gi = 0; gi < prog.gates.size(); ++gi) {
         RegGate &R = prog.gates[gi];
         const int src = prog.gate_src[gi];
         std::memcpy(R.U, plans[src].U, sizeof(R.U));
         for (int q = 0; q < 8; ++q) R.Uf[q] = (float)R.U[q];
-        if (dusp && R.slot >= 0 && (*dusp)[src]) {
-            std::memcpy(R.D, (*dusp)[src], sizeof(R.D));
-            for (int q = 0; q < 8; ++q) R.Df[q] = (float)R.D[q];
-        }
     }
 }
 
@@ -674,8 +686,7 @@ static qs_status adjoint_schedule(const qs_state *shape, const qs_gate *gates, s
             for (const GatePlan &p : *pl) {
                 if (p.units == 0 && pl == &ap.fwd) continue;
                 ++r.single_gates;
-                // a sweep step of a parameterised gate reads both sides even when it is diagonal
-                const double b = p.op == OP_SIDE && pl == &ap.fwd ? 0.5 : 1.0;
+                const double b = p.op == OP_SIDE ? 0.5 : 1.0;
                 r.algorithmic_bytes += vectors * b * 2.0 * std::ldexp(dtype == QS_C64 ? 8.0 : 16.0,
                                                                       n - __builtin_popcountll(p.ctrl_mask));
                 r.model_cost += vectors * (single_launch_cost(p, dtype) + launch_latency_cost(n, dtype));
@@ -724,7 +735,7 @@ qs_status qs_circuit_schedule(int n, qs_dtype dtype, const qs_gate *gates, size_
         std::vector<int> seq(plans.size());
         for (size_t i = 0; i < plans.size(); ++i) seq[i] = (int)i;
         FusedProgram prog;
-        plan_fused(n, dtype, tile_bits(dtype, false), seq, plans, nullptr, nullptr, &prog, kPassMaxGates, true, 0,
+        plan_fused(n, dtype, tile_bits(dtype, false), seq, plans, nullptr, &prog, kPassMaxGates, true, 0,
                    (flags & QS_FLAG_JIT) != 0);
         for (const FusedOp &op : prog.ops) {
             if (op.drun >= 0)
@@ -797,7 +808,7 @@ qs_status qs_circuit_order(int n, qs_dtype dtype, const qs_gate *gates, size_t c
             std::vector<int> seq(plans.size());
             for (size_t i = 0; i < plans.size(); ++i) seq[i] = (int)i;
             FusedProgram prog;
-            plan_fused(n, dtype, tile_bits(dtype, false), seq, plans, nullptr, nullptr, &prog, kPassMaxGates, true, 0,
+            plan_fused(n, dtype, tile_bits(dtype, false), seq, plans, nullptr, &prog, kPassMaxGates, true, 0,
                        (flags & QS_FLAG_JIT) != 0);
             for (int pl : prog.order)
                 for (int r = first_rec[pl]; r < first_rec[pl + 1]; ++r) put(r);
@@ -836,7 +847,7 @@ qs_status qs_circuit_compile(int n, qs_dtype dtype, const qs_gate *gates, size_t
         fold_phases(&shape, plans, fl);
         std::vector<int> seq(plans.size());
         for (size_t i = 0; i < plans.size(); ++i) seq[i] = (int)i;
-        plan_fused(n, dtype, tile_bits(dtype, false), seq, plans, nullptr, nullptr, &prog, kPassMaxGates, true, 0,
+        plan_fused(n, dtype, tile_bits(dtype, false), seq, plans, nullptr, &prog, kPassMaxGates, true, 0,
                    (fl & QS_FLAG_JIT) != 0);
         progs.push_back(&prog);
         adj_of.push_back(false);
@@ -918,11 +929,11 @@ qs_status qs_apply_circuit(qs_state *s, const qs_gate *gates, size_t count, cons
         std::vector<uint64_t> sig;
         plans_signature(plans, &sig);
         if (plan_cache_take(pkey, sig, &prog, nullptr, &jit, nullptr)) {
-            refresh_matrices(prog, plans, nullptr);
+            refresh_matrices(prog, plans);
         } else {
             std::vector<int> seq(plans.size());  // after merging: fewer plans than records
             for (size_t i = 0; i < plans.size(); ++i) seq[i] = (int)i;
-            plan_fused(s->n, s->dtype, tile_bits(s->dtype, false), seq, plans, nullptr, nullptr, &prog, kPassMaxGates,
+            plan_fused(s->n, s->dtype, tile_bits(s->dtype, false), seq, plans, nullptr, &prog, kPassMaxGates,
                        true, 0, (flags & QS_FLAG_JIT) != 0);
             if (flags & QS_FLAG_JIT) {
                 std::string jerr;
@@ -1033,7 +1044,6 @@ qs_status qs_adjoint_grad(qs_state *s, const qs_gate *gates, size_t count, const
     }
     std::vector<GatePlan> &fwd = ap.fwd, &adj = ap.adj;
     std::vector<int> &slot_of = ap.slot_of, &slot_param = ap.slot_param;
-    std::vector<const double *> &dusp = ap.dusp;
     FusedProgram &pf = ap.pf, &pa = ap.pa;
     const int nslots = (int)slot_param.size();
     const bool fuse = (flags & QS_FLAG_FUSE) != 0;
@@ -1043,8 +1053,8 @@ qs_status qs_adjoint_grad(qs_state *s, const qs_gate *gates, size_t count, const
         std::vector<unsigned char> key = plan_cache_key('A', s, gates, count, n_theta, flags);
         std::vector<uint64_t> sig = adj_signature(ap);
         if (plan_cache_take(key, sig, &pf, &pa, &jf, &ja)) {
-            refresh_matrices(pf, fwd, nullptr);
-            refresh_matrices(pa, adj, &dusp);
+            refresh_matrices(pf, fwd);
+            refresh_matrices(pa, adj);
         } else {
             plan_adjoint_programs(s, flags, &ap);
             if (use_jit) {

@@ -278,8 +278,7 @@ static int count_groups(const std::vector<LocalGate> &lg, int r) {
 // The pass's gates in an order of fewer register groups where the gate order allows it (the
 // commutation rule of block_schedule on the local positions: non-local controls are controls
 // of every gate that has them, so they never order two gates).
-static void order_for_groups(std::vector<LocalGate> &lg, std::vector<int> &slots, std::vector<const double *> &ds,
-                             std::vector<int> &src, int k, int r) {
+static void order_for_groups(std::vector<LocalGate> &lg, std::vector<int> &slots, std::vector<int> &src, int k, int r) {
     if (lg.size() < 3) return;
     uint32_t targets = 0;
     for (const LocalGate &g : lg) targets |= 1u << g.t;
@@ -296,23 +295,19 @@ static void order_for_groups(std::vector<LocalGate> &lg, std::vector<int> &slots
     for (size_t i = 0; i < ord.size(); ++i) lg2[i] = lg[ord[i]];
     if (count_groups(lg2, r) >= in_order) return;
     std::vector<int> slots2(lg.size()), src2(lg.size());
-    std::vector<const double *> ds2(lg.size());
     for (size_t i = 0; i < ord.size(); ++i) {
         slots2[i] = slots[ord[i]];
         src2[i] = src[ord[i]];
-        ds2[i] = ds[ord[i]];
     }
     lg.swap(lg2);
     slots.swap(slots2);
     src.swap(src2);
-    ds.swap(ds2);
 }
 
-static void add_groups(std::vector<LocalGate> lg, std::vector<int> slots, std::vector<const double *> ds,
-                       std::vector<int> src, int k, int dtype, int group_bits, FusedProgram *prog, TilePass *P) {
+static void add_groups(std::vector<LocalGate> lg, std::vector<int> slots, std::vector<int> src, int k, int dtype, int group_bits, FusedProgram *prog, TilePass *P) {
     const int r = std::min(group_bits, k);
     const int sw = dtype == QS_C64 ? 4 : 3;
-    order_for_groups(lg, slots, ds, src, k, r);
+    order_for_groups(lg, slots, src, k, r);
     prog->order.insert(prog->order.end(), src.begin(), src.end());  // the executed order
     P->group_begin = (int)prog->groups.size();
     P->gate_begin = (int)prog->gates.size();
@@ -374,10 +369,6 @@ static void add_groups(std::vector<LocalGate> lg, std::vector<int> slots, std::v
             R.slot = slots[g];
             std::memcpy(R.U, L.U, sizeof(R.U));
             for (int q = 0; q < 8; ++q) R.Uf[q] = (float)R.U[q];
-            if (ds[g]) {
-                std::memcpy(R.D, ds[g], sizeof(R.D));
-                for (int q = 0; q < 8; ++q) R.Df[q] = (float)R.D[q];
-            }
             rg.push_back(R);
             rsrc.push_back(src[g]);
         }
@@ -504,8 +495,7 @@ struct Segments {
 // The planner proper, gates in the order seq gives: cuts the sequence (into `sg`, unless it is
 // already cut) and, with `prog`, emits the program.
 static void plan_in_order(int n, int dtype, int k, const std::vector<int> &seq, const std::vector<GatePlan> &plans,
-                          const std::vector<const double *> *dus, const std::vector<int> *gslots, FusedProgram *prog,
-                          int max_gates, bool allow_single, int group_bits, bool jit, Segments *sg) {
+                          const std::vector<int> *gslots, FusedProgram *prog, int max_gates, bool allow_single, int group_bits, bool jit, Segments *sg) {
     if (prog) {
         prog->order.clear();
         prog->ops.clear();
@@ -523,9 +513,9 @@ static void plan_in_order(int n, int dtype, int k, const std::vector<int> &seq, 
     k = std::min(std::min(std::max(k, b0 + 1), kTileMaxBits), n);
     const int b = std::min(k, b0);
     const uint64_t low = (b >= 64) ? ~0ull : ((1ull << b) - 1ull);
-    const bool adjoint = dus != nullptr;
+    const bool adjoint = gslots != nullptr;
     const bool diag_runs = !adjoint && allow_single && n >= kDiagChunkBits;
-    auto is_param = [&](int g) { return adjoint && (*dus)[g] != nullptr; };
+    auto is_param = [&](int g) { return adjoint && (*gslots)[g] >= 0; };
     const size_t N = seq.size();
     // per position: target bit (0: changes nothing), controls, parameter, per-gate pass cost
     std::vector<uint64_t> tbit_of(N), ctrl_of(N);
@@ -577,25 +567,20 @@ static void plan_in_order(int n, int dtype, int k, const std::vector<int> &seq, 
         make_pass(n, L, &P);
         std::vector<LocalGate> lg;
         std::vector<int> slots, src;
-        std::vector<const double *> ds;
         for (size_t j = a; j < b; ++j) {
             const int mbr = seq[j];
             if (plans[mbr].units == 0 && !is_param(mbr)) continue;
             LocalGate g = make_local_gate(plans[mbr], L, local_of);
-            const double *d = nullptr;
             int slot = -1;
             if (is_param(mbr)) {
-                if (g.op != OP_GEN && g.op != OP_DIAG && g.op != OP_REAL) g.op = OP_GEN;
-                d = (*dus)[mbr];
                 slot = P.nparam;
                 P.param_gslot[P.nparam++] = (*gslots)[mbr];
             }
             lg.push_back(g);
             slots.push_back(slot);
-            ds.push_back(d);
             src.push_back(mbr);
         }
-        add_groups(lg, slots, ds, src, P.k, dtype, group_bits > 0 ? group_bits : (adjoint ? kGroupBitsAdjoint : kGroupBits),
+        add_groups(lg, slots, src, P.k, dtype, group_bits > 0 ? group_bits : (adjoint ? kGroupBitsAdjoint : kGroupBits),
                    prog, &P);
         prog->ops.push_back({(int)prog->passes.size(), -1});
         prog->passes.push_back(P);
@@ -765,18 +750,17 @@ static void plan_in_order(int n, int dtype, int k, const std::vector<int> &seq, 
 }
 
 bool plan_fused(int n, int dtype, int k, const std::vector<int> &seq, const std::vector<GatePlan> &plans,
-                const std::vector<const double *> *dus, const std::vector<int> *gslots, FusedProgram *prog,
-                int max_gates, bool allow_single, int group_bits, bool jit) {
+                const std::vector<int> *gslots, FusedProgram *prog, int max_gates, bool allow_single, int group_bits, bool jit) {
     // The gates in the given order and in the order block_schedule gives for passes of k local
     // qubits (the same limits as plan_in_order's passes): both are cut, and the program of the
     // one of lower modelled cost is emitted.
     Segments s1;
     const int N = (int)seq.size();
     if (N < 3) {
-        plan_in_order(n, dtype, k, seq, plans, dus, gslots, prog, max_gates, allow_single, group_bits, jit, &s1);
+        plan_in_order(n, dtype, k, seq, plans, gslots, prog, max_gates, allow_single, group_bits, jit, &s1);
         return true;
     }
-    plan_in_order(n, dtype, k, seq, plans, dus, gslots, nullptr, max_gates, allow_single, group_bits, jit, &s1);
+    plan_in_order(n, dtype, k, seq, plans, gslots, nullptr, max_gates, allow_single, group_bits, jit, &s1);
     const int b0 = dtype == QS_C64 ? 4 : 3;
     const int kk = std::min(std::min(std::max(k, b0 + 1), kTileMaxBits), n);
     const int b = std::min(kk, b0);
@@ -786,7 +770,7 @@ bool plan_fused(int n, int dtype, int k, const std::vector<int> &seq, const std:
     for (int i = 0; i < N; ++i) {
         const int g = seq[i];
         const GatePlan &p = plans[g];
-        const bool param = dus != nullptr && (*dus)[g] != nullptr;
+        const bool param = gslots != nullptr && (*gslots)[g] >= 0;
         if (p.units == 0 && !param) {
             items[i] = {-1, 0ull, 0ull, false};
             continue;
@@ -794,20 +778,20 @@ bool plan_fused(int n, int dtype, int k, const std::vector<int> &seq, const std:
         const bool diag = p.op == OP_DIAG || p.op == OP_SIDE;
         items[i] = {p.t, (1ull << p.t) | p.ctrl_mask, diag ? 0ull : (1ull << p.t), param};
     }
-    const std::vector<int> ord = block_schedule(items, n, kk, low, mg, dus ? kTileMaxParam : N);
+    const std::vector<int> ord = block_schedule(items, n, kk, low, mg, gslots ? kTileMaxParam : N);
     bool same = true;
     for (int i = 0; i < N && same; ++i) same = ord[i] == i;
     if (!same) {
         std::vector<int> seq2(N);
         for (int i = 0; i < N; ++i) seq2[i] = seq[ord[i]];
         Segments s2;
-        plan_in_order(n, dtype, k, seq2, plans, dus, gslots, nullptr, max_gates, allow_single, group_bits, jit, &s2);
+        plan_in_order(n, dtype, k, seq2, plans, gslots, nullptr, max_gates, allow_single, group_bits, jit, &s2);
         if (s2.cost < s1.cost - 1e-9) {
-            plan_in_order(n, dtype, k, seq2, plans, dus, gslots, prog, max_gates, allow_single, group_bits, jit, &s2);
+            plan_in_order(n, dtype, k, seq2, plans, gslots, prog, max_gates, allow_single, group_bits, jit, &s2);
             return true;
         }
     }
-    plan_in_order(n, dtype, k, seq, plans, dus, gslots, prog, max_gates, allow_single, group_bits, jit, &s1);
+    plan_in_order(n, dtype, k, seq, plans, gslots, prog, max_gates, allow_single, group_bits, jit, &s1);
     return true;
 }
 

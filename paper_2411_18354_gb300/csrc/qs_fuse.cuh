@@ -50,16 +50,15 @@ const RegGate *table_gates(const FusedProgram &p, const void *dev_base);
 const DiagGate *table_dgates(const FusedProgram &p, const void *dev_base);
 
 // Plan the gates plans[seq[0]], plans[seq[1]], ... (the circuit's order; the program may apply
-// gates that commute in another order, see `order`). For the adjoint
-// sweep, `dus[g]` is dU/dtheta of gate g (nullptr when g has no parameter) and `gslots[g]` its
-// gradient slot; pass nullptr for both in forward mode. k = local qubits per tile.
+// gates that commute in another order, see `order`). For the adjoint sweep, `gslots[g]` is the
+// gradient slot of gate g (-1 when it has no parameter); nullptr in forward mode. k = local qubits
+// per tile.
 // max_gates bounds the gates of one pass (fusion depth); with allow_single == false every gate
 // goes into a pass, also when the pass holds only that gate.
 bool plan_fused(int n, int dtype, int k, const std::vector<int> &seq, const std::vector<GatePlan> &plans,
-                const std::vector<const double *> *dus, const std::vector<int> *gslots, FusedProgram *prog,
-                int max_gates = kPassMaxGates, bool allow_single = true, int group_bits = 0, bool jit = false);
+                const std::vector<int> *gslots, FusedProgram *prog, int max_gates = kPassMaxGates, bool allow_single = true, int group_bits = 0, bool jit = false);
 // group_bits: register qubits per group; 0 = kGroupBits for forward programs and
-// kGroupBitsAdjoint when dus != nullptr. The kernel that runs the program must use the same.
+// kGroupBitsAdjoint when gslots != nullptr. The kernel that runs the program must use the same.
 // Forward programs with allow_single (not the batched kernel) may also put consecutive
 // diagonal gates, optionally after one uncontrolled gate, into diagonal-run ops.
 // jit: the passes will run as kernels compiled for their shape (QS_FLAG_JIT), whose per-gate

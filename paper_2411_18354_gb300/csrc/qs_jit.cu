@@ -122,14 +122,12 @@ void preamble(Out &o, bool dbl) {
     o.f("__device__ __forceinline__ void u_diag(T2 &x, T2 &y, const R *m) { u_mul(x, m[0], m[1]); u_mul(y, m[6], m[7]); }\n");
     o.f("__device__ __forceinline__ void u_swap(T2 &x, T2 &y) { T2 t = x; x = y; y = t; }\n");
     // a parameterised gate from (c, s) = (cos, sin) of theta / 2: kind 2 = RY = [[c, -s], [s, c]],
-    // kind 3 = RZ = diag(c - i s, c + i s); adj: the dagger; d: dU/dtheta of the gate itself
-    o.f("__device__ __forceinline__ void pmat(int kind, R c, R s, int adj, R *u, R *d) {\n"
-        "  for (int i = 0; i < 8; ++i) { u[i] = 0; d[i] = 0; }\n"
-        "  const R h = (R)0.5;\n"
+    // kind 3 = RZ = diag(c - i s, c + i s); adj: the dagger
+    o.f("__device__ __forceinline__ void pmat(int kind, R c, R s, int adj, R *u) {\n"
+        "  for (int i = 0; i < 8; ++i) u[i] = 0;\n"
         "  u[0] = c; u[6] = c;\n"
-        "  if (kind == 2) { u[2] = adj ? s : -s; u[4] = adj ? -s : s; d[0] = -h * s; d[2] = -h * c; d[4] = h * c; "
-        "d[6] = -h * s; }\n"
-        "  else { u[1] = adj ? s : -s; u[7] = adj ? -s : s; d[0] = -h * s; d[1] = -h * c; d[6] = -h * s; d[7] = h * c; }\n"
+        "  if (kind == 2) { u[2] = adj ? s : -s; u[4] = adj ? -s : s; }\n"
+        "  else { u[1] = adj ? s : -s; u[7] = adj ? -s : s; }\n"
         "}\n");
     // w = a b for row-major complex 2x2 matrices (interleaved re, im)
     o.f("__device__ __forceinline__ void mat2(const R *a, const R *b, R *w) {\n"
@@ -176,9 +174,9 @@ std::string any_selects(const RegGate *g, int count, const char *bv = "base") {
     return c;
 }
 
-// Expressions of the gates' matrices (m), derivatives (d) and gradient accumulator indices.
+// Expressions of the gates' matrices (m) and gradient accumulator indices.
 struct Refs {
-    std::vector<std::string> m, d;
+    std::vector<std::string> m;
     std::vector<int> acc;
 };
 
@@ -187,13 +185,12 @@ struct Refs {
 // (pauli 'Y' / 'Z') has dU/dtheta = (-i/2) P U, so with psi' = U^dagger psi (the amplitudes
 // after the un-apply) Re <lambda| dU psi'> = Re <lambda| (-i/2) P psi> = Im <lambda| P psi> / 2:
 // it is taken from the pair before the un-apply, 4 products per pair, no derivative matrix
-// (the caller halves the sum). pauli == 0: the derivative matrix is applied to a copy of the
-// un-applied pair and dotted with lambda.
+// (the caller halves the sum). pauli 'S': a Z rotation on one side, whose other side follows from
+// Im <lambda|psi> = 0 (plan_adjoint_gates).
 void emit_gate_pairs(Out &o, const RegGate &G, int gi, int E, bool adjoint, bool param, char pauli, const char *v,
                      const char *w, const Refs &refs) {
     const char *M = refs.m[gi].c_str();
     const int p = G.p;
-    int dop = G.op == OP_DIAG ? OP_DIAG : (G.op == OP_REAL ? OP_REAL : OP_GEN);
     for (int e = 0; e < E; ++e) {
         if ((e >> p) & 1) continue;
         if ((e & G.cqm) != G.cqv) continue;
@@ -214,17 +211,13 @@ void emit_gate_pairs(Out &o, const RegGate &G, int gi, int E, bool adjoint, bool
         else if (adjoint && param && pauli == 'Z')  // Im <l|Z p> = Im(conj(l0) p0) - Im(conj(l1) p1)
             o.f("dot += (%s[%d].x * %s[%d].y - %s[%d].y * %s[%d].x) - (%s[%d].x * %s[%d].y - %s[%d].y * %s[%d].x);\n", w, e, v,
                 e, w, e, v, e, w, e2, v, e2, w, e2, v, e2);
-        op(v);
-        if (adjoint) {
-            if (param && !pauli) {
-                o.f("{ T2 mx = %s[%d], my = %s[%d]; ", v, e, v, e2);
-                o.f("%s(mx, my, %s); ", dop == OP_DIAG ? "u_diag" : (dop == OP_REAL ? "u_real" : "u_gen"),
-                    refs.d[gi].c_str());
-                o.f("dot += %s[%d].x * mx.x + %s[%d].y * mx.y + %s[%d].x * my.x + %s[%d].y * my.y; }\n", w, e, w, e, w,
-                    e2, w, e2);
-            }
-            op(w);
+        else if (adjoint && param && pauli == 'S') {
+            const int es = G.side ? e2 : e;
+            o.f("dot %s= (R)2 * (%s[%d].x * %s[%d].y - %s[%d].y * %s[%d].x);\n", G.side ? "-" : "+", w, es, v, es, w, es, v,
+                es);
         }
+        op(v);
+        if (adjoint) op(w);
     }
 }
 
@@ -301,7 +294,7 @@ void emit_diag_run(Out &o, const RegGate *gs, int gi0, int count, int E, bool ad
 // the planner forces on rotations (RY: real, RZ: diagonal); 0 when neither.
 char pauli_of(const RegGate &R, bool batched) {
     if (batched) return R.pkind == QS_GATE_RY ? 'Y' : R.pkind == QS_GATE_RZ ? 'Z' : 0;
-    return R.op == OP_REAL ? 'Y' : R.op == OP_DIAG ? 'Z' : 0;
+    return R.op == OP_REAL ? 'Y' : R.op == OP_DIAG ? 'Z' : R.op == OP_SIDE ? 'S' : 0;
 }
 
 }  // namespace
@@ -324,9 +317,9 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
     const uint32_t steps = (nvec + T - 1) / T;
     const int G = P.gate_count;
     const RegGate *pg = gates + P.gate_begin;
-    // Matrix (and derivative) of each gate as an expression: parameters of the kernel (single
+    // Matrix of each gate as an expression: parameters of the kernel (single
     // state), or, in a batch, shared-memory rows formed per tile from the tile's state's angles
-    // for the parameterised gates (pm_, pd_; J = index among them).
+    // for the parameterised gates (pm_; J = index among them).
     std::vector<int> pj(G, -1);
     int NPG = 0;
     if (batched)
@@ -335,15 +328,11 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
     const int NP = adjoint ? (batched ? NPG : P.nparam) : 0;  // gradient accumulators
     Refs refs;
     refs.m.resize(G);
-    refs.d.resize(G);
     for (int i = 0; i < G; ++i) {
         char b[48];
         if (pj[i] >= 0) std::snprintf(b, sizeof(b), "(pm_ + %d)", 8 * pj[i]);
         else std::snprintf(b, sizeof(b), "a.m[%d]", i);
         refs.m[i] = b;
-        if (pj[i] >= 0) std::snprintf(b, sizeof(b), "(pd_ + %d)", 8 * pj[i]);
-        else std::snprintf(b, sizeof(b), "a.d[%d]", pg[i].slot);
-        refs.d[i] = b;
         refs.acc.push_back(batched ? pj[i] : pg[i].slot);
     }
     // debug build: every global access checked against the state's size (2^n), writes counted
@@ -360,10 +349,10 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
             "  for (int j = 0; j < span; ++j) if (i + j < d->count_n) atomicAdd(d->counts + i + j, 1u);\n}\n");
     }
     // parameter block: the fixed matrices of the pass's gates (U, or U^dagger in the adjoint
-    // sweep); single state: the derivatives of its parameterised gates and their global
-    // gradient slots; batch: the parameter indices of the parameterised gates
+    // sweep); single-state sweep: the global gradient slots of its parameterised gates; batch:
+    // the parameter indices of the parameterised gates
     o.f("struct alignas(16) A {\n  R m[%d][8];\n", G > 0 ? G : 1);
-    if (adjoint && !batched) o.f("  R d[%d][8];\n  int gs[%d];\n", NP > 0 ? NP : 1, NP > 0 ? NP : 1);
+    if (adjoint && !batched) o.f("  int gs[%d];\n", NP > 0 ? NP : 1);
     if (batched) o.f("  int pix[%d][2];\n", G > 0 ? G : 1);
     o.f("};\n");
     o.f("__device__ __forceinline__ u32 swz(u32 a) { return %s; }\n", swz_expr("a", SW).c_str());
@@ -386,11 +375,8 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
     o.f("  extern __shared__ __align__(16) unsigned char sm_[];\n");
     o.f("  T2 *const sm0 = reinterpret_cast<T2 *>(sm_);\n");
     o.f("  R *const sr_ = reinterpret_cast<R *>(sm0 + %u);\n", (db ? 2 : 1) * BUF);
-    if (batched) {
-        o.f("  R *const pm_ = sr_;\n");
-        if (adjoint) o.f("  R *const pd_ = pm_ + %d;\n", 8 * (NPG > 0 ? NPG : 1));
-    }
-    const int pm_words = batched ? (adjoint ? 2 : 1) * 8 * (NPG > 0 ? NPG : 1) : 0;
+    if (batched) o.f("  R *const pm_ = sr_;\n");
+    const int pm_words = batched ? 8 * (NPG > 0 ? NPG : 1) : 0;
     if (adjoint) {
         o.f("  R *acc_s = sr_ + %d;\n", pm_words);
         o.f("  R *acc_c = acc_s + %d;\n", (NP > 0 ? NP : 1) * (T / 32));
@@ -484,15 +470,14 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
         for (int i = 0; i < G; ++i) {
             if (pj[i] < 0) continue;
             const RegGate &R = pg[i];
-            o.f("      if (tid == %d) { R u1[8], d1[8]; pmat(%d, cq[2 * a.pix[%d][0]], cq[2 * a.pix[%d][0] + 1], %d, u1, d1);",
+            o.f("      if (tid == %d) { R u1[8]; pmat(%d, cq[2 * a.pix[%d][0]], cq[2 * a.pix[%d][0] + 1], %d, u1);",
                 pj[i] % T, R.pkind, i, i, adjoint ? 1 : 0);
             if (!adjoint && R.pkind2 != 0)
-                o.f(" R u2[8], d2[8]; pmat(%d, cq[2 * a.pix[%d][1]], cq[2 * a.pix[%d][1] + 1], 0, u2, d2);"
+                o.f(" R u2[8]; pmat(%d, cq[2 * a.pix[%d][1]], cq[2 * a.pix[%d][1] + 1], 0, u2);"
                     " mat2(u2, u1, pm_ + %d);",
                     R.pkind2, i, i, 8 * pj[i]);
             else
                 o.f(" for (int q_ = 0; q_ < 8; ++q_) pm_[%d + q_] = u1[q_];", 8 * pj[i]);
-            if (adjoint && !pauli_of(R, true)) o.f(" for (int q_ = 0; q_ < 8; ++q_) pd_[%d + q_] = d1[q_];", 8 * pj[i]);
             o.f(" }\n");
         }
         o.f("    }\n");
@@ -989,16 +974,13 @@ bool jit_prepare_programs(int dtype, const std::vector<JitRequest> &reqs, std::s
         if (it.batched)
             for (int g = P.gate_begin; g < P.gate_begin + P.gate_count; ++g) npg += prog.gates[g].pkind != 0;
         const size_t NP = it.adjoint ? (size_t)std::max(1, it.batched ? npg : P.nparam) : 0;
-        const size_t pm = it.batched ? (it.adjoint ? 2 : 1) * 8 * (size_t)std::max(1, npg) : 0;
+        const size_t pm = it.batched ? 8 * (size_t)std::max(1, npg) : 0;
         j.smem = (jit_double_buffer(dtype, it.adjoint, P.k) ? 2 : 1) * (it.adjoint ? 2 : 1) * T * es +
                  (pm + 2 * NP * (kTileThreads / 32)) * rs;
         j.nparam_gates = npg;
         const size_t G = P.gate_count > 0 ? P.gate_count : 1;
         size_t bytes = G * 8 * rs;
-        if (it.adjoint && !it.batched) {
-            bytes += NP * 8 * rs;
-            bytes += NP * sizeof(int);
-        }
+        if (it.adjoint && !it.batched) bytes += NP * sizeof(int);
         if (it.batched) bytes = ((bytes + 3) & ~size_t(3)) + G * 2 * sizeof(int);
         j.arg_bytes = (bytes + 15) & ~size_t(15);
         j.batched = it.batched;
@@ -1090,7 +1072,7 @@ cudaError_t launch_jit_pass(int dtype, const JitPass &jp, const FusedProgram &pr
     if (e != cudaSuccess) return e;
     const TilePass &P = prog.passes[p];
     const bool adjoint = lam != nullptr;
-    // parameter block: matrices (state precision), derivatives, gradient slots
+    // parameter block: matrices (state precision), gradient slots
     std::vector<unsigned char> blk(jp.arg_bytes, 0);
     const int G = P.gate_count;
     const RegGate *g = prog.gates.data() + P.gate_begin;
@@ -1098,16 +1080,7 @@ cudaError_t launch_jit_pass(int dtype, const JitPass &jp, const FusedProgram &pr
     const size_t G1 = G > 0 ? G : 1;
     put_matrices(dtype, prog, P, blk.data());
     if (adjoint) {
-        const size_t NP1 = P.nparam > 0 ? P.nparam : 1;
-        unsigned char *d = &blk[G1 * 8 * rs];
-        for (int i = 0; i < G; ++i) {
-            if (g[i].slot < 0) continue;
-            if (dtype == QS_C64)
-                std::memcpy(d + (size_t)g[i].slot * 8 * rs, g[i].Df, 8 * rs);
-            else
-                std::memcpy(d + (size_t)g[i].slot * 8 * rs, g[i].D, 8 * rs);
-        }
-        int *gs = reinterpret_cast<int *>(d + NP1 * 8 * rs);
+        int *gs = reinterpret_cast<int *>(&blk[G1 * 8 * rs]);
         for (int i = 0; i < P.nparam; ++i) gs[i] = P.param_gslot[i];
     }
     uint64_t cap = (uint64_t)device_sm_count() * occ;

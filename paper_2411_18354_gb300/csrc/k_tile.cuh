@@ -40,7 +40,7 @@ struct RegGate {
     int32_t pkind;            // batch: QS_GATE_RY / QS_GATE_RZ -> matrices from theta[pidx]; 0 = fixed
     int32_t pidx;             // batch: parameter index inside the state
     int32_t pkind2, pidx2;    // batch forward: a second rotation applied after the first (0 = none)
-    int32_t pad1;
+    int32_t rot;              // OP_REAL: 1 = a rotation [a -b; b a], 2 = a reflection [a b; b -a], 0 = neither
     uint64_t hmask, hvals;    // non-local controls: the tile predicate (global bits)
     double U[8];              // forward: U; adjoint: U^dagger
     float Uf[8];              // the same, rounded once to float32 for complex64 states
@@ -88,12 +88,15 @@ cudaError_t launch_tile_pass(int dtype, void *psi, void *lam, const TilePass &p,
 size_t tile_smem_bytes(int dtype, int k, bool adjoint, int groups, int gates);
 constexpr size_t kTileMaxSmem = 227 * 1024;  // opt-in shared memory per block
 
-// Shared-memory position of local index a (XOR swizzle of the low `sw` bits with the folded
-// higher bits; sw = 4 for complex64, 3 for complex128). A bijection on [0, 2^k).
+// Shared-memory position of local index a: an XOR swizzle of the low 3 bits of the 16-byte unit
+// index with its folded higher bits (a unit is one complex128 amplitude, sw = 3, or a pair of
+// complex64 amplitudes, sw = 4: bit 0 stays, so that amplitude pairs move as 16-byte vectors). A
+// bijection on [0, 2^k) and its own inverse, linear over XOR.
 __host__ __device__ __forceinline__ uint32_t tile_swizzle(uint32_t a, int sw) {
+    const int low = sw - 3;  // bits below the unit index
     uint32_t x = a >> sw, f = 0;
-    for (int i = 0; i < kTileMaxBits; i += sw) f ^= x >> i;
-    return a ^ (f & ((1u << sw) - 1u));
+    for (int i = 0; i < kTileMaxBits; i += 3) f ^= x >> i;
+    return a ^ ((f & 7u) << low);
 }
 
 }  // namespace qs

@@ -368,13 +368,9 @@ __device__ __forceinline__ void apply_groups(typename TileT<Real>::T2 *tp, typen
 }
 
 // Global <-> shared copies of one tile (swizzled in shared memory). Loads are asynchronous
-// copies (cp.async, one per amplitude: 8 bytes for complex64, 16 for complex128) that need no
+// copies (cp.async, 16 bytes: one complex128 amplitude or two of complex64) that need no
 // registers, so every thread has all its copies of the tile in flight at once; the caller's
 // block barrier follows the final wait.
-__device__ __forceinline__ void cp_async_8(void *smem, const void *gmem) {
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
-}
 __device__ __forceinline__ void cp_async_16(void *smem, const void *gmem) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
@@ -392,7 +388,6 @@ constexpr int kTileMaxSteps = (1 << kTileMaxBits) / kTileThreads;  // 64
 struct TileAddr {
     uint64_t g_t;   // this thread's part of the global offset
     uint32_t s_t;   // this thread's part of the shared-memory position
-    uint32_t s_1;   // position offset of element bit i = 1 (complex64 pairs)
     uint32_t steps; // blockDim-strided steps that cover the tile (0 for threads past a small tile)
 };
 
@@ -406,7 +401,6 @@ __device__ __forceinline__ TileAddr tile_addr(const TilePass &P, uint64_t *g_j, 
     const uint32_t o_t = threadIdx.x * VEC;
     a.g_t = scatter_local(P, o_t);
     a.s_t = tile_swizzle(o_t, SW);
-    a.s_1 = tile_swizzle(1u, SW);
     a.steps = threadIdx.x < nvec ? (nvec + blockDim.x - 1) / blockDim.x : 0u;
     const uint32_t nsteps = (nvec + blockDim.x - 1) / blockDim.x;
     for (uint32_t j = threadIdx.x; j < nsteps; j += blockDim.x) {
@@ -426,12 +420,7 @@ __device__ __forceinline__ void load_tile(const TileAddr &ta, const uint64_t *g_
         if (!QS_DBG_OK(g0 | g_j[j], TileT<Real>::VEC)) continue;
         const typename TileT<Real>::T2 *g = src + (g0 | g_j[j]);
         const uint32_t s = ta.s_t ^ s_j[j];
-        if (sizeof(Real) == 4) {
-            cp_async_8(dst + s, g);
-            cp_async_8(dst + (s ^ ta.s_1), g + 1);
-        } else {
-            cp_async_16(dst + s, g);
-        }
+        cp_async_16(dst + s, g);  // one complex128 amplitude or a pair of complex64 (tile_swizzle)
     }
     cp_async_wait_all();
 }
@@ -439,19 +428,13 @@ __device__ __forceinline__ void load_tile(const TileAddr &ta, const uint64_t *g_
 template <typename Real>
 __device__ __forceinline__ void store_tile(const TileAddr &ta, const uint64_t *g_j, const uint32_t *s_j, uint64_t base,
                                            const typename TileT<Real>::T2 *src, typename TileT<Real>::T2 *dst) {
-    using V = typename TileT<Real>::V;
-    using T2 = typename TileT<Real>::T2;
+    using V = typename TileT<Real>::V;  // 16 bytes
     constexpr int VEC = TileT<Real>::VEC;
     const uint64_t g0 = base | ta.g_t;
     for (uint32_t j = 0; j < ta.steps; ++j) {
         if (!QS_DBG_OK(g0 | g_j[j], VEC)) continue;
         QS_DBG_WRITE(g0 | g_j[j], VEC);
-        const uint32_t s = ta.s_t ^ s_j[j];
-        V x;
-        T2 *xs = reinterpret_cast<T2 *>(&x);
-        xs[0] = src[s];
-        if (VEC == 2) xs[VEC - 1] = src[s ^ ta.s_1];
-        *reinterpret_cast<V *>(dst + (g0 | g_j[j])) = x;
+        *reinterpret_cast<V *>(dst + (g0 | g_j[j])) = *reinterpret_cast<const V *>(src + (ta.s_t ^ s_j[j]));
     }
 }
 

@@ -510,7 +510,7 @@ static bool plan_adjoint(const qs_state *s, const qs_gate *gates, size_t count, 
 // ---------------------------------------------------------------------------------------------
 // A training loop applies or differentiates the same circuit with new angles again and again.
 // A fused program depends on the angles only through the gates' matrices, as long as every
-// gate keeps its structure (operation class, one-sided side, identity or not): the last
+// gate keeps its structure (operation class, one-sided side, real shape, identity or not): the last
 // kPlanCacheEntries programs (of qs_apply_circuit: one; of qs_adjoint_grad: forward and sweep)
 // are kept process-wide, keyed by everything else they depend on (entry point, size,
 // precision, flags, tile sizes, the gate records), and a call whose per-gate structure equals
@@ -549,20 +549,20 @@ std::vector<unsigned char> plan_cache_key(char entry, const qs_state *s, const q
 }
 
 // The structure of per-gate plans (what a program built from them depends on besides values).
-void plans_signature(const std::vector<GatePlan> &plans, std::vector<uint64_t> *sig) {
+void plans_signature(int dtype, const std::vector<GatePlan> &plans, std::vector<uint64_t> *sig) {
     sig->push_back(plans.size());
     for (const GatePlan &p : plans) {
         sig->push_back((uint64_t)(uint32_t)p.op | ((uint64_t)(uint32_t)p.side << 8) | ((uint64_t)(p.units == 0) << 16) |
-                       ((uint64_t)(uint32_t)p.t << 24));
+                       ((uint64_t)real_shape(dtype, p) << 20) | ((uint64_t)(uint32_t)p.t << 24));
         sig->push_back(p.ctrl_mask);
         sig->push_back(p.ctrl_vals);
     }
 }
 
-std::vector<uint64_t> adj_signature(const AdjPlan &ap) {
+std::vector<uint64_t> adj_signature(int dtype, const AdjPlan &ap) {
     std::vector<uint64_t> sig;
-    plans_signature(ap.fwd, &sig);
-    plans_signature(ap.adj, &sig);
+    plans_signature(dtype, ap.fwd, &sig);
+    plans_signature(dtype, ap.adj, &sig);
     for (int x : ap.slot_of) sig.push_back((uint64_t)(int64_t)x);
     return sig;
 }
@@ -927,7 +927,7 @@ qs_status qs_apply_circuit(qs_state *s, const qs_gate *gates, size_t count, cons
     if (fuse) {
         std::vector<unsigned char> pkey = plan_cache_key('F', s, gates, count, n_theta, flags);
         std::vector<uint64_t> sig;
-        plans_signature(plans, &sig);
+        plans_signature(s->dtype, plans, &sig);
         if (plan_cache_take(pkey, sig, &prog, nullptr, &jit, nullptr)) {
             refresh_matrices(prog, plans);
         } else {
@@ -1051,7 +1051,7 @@ qs_status qs_adjoint_grad(qs_state *s, const qs_gate *gates, size_t count, const
     const bool use_jit = (flags & QS_FLAG_JIT) != 0;
     if (fuse) {
         std::vector<unsigned char> key = plan_cache_key('A', s, gates, count, n_theta, flags);
-        std::vector<uint64_t> sig = adj_signature(ap);
+        std::vector<uint64_t> sig = adj_signature(s->dtype, ap);
         if (plan_cache_take(key, sig, &pf, &pa, &jf, &ja)) {
             refresh_matrices(pf, fwd);
             refresh_matrices(pa, adj);

@@ -51,11 +51,11 @@ struct LocalGate {
     int t;                 // local target position
     uint32_t cm, cv;       // local controls (local index bits) and their values
     uint64_t hmask, hvals; // non-local controls
-    int op, side;
+    int op, side, rot;
     double U[8];
 };
 
-static LocalGate make_local_gate(const GatePlan &p, uint64_t Lmask, const int *local_of) {
+static LocalGate make_local_gate(int dtype, const GatePlan &p, uint64_t Lmask, const int *local_of) {
     LocalGate g;
     std::memset(&g, 0, sizeof(g));
     g.t = local_of[p.t];
@@ -70,6 +70,7 @@ static LocalGate make_local_gate(const GatePlan &p, uint64_t Lmask, const int *l
     g.hvals = p.ctrl_vals & g.hmask;
     g.op = p.op;
     g.side = p.side;
+    g.rot = real_shape(dtype, p);
     std::memcpy(g.U, p.U, sizeof(g.U));
     return g;
 }
@@ -214,17 +215,20 @@ static std::vector<int> block_schedule(const std::vector<OrderItem> &it, int npo
 }
 
 // Choose the group qubits Q (r of them, containing the targets S): the rows of a warp vary
-// the lowest local qubits outside Q, and for shared-memory accesses without bank conflicts
-// the lowest `sw` of those must land on distinct low bits after the swizzle (qubit b lands on
-// b mod sw). Pads S with the lowest positions that keep that property, else with the best
+// the lowest local qubits outside Q, and for shared-memory accesses without bank conflicts the
+// lowest of those must land on distinct low bits after the swizzle: three of them for 16-byte
+// accesses (complex128, or complex64 with qubit 0 in Q, whose pairs move together), four for
+// single complex64 amplitudes (qubit 0 stays in place, qubit b above lands on 1 + (b - 1) mod 3;
+// complex128: on b mod 3). Pads S with the lowest positions that keep that property, else with the best
 // found.
 static uint32_t choose_group(uint32_t S, int k, int r, int sw) {
     auto score = [&](uint32_t Q) {
         int seen = 0, distinct = 0, taken = 0;
-        for (int b = 0; b < k && taken < sw; ++b) {
+        const int want = sw == 4 && !(Q & 1u) ? 4 : 3, low = sw - 3;
+        for (int b = 0; b < k && taken < want; ++b) {
             if ((Q >> b) & 1u) continue;
             ++taken;
-            const int res = b % sw;
+            const int res = b < low ? 3 : (b - low) % 3;
             if (!((seen >> res) & 1)) {
                 seen |= 1 << res;
                 ++distinct;
@@ -366,6 +370,7 @@ static void add_groups(std::vector<LocalGate> lg, std::vector<int> slots, std::v
             R.hvals = L.hvals;
             R.op = L.op;
             R.side = L.side;
+            R.rot = L.rot;
             R.slot = slots[g];
             std::memcpy(R.U, L.U, sizeof(R.U));
             for (int q = 0; q < 8; ++q) R.Uf[q] = (float)R.U[q];
@@ -570,7 +575,7 @@ static void plan_in_order(int n, int dtype, int k, const std::vector<int> &seq, 
         for (size_t j = a; j < b; ++j) {
             const int mbr = seq[j];
             if (plans[mbr].units == 0 && !is_param(mbr)) continue;
-            LocalGate g = make_local_gate(plans[mbr], L, local_of);
+            LocalGate g = make_local_gate(dtype, plans[mbr], L, local_of);
             int slot = -1;
             if (is_param(mbr)) {
                 slot = P.nparam;

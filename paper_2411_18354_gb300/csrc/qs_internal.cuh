@@ -68,6 +68,8 @@ struct GatePlan {
 // force_op >= 0 skips the structure analysis and uses that GateOp with the full U.
 bool plan_gate(int n, int dtype, int target, uint64_t ctrl_mask, uint64_t ctrl_vals,
                const double U[8], int kind, int force_op, GatePlan *out, char *err, size_t errlen);
+// Shape of an OP_REAL matrix: 1 = [a -b; b a], 2 = [a b; b -a], 0 = neither.
+int real_shape(int dtype, const GatePlan &p);
 // Counter -> index segments for inserted positions pos[0..m-1] (ascending, values `ins`).
 void build_map(int n, const int *pos, int m, uint64_t ins, IndexMap *map);
 // Same plan with all 2^(n-1) pairs scheduled and masked (baseline comparator).

@@ -10,6 +10,7 @@
 #include <algorithm>
 #include <atomic>
 #include <chrono>
+#include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstdlib>
@@ -112,11 +113,28 @@ void preamble(Out &o, bool dbl) {
             "  b.y = F(m[4], x.y, F(m[5], x.x, F(m[6], y.y, m[7] * y.x)));\n"
             "  x = a; y = b;\n}\n");
         o.f("__device__ __forceinline__ void u_real(T2 &x, T2 &y, const R *m) {\n"
-            "  const u64 X = pk(x.x, x.y), Y = pk(y.x, y.y);\n"
-            "  const u64 a = fma2(pk(m[0], m[0]), X, mul2(pk(m[2], m[2]), Y));\n"
-            "  const u64 b = fma2(pk(m[4], m[4]), X, mul2(pk(m[6], m[6]), Y));\n"
+            "  const u64 *q = (const u64 *)m; const u64 X = pk(x.x, x.y), Y = pk(y.x, y.y);\n"
+            "  const u64 a = fma2(q[0], X, mul2(q[1], Y));\n"
+            "  const u64 b = fma2(q[2], X, mul2(q[3], Y));\n"
             "  x = upk(a); y = upk(b);\n}\n");
     }
+    // rotations [a -b; b a] and reflections [a b; b -a] with the larger entry divided out (its
+    // product over the pass is applied by a later gate, real_forms): q = b / a or a / b
+    if (dbl) {
+        o.f("__device__ __forceinline__ void u_rot_a(T2 &x, T2 &y, const R *m) { const R q = m[0]; T2 a; a.x = F(-q, y.x, x.x); "
+            "a.y = F(-q, y.y, x.y); y.x = F(q, x.x, y.x); y.y = F(q, x.y, y.y); x = a; }\n");
+        o.f("__device__ __forceinline__ void u_ref_b(T2 &x, T2 &y, const R *m) { const R q = m[0]; T2 a; a.x = F(q, x.x, y.x); "
+            "a.y = F(q, x.y, y.y); y.x = F(-q, y.x, x.x); y.y = F(-q, y.y, x.y); x = a; }\n");
+    } else {  // m = {q, q, -q, -q}
+        o.f("__device__ __forceinline__ void u_rot_a(T2 &x, T2 &y, const R *m) { const u64 *q = (const u64 *)m; "
+            "const u64 X = pk(x.x, x.y), Y = pk(y.x, y.y); x = upk(fma2(q[1], Y, X)); y = upk(fma2(q[0], X, Y)); }\n");
+        o.f("__device__ __forceinline__ void u_ref_b(T2 &x, T2 &y, const R *m) { const u64 *q = (const u64 *)m; "
+            "const u64 X = pk(x.x, x.y), Y = pk(y.x, y.y); x = upk(fma2(q[0], X, Y)); y = upk(fma2(q[1], Y, X)); }\n");
+    }
+    o.f("__device__ __forceinline__ void u_rot_b(T2 &x, T2 &y, const R *m) { const R q = m[0]; T2 a; a.x = F(q, x.x, -y.x); "
+        "a.y = F(q, x.y, -y.y); y.x = F(q, y.x, x.x); y.y = F(q, y.y, x.y); x = a; }\n");
+    o.f("__device__ __forceinline__ void u_ref_a(T2 &x, T2 &y, const R *m) { const R q = m[0]; T2 a; a.x = F(q, y.x, x.x); "
+        "a.y = F(q, y.y, x.y); y.x = F(q, x.x, -y.x); y.y = F(q, x.y, -y.y); x = a; }\n");
     o.f("__device__ __forceinline__ void u_mul(T2 &x, R ar, R ai) {\n"
         "  T2 a; a.x = F(ar, x.x, -ai * x.y); a.y = F(ar, x.y, ai * x.x); x = a;\n}\n");
     o.f("__device__ __forceinline__ void u_diag(T2 &x, T2 &y, const R *m) { u_mul(x, m[0], m[1]); u_mul(y, m[6], m[7]); }\n");
@@ -128,7 +146,8 @@ void preamble(Out &o, bool dbl) {
         "  u[0] = c; u[6] = c;\n"
         "  if (kind == 2) { u[2] = adj ? s : -s; u[4] = adj ? -s : s; }\n"
         "  else { u[1] = adj ? s : -s; u[7] = adj ? -s : s; }\n"
-        "}\n");
+        "}\n"
+        "__device__ __forceinline__ void dup(R *u) { u[1] = u[0]; u[3] = u[2]; u[5] = u[4]; u[7] = u[6]; }\n");
     // w = a b for row-major complex 2x2 matrices (interleaved re, im)
     o.f("__device__ __forceinline__ void mat2(const R *a, const R *b, R *w) {\n"
         "  for (int i = 0; i < 2; ++i) for (int j = 0; j < 2; ++j) {\n"
@@ -136,9 +155,26 @@ void preamble(Out &o, bool dbl) {
         "    w[4 * i + 2 * j] = x[0] * y0[0] - x[1] * y0[1] + x[2] * y1[0] - x[3] * y1[1];\n"
         "    w[4 * i + 2 * j + 1] = x[0] * y0[1] + x[1] * y0[0] + x[2] * y1[1] + x[3] * y1[0];\n"
         "  }\n}\n");
-    o.f("__device__ __forceinline__ void cp8(void *s, const void *g) {\n"
-        "  asm volatile(\"cp.async.ca.shared.global [%%0], [%%1], 8;\\n\" :: \"r\"((u32)__cvta_generic_to_shared(s)), "
-        "\"l\"(g) : \"memory\");\n}\n");
+    // Sums over the warp of M values per lane at once: each step trades half of the values with the
+    // partner lane, so M sums take M - 1 + log2(32 / M) shuffles instead of 5 M; value i ends in the
+    // lanes with lane / (32 / M) == i.
+    o.f("template <int M> __device__ __forceinline__ R warp_sums(R (&q)[M], int lane) {\n"
+        "  int of = 16;\n"
+        "#pragma unroll\n"
+        "  for (int m = M; m > 1; m >>= 1, of >>= 1) {\n"
+        "    const bool up = lane & of;\n"
+        "#pragma unroll\n"
+        "    for (int i = 0; i < M / 2; ++i) if (i < m / 2) {\n"
+        "      const R keep = up ? q[i + m / 2] : q[i], send = up ? q[i] : q[i + m / 2];\n"
+        "      q[i] = keep + __shfl_xor_sync(0xffffffffu, send, of);\n"
+        "    }\n"
+        "  }\n"
+        "  R s = q[0];\n"
+        "#pragma unroll\n"
+        "  for (int o_ = 16 / M; o_ > 0; o_ >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o_);\n"
+        "  return s;\n}\n");
+    o.f("__device__ __forceinline__ void kahan(R *s, R *c, R v) { const R y = v - *c; const R t = *s + y; *c = (t - *s) - y; "
+        "*s = t; }\n");
     o.f("__device__ __forceinline__ void cp16(void *s, const void *g) {\n"
         "  asm volatile(\"cp.async.cg.shared.global [%%0], [%%1], 16;\\n\" :: \"r\"((u32)__cvta_generic_to_shared(s)), "
         "\"l\"(g) : \"memory\");\n}\n");
@@ -151,8 +187,8 @@ void preamble(Out &o, bool dbl) {
 std::string swz_expr(const char *a, int sw) {
     std::string x = std::string("(") + a + " >> " + std::to_string(sw) + ")";
     std::string f = x;
-    for (int i = sw; i < kTileMaxBits; i += sw) f += " ^ (" + x + " >> " + std::to_string(i) + ")";
-    return std::string("(") + a + " ^ ((" + f + ") & " + std::to_string((1u << sw) - 1u) + "u))";
+    for (int i = 3; i < kTileMaxBits; i += 3) f += " ^ (" + x + " >> " + std::to_string(i) + ")";
+    return std::string("(") + a + " ^ (((" + f + ") & 7u) << " + std::to_string(sw - 3) + "))";
 }
 
 // Tile predicate of a set of gates: "" if some gate has no non-local control (every tile
@@ -174,11 +210,61 @@ std::string any_selects(const RegGate *g, int count, const char *bv = "base") {
     return c;
 }
 
-// Expressions of the gates' matrices (m) and gradient accumulator indices.
+// Expressions of the gates' matrices (m), their update forms (real_forms) and gradient
+// accumulator indices (consecutive in the order of the pass's gates).
 struct Refs {
     std::vector<std::string> m;
+    std::vector<int> form;
     std::vector<int> acc;
 };
+
+// How a pass applies its real gates. An uncontrolled rotation or reflection acts on every pair, so
+// its larger entry can be divided out of the whole vector: 2 multiply-adds per output pair instead
+// of a product and a multiply-add each (half the arithmetic; the divided entry is at least 1/sqrt(2)
+// of the row, so nothing grows by more than sqrt(2) per gate). The last such gate of a pass, and
+// every kRealRun-th, is applied in full with the product of the divided entries. Form 0: in full; 1:
+// rotation, 2: reflection, divided. Inner products of psi and lambda taken in between are scaled
+// back by the square of the product when the pass writes its partial sums.
+constexpr int kRealRun = 24;
+std::vector<int> real_forms(const RegGate *g, int count) {
+    std::vector<int> form(count, 0), at;
+    for (int i = 0; i < count; ++i)
+        if (g[i].op == OP_REAL && g[i].rot && g[i].cqm == 0 && g[i].crm == 0 && g[i].hmask == 0) at.push_back(i);
+    for (size_t j = 0; j + 1 < at.size(); ++j)
+        if ((j + 1) % kRealRun != 0) form[at[j]] = g[at[j]].rot;
+    return form;
+}
+
+// The derivative products of one rotation over its selected pairs, added up in `dot`: for float32 as
+// packed multiply-adds (real and imaginary parts in the two lanes).
+void emit_dots(Out &o, const RegGate &G, int E, char pauli, const char *v, const char *w, bool dbl) {
+    const int p = G.p;
+    bool first = true;
+    for (int e = 0; e < E; ++e) {
+        if (((e >> p) & 1) || (e & G.cqm) != G.cqv) continue;
+        const int e2 = e | (1 << p);
+        if (pauli == 'Y' && !dbl) {  // Im <l|Y p> = (l1 . p0) - (l0 . p1), real dot products
+            o.f(first ? "u64 dp = mul2(pk(%s[%d].x, %s[%d].y), pk(%s[%d].x, %s[%d].y));\n"
+                      : "dp = fma2(pk(%s[%d].x, %s[%d].y), pk(%s[%d].x, %s[%d].y), dp);\n",
+                w, e2, w, e2, v, e, v, e);
+            o.f(first ? "u64 dm = mul2(pk(%s[%d].x, %s[%d].y), pk(%s[%d].x, %s[%d].y));\n"
+                      : "dm = fma2(pk(%s[%d].x, %s[%d].y), pk(%s[%d].x, %s[%d].y), dm);\n",
+                w, e, w, e, v, e2, v, e2);
+        } else if (pauli == 'Y') {
+            o.f("dot += (%s[%d].x * %s[%d].x + %s[%d].y * %s[%d].y) - (%s[%d].x * %s[%d].x + %s[%d].y * %s[%d].y);\n", w, e2, v,
+                e, w, e2, v, e, w, e, v, e2, w, e, v, e2);
+        } else if (pauli == 'Z') {  // Im <l|Z p> = Im(conj(l0) p0) - Im(conj(l1) p1)
+            o.f("dot += (%s[%d].x * %s[%d].y - %s[%d].y * %s[%d].x) - (%s[%d].x * %s[%d].y - %s[%d].y * %s[%d].x);\n", w, e, v,
+                e, w, e, v, e, w, e2, v, e2, w, e2, v, e2);
+        } else if (pauli == 'S') {
+            const int es = G.side ? e2 : e;
+            o.f("dot %s= (R)2 * (%s[%d].x * %s[%d].y - %s[%d].y * %s[%d].x);\n", G.side ? "-" : "+", w, es, v, es, w, es, v,
+                es);
+        }
+        first = false;
+    }
+    if (pauli == 'Y' && !dbl) o.f("{ const T2 sp = upk(dp), sm = upk(dm); dot += (sp.x + sp.y) - (sm.x + sm.y); }\n");
+}
 
 // The pair updates of one gate on row registers v (and, adjoint, w with the derivative dot
 // when the gate has a parameter). A rotation U = exp(-i theta P / 2) about the Pauli P = Y or Z
@@ -188,9 +274,24 @@ struct Refs {
 // (the caller halves the sum). pauli 'S': a Z rotation on one side, whose other side follows from
 // Im <lambda|psi> = 0 (plan_adjoint_gates).
 void emit_gate_pairs(Out &o, const RegGate &G, int gi, int E, bool adjoint, bool param, char pauli, const char *v,
-                     const char *w, const Refs &refs) {
+                     const char *w, const Refs &refs, bool dbl) {
     const char *M = refs.m[gi].c_str();
     const int p = G.p;
+    if (refs.form[gi]) {  // divided: which entry was larger is a (uniform) parameter
+        if (adjoint && param) emit_dots(o, G, E, pauli, v, w, dbl);
+        const char *fn = refs.form[gi] == 1 ? "u_rot" : "u_ref";
+        for (int b = 0; b < 2; ++b) {
+            o.f(b ? "} else {\n" : "if (%s[4] == 0) {\n", M);
+            for (int e = 0; e < E; ++e) {
+                if ((e >> p) & 1) continue;
+                o.f("%s_%c(%s[%d], %s[%d], %s);\n", fn, "ab"[b], v, e, v, e | (1 << p), M);
+                if (adjoint) o.f("%s_%c(%s[%d], %s[%d], %s);\n", fn, "ab"[b], w, e, w, e | (1 << p), M);
+            }
+        }
+        o.f("}\n");
+        return;
+    }
+    if (adjoint && param) emit_dots(o, G, E, pauli, v, w, dbl);
     for (int e = 0; e < E; ++e) {
         if ((e >> p) & 1) continue;
         if ((e & G.cqm) != G.cqv) continue;
@@ -205,17 +306,6 @@ void emit_gate_pairs(Out &o, const RegGate &G, int gi, int E, bool adjoint, bool
             default: break;
             }
         };
-        if (adjoint && param && pauli == 'Y')  // Im <l|Y p> = (l1 . p0) - (l0 . p1), real dot products
-            o.f("dot += (%s[%d].x * %s[%d].x + %s[%d].y * %s[%d].y) - (%s[%d].x * %s[%d].x + %s[%d].y * %s[%d].y);\n", w, e2, v,
-                e, w, e2, v, e, w, e, v, e2, w, e, v, e2);
-        else if (adjoint && param && pauli == 'Z')  // Im <l|Z p> = Im(conj(l0) p0) - Im(conj(l1) p1)
-            o.f("dot += (%s[%d].x * %s[%d].y - %s[%d].y * %s[%d].x) - (%s[%d].x * %s[%d].y - %s[%d].y * %s[%d].x);\n", w, e, v,
-                e, w, e, v, e, w, e2, v, e2, w, e2, v, e2);
-        else if (adjoint && param && pauli == 'S') {
-            const int es = G.side ? e2 : e;
-            o.f("dot %s= (R)2 * (%s[%d].x * %s[%d].y - %s[%d].y * %s[%d].x);\n", G.side ? "-" : "+", w, es, v, es, w, es, v,
-                es);
-        }
         op(v);
         if (adjoint) op(w);
     }
@@ -328,12 +418,14 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
     const int NP = adjoint ? (batched ? NPG : P.nparam) : 0;  // gradient accumulators
     Refs refs;
     refs.m.resize(G);
+    refs.form = batched ? std::vector<int>(G, 0) : real_forms(pg, G);
+    int nacc = 0;
     for (int i = 0; i < G; ++i) {
         char b[48];
         if (pj[i] >= 0) std::snprintf(b, sizeof(b), "(pm_ + %d)", 8 * pj[i]);
         else std::snprintf(b, sizeof(b), "a.m[%d]", i);
         refs.m[i] = b;
-        refs.acc.push_back(batched ? pj[i] : pg[i].slot);
+        refs.acc.push_back(adjoint && pg[i].slot >= 0 ? nacc++ : -1);
     }
     // debug build: every global access checked against the state's size (2^n), writes counted
     const bool dbg = kDebugBuild && !batched;
@@ -352,7 +444,7 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
     // sweep); single-state sweep: the global gradient slots of its parameterised gates; batch:
     // the parameter indices of the parameterised gates
     o.f("struct alignas(16) A {\n  R m[%d][8];\n", G > 0 ? G : 1);
-    if (adjoint && !batched) o.f("  int gs[%d];\n", NP > 0 ? NP : 1);
+    if (adjoint && !batched) o.f("  double f[%d];\n  int gs[%d];\n", NP > 0 ? NP : 1, NP > 0 ? NP : 1);
     if (batched) o.f("  int pix[%d][2];\n", G > 0 ? G : 1);
     o.f("};\n");
     o.f("__device__ __forceinline__ u32 swz(u32 a) { return %s; }\n", swz_expr("a", SW).c_str());
@@ -426,7 +518,6 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
     if (P.hctrl) sel = any_selects(pg, G, "b_");
     if (!sel.empty()) o.f("  auto selected = [](u64 b_) -> bool { return %s; };\n", sel.c_str());
     // tile copies (asynchronous loads into swizzled shared-memory positions; stores from registers)
-    const uint32_t s1 = tile_swizzle(1u, SW);
     auto copies = [&](bool load, const char *gname, const char *tname, const char *bname) {
         if (cp_guard) o.f("    if (tid < %uu) {\n", nvec);
         for (uint32_t j = 0; j < steps; ++j) {
@@ -437,16 +528,12 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
                 o.f("    if (dok(dbg, %s | g_t | 0x%llxull, %d)) ", bname, gj, VEC);
                 if (!load) o.f("{ dcount(dbg, %s | g_t | 0x%llxull, %d); ", bname, gj, VEC);
             }
-            if (load && !dbl)
-                o.f("    { const T2 *g = %s + (%s | g_t | 0x%llxull); const u32 s = s_t ^ %uu; "
-                    "cp8(%s + s, g); cp8(%s + (s ^ %uu), g + 1); }\n",
-                    gname, bname, gj, sj, tname, tname, s1);
-            else if (load)
+            if (load)  // 16 bytes: a complex128 amplitude or a pair of complex64 (tile_swizzle)
                 o.f("    cp16(%s + (s_t ^ %uu), %s + (%s | g_t | 0x%llxull));\n", tname, sj, gname, bname, gj);
             else if (!dbl)
-                o.f("    { const u32 s = s_t ^ %uu; const T2 x0 = %s[s], x1 = %s[s ^ %uu]; T4 q; q.x = x0.x; "
-                    "q.y = x0.y; q.z = x1.x; q.w = x1.y; *reinterpret_cast<T4 *>(%s + (%s | g_t | 0x%llxull)) = q; }\n",
-                    sj, tname, tname, s1, gname, bname, gj);
+                o.f("    *reinterpret_cast<T4 *>(%s + (%s | g_t | 0x%llxull)) = *reinterpret_cast<const T4 *>(%s + (s_t ^ "
+                    "%uu));\n",
+                    gname, bname, gj, tname, sj);
             else
                 o.f("    %s[%s | g_t | 0x%llxull] = %s[s_t ^ %uu];\n", gname, bname, gj, tname, sj);
             if (dbg && !load) o.f("    }\n");
@@ -478,6 +565,7 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
                     R.pkind2, i, i, 8 * pj[i]);
             else
                 o.f(" for (int q_ = 0; q_ < 8; ++q_) pm_[%d + q_] = u1[q_];", 8 * pj[i]);
+            if (!dbl && R.op == OP_REAL) o.f(" dup(pm_ + %d);", 8 * pj[i]);
             o.f(" }\n");
         }
         o.f("    }\n");
@@ -546,10 +634,29 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
             o.f("      T2 v[%d];\n", E);
             if (adjoint) o.f("      T2 w[%d];\n", E);
             o.f("      if (act) {\n");
-            for (int e = 0; e < E; ++e) {
-                o.f("        v[%d] = tp[rs ^ %uu];\n", e, og[e]);
-                if (adjoint) o.f("        w[%d] = tl[rs ^ %uu];\n", e, og[e]);
-            }
+            // float32 amplitudes that differ in local qubit 0 are one 16-byte vector
+            auto row_move = [&](bool load, const char *reg, const char *tile, const std::vector<uint32_t> &off) {
+                for (int e = 0; e < E; ++e) {
+                    if (!dbl && !(e & 1) && E > 1 && (off[e] ^ off[e | 1]) == 1u) {
+                        const int e0 = (off[e] & 1u) ? e | 1 : e, e1 = e0 ^ 1;
+                        if (load)
+                            o.f("        { const T4 q = *reinterpret_cast<const T4 *>(%s + (rs ^ %uu)); %s[%d].x = q.x; "
+                                "%s[%d].y = q.y; %s[%d].x = q.z; %s[%d].y = q.w; }\n",
+                                tile, off[e0], reg, e0, reg, e0, reg, e1, reg, e1);
+                        else
+                            o.f("        { T4 q; q.x = %s[%d].x; q.y = %s[%d].y; q.z = %s[%d].x; q.w = %s[%d].y; "
+                                "*reinterpret_cast<T4 *>(%s + (rs ^ %uu)) = q; }\n",
+                                reg, e0, reg, e0, reg, e1, reg, e1, tile, off[e0]);
+                        ++e;
+                    } else if (load) {
+                        o.f("        %s[%d] = %s[rs ^ %uu];\n", reg, e, tile, off[e]);
+                    } else {
+                        o.f("        %s[rs ^ %uu] = %s[%d];\n", tile, off[e], reg, e);
+                    }
+                }
+            };
+            row_move(true, "v", "tp", og);
+            if (adjoint) row_move(true, "w", "tl", og);
             o.f("      } else {\n");
             for (int e = 0; e < E; ++e) {
                 o.f("        v[%d].x = 0; v[%d].y = 0;\n", e, e);
@@ -559,6 +666,25 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
             auto mergeable = [&](int g) {
                 const RegGate &R = pg[gb + g];
                 return (R.op == OP_DIAG || R.op == OP_SIDE) && !(adjoint && R.slot >= 0);
+            };
+            // derivative products wait in registers and are summed over the warp kDotRun at a time
+            constexpr int kDotRun = 8;
+            int npend = 0, pend0 = 0;
+            auto flush_dots = [&]() {
+                if (npend == 0) return;
+                int M = 1;
+                while (M < npend) M *= 2;
+                o.f("      { R q_[%d] = {", M);
+                for (int i = 0; i < M; ++i) {
+                    if (i < npend) o.f("%sdt%d", i ? ", " : "", pend0 + i);
+                    else o.f(", 0");
+                }
+                o.f("};\n        const R s_ = warp_sums<%d>(q_, lane);\n", M);
+                o.f("        if ((lane & %d) == 0%s) { const int j_ = (%d + (lane / %d)) * %d + warp; kahan(acc_s + j_, acc_c + j_, "
+                    "s_); } }\n",
+                    32 / M - 1, M > npend ? (" && lane / " + std::to_string(32 / M) + " < " + std::to_string(npend)).c_str() : "",
+                    pend0, 32 / M, T / 32);
+                npend = 0;
             };
             for (int g = 0; g < Gr.gate_count; ++g) {
                 if (g + 1 < Gr.gate_count && mergeable(g) && mergeable(g + 1)) {
@@ -573,6 +699,11 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
                 const int slot = adjoint && R.slot >= 0 ? refs.acc[gi] : -1;
                 o.f("      // gate %d: op %d, place %d, cq %x/%x, rows %x/%x\n", gi, R.op, R.p, R.cqm, R.cqv, R.crm, R.crv);
                 const bool tile_guard = R.hmask != 0;
+                if (slot >= 0) {
+                    if (npend == 0) pend0 = slot;
+                    o.f("      R dt%d = 0;\n", slot);
+                    ++npend;
+                }
                 if (tile_guard)
                     o.f("      if ((base & 0x%llxull) == 0x%llxull) {\n", (unsigned long long)R.hmask,
                         (unsigned long long)R.hvals);
@@ -588,22 +719,16 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
                 const bool need_rc = guard || R.crm;
                 if (need_rc) o.f("        if (%s) {\n", rc.c_str());
                 const char pauli = slot >= 0 ? pauli_of(R, batched) : 0;
-                emit_gate_pairs(o, R, gi, E, adjoint, slot >= 0, pauli, "v", "w", refs);
+                emit_gate_pairs(o, R, gi, E, adjoint, slot >= 0, pauli, "v", "w", refs, dbl);
                 if (need_rc) o.f("        }\n");
-                if (slot >= 0 && pauli) o.f("        dot *= (R)0.5;\n");
-                if (slot >= 0) {
-                    o.f("        for (int of = 16; of > 0; of >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, of);\n");
-                    o.f("        if (lane == 0) { R *s_ = acc_s + %d * %d + warp, *c_ = acc_c + %d * %d + warp; "
-                        "const R y = dot - *c_; const R t = *s_ + y; *c_ = (t - *s_) - y; *s_ = t; }\n",
-                        slot, T / 32, slot, T / 32);
-                }
+                if (slot >= 0) o.f("        dt%d = (R)0.5 * dot;\n", slot);
                 o.f("      }\n");
+                if (npend == kDotRun) flush_dots();
             }
+            flush_dots();
             o.f("      if (act) {\n");
-            for (int e = 0; e < E; ++e) {
-                o.f("        tp[rs ^ %uu] = v[%d];\n", os[e], e);
-                if (adjoint) o.f("        tl[rs ^ %uu] = w[%d];\n", os[e], e);
-            }
+            row_move(false, "v", "tp", os);
+            if (adjoint) row_move(false, "w", "tl", os);
             o.f("      }\n    }\n");
         }
         o.f("    }\n    __syncthreads();\n");
@@ -633,7 +758,7 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
         o.f("    double s = 0.0;\n");
         o.f("    for (int w_ = 0; w_ < %d; ++w_) s += (double)acc_s[p * %d + w_] - (double)acc_c[p * %d + w_];\n", T / 32,
             T / 32, T / 32);
-        o.f("    part[(u64)a.gs[p] * part_stride + blockIdx.x] = s;\n  }\n");
+        o.f("    part[(u64)a.gs[p] * part_stride + blockIdx.x] = s * a.f[p];\n  }\n");
     }
     o.f("}\n");
     return o.s;
@@ -694,6 +819,7 @@ std::string shape_key(int dtype, bool adjoint, bool batched, const TilePass &P, 
         put(&g.op, sizeof(g.op));
         put(&g.side, sizeof(g.side));
         put(&g.slot, sizeof(g.slot));
+        put(&g.rot, sizeof(g.rot));
         put(&g.hmask, sizeof(g.hmask));
         put(&g.hvals, sizeof(g.hvals));
         if (batched) {  // the kinds of the rotations whose matrices the kernel forms
@@ -980,7 +1106,7 @@ bool jit_prepare_programs(int dtype, const std::vector<JitRequest> &reqs, std::s
         j.nparam_gates = npg;
         const size_t G = P.gate_count > 0 ? P.gate_count : 1;
         size_t bytes = G * 8 * rs;
-        if (it.adjoint && !it.batched) bytes += NP * sizeof(int);
+        if (it.adjoint && !it.batched) bytes = ((bytes + 7) & ~size_t(7)) + NP * (sizeof(double) + sizeof(int));
         if (it.batched) bytes = ((bytes + 3) & ~size_t(3)) + G * 2 * sizeof(int);
         j.arg_bytes = (bytes + 15) & ~size_t(15);
         j.batched = it.batched;
@@ -1040,16 +1166,42 @@ cudaError_t jit_kernel(const JitPass &jp, cudaKernel_t *kern, int *occ) {
     return cudaSuccess;
 }
 
-// The fixed matrices of a pass's gates (state precision), row-major 8 reals each.
-void put_matrices(int dtype, const FusedProgram &prog, const TilePass &P, unsigned char *dst) {
-    const size_t rs = dtype == QS_C64 ? 4 : 8;
+// The matrices of a pass's gates (state precision), 8 reals each: row-major complex; float32 real
+// gates as {a, a, b, b, c, c, d, d} for the packed update; divided gates (real_forms) as
+// {q, q, -q, -q, which, ...}. scale (may be null): per gate, the product divided out before it.
+template <typename Real>
+void put_matrices(const FusedProgram &prog, const TilePass &P, const std::vector<int> &form, unsigned char *dst,
+                  std::vector<double> *scale) {
     const RegGate *g = prog.gates.data() + P.gate_begin;
-    for (int i = 0; i < P.gate_count; ++i) {
-        if (dtype == QS_C64)
-            std::memcpy(dst + (size_t)i * 8 * rs, g[i].Uf, 8 * rs);
-        else
-            std::memcpy(dst + (size_t)i * 8 * rs, g[i].U, 8 * rs);
+    Real *out = reinterpret_cast<Real *>(dst);
+    double pending = 1.0;
+    for (int i = 0; i < P.gate_count; ++i, out += 8) {
+        if (scale) (*scale)[i] = pending;
+        const double *U = g[i].U;
+        if (form[i]) {
+            const double a = U[0], b = U[4];
+            // (a Hadamard's entries are equal: dividing by b leaves two packed multiply-adds)
+            const bool wide = std::fabs(b) > std::fabs(a) || (form[i] == 2 && std::fabs(b) == std::fabs(a));
+            const double d = wide ? b : a, q = d != 0.0 ? (wide ? a : b) / d : 0.0;
+            out[0] = out[1] = (Real)q;
+            out[2] = out[3] = (Real)-q;
+            out[4] = wide ? (Real)1 : (Real)0;
+            out[5] = out[6] = out[7] = 0;
+            pending *= d;
+            continue;
+        }
+        const bool full = g[i].op == OP_REAL && g[i].rot && pending != 1.0 && g[i].cqm == 0 && g[i].crm == 0 && g[i].hmask == 0;
+        for (int k = 0; k < 8; ++k) out[k] = (Real)(full ? U[k] * pending : U[k]);
+        if (full) pending = 1.0;
+        if (sizeof(Real) == 4 && g[i].op == OP_REAL)
+            for (int k = 0; k < 8; k += 2) out[k + 1] = out[k];
     }
+}
+
+void put_matrices(int dtype, const FusedProgram &prog, const TilePass &P, const std::vector<int> &form, unsigned char *dst,
+                  std::vector<double> *scale = nullptr) {
+    if (dtype == QS_C64) put_matrices<float>(prog, P, form, dst, scale);
+    else put_matrices<double>(prog, P, form, dst, scale);
 }
 
 }  // namespace
@@ -1078,10 +1230,18 @@ cudaError_t launch_jit_pass(int dtype, const JitPass &jp, const FusedProgram &pr
     const RegGate *g = prog.gates.data() + P.gate_begin;
     const size_t rs = dtype == QS_C64 ? 4 : 8;
     const size_t G1 = G > 0 ? G : 1;
-    put_matrices(dtype, prog, P, blk.data());
+    std::vector<double> scale(G);
+    put_matrices(dtype, prog, P, real_forms(g, G), blk.data(), &scale);
     if (adjoint) {
-        int *gs = reinterpret_cast<int *>(&blk[G1 * 8 * rs]);
-        for (int i = 0; i < P.nparam; ++i) gs[i] = P.param_gslot[i];
+        const size_t NP1 = P.nparam > 0 ? P.nparam : 1;
+        double *f = reinterpret_cast<double *>(&blk[(G1 * 8 * rs + 7) & ~size_t(7)]);
+        int *gs = reinterpret_cast<int *>(f + NP1);
+        int j = 0;
+        for (int i = 0; i < G; ++i)
+            if (g[i].slot >= 0) {
+                f[j] = scale[i] * scale[i];
+                gs[j++] = P.param_gslot[g[i].slot];
+            }
     }
     uint64_t cap = (uint64_t)device_sm_count() * occ;
     if (adjoint) cap = std::min<uint64_t>(cap, part_stride);
@@ -1107,7 +1267,7 @@ cudaError_t launch_jit_pass_batched(int dtype, const JitPass &jp, const FusedPro
     const int G = P.gate_count;
     const size_t rs = dtype == QS_C64 ? 4 : 8;
     const size_t G1 = G > 0 ? G : 1;
-    put_matrices(dtype, prog, P, blk.data());
+    put_matrices(dtype, prog, P, std::vector<int>(G, 0), blk.data());
     int *pix = reinterpret_cast<int *>(blk.data() + ((G1 * 8 * rs + 3) & ~size_t(3)));
     const RegGate *g = prog.gates.data() + P.gate_begin;
     for (int i = 0; i < G; ++i) {

@@ -184,6 +184,17 @@ bool plan_gate(int n, int dtype, int target, uint64_t ctrl_mask, uint64_t ctrl_v
     return true;
 }
 
+// complex64: up to 1e-12, so that a product of rotations keeps its shape whatever its rounding
+// (float32 states do not see the difference); complex128: exactly.
+int real_shape(int dtype, const GatePlan &p) {
+    if (p.op != OP_REAL) return 0;
+    const double a = p.U[0], b = p.U[2], c = p.U[4], d = p.U[6];
+    const double tol = dtype == QS_C64 ? 1e-12 * std::max(std::fabs(a), std::fabs(c)) : 0.0;
+    if (std::fabs(a - d) <= tol && std::fabs(b + c) <= tol) return 1;
+    if (std::fabs(a + d) <= tol && std::fabs(b - c) <= tol) return 2;
+    return 0;
+}
+
 void plan_masked(const GatePlan &compact, GatePlan *out) {
     *out = compact;
     int pos[1] = {compact.t};

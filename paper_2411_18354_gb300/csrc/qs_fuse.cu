@@ -241,6 +241,9 @@ static uint32_t choose_group(uint32_t S, int k, int r, int sw) {
     std::vector<int> free_pos;
     for (int b = 0; b < k; ++b)
         if (!((S >> b) & 1u)) free_pos.push_back(b);
+    // among equals, leave the qubits inside a 32-byte run to the lanes (except complex64's qubit 0,
+    // whose pairs are vectors), so that rows can also move straight to and from the state
+    const uint32_t run = sw == 4 ? 6u : 3u;
     uint32_t best = 0;
     int best_score = 1 << 30;
     // combinations of `need` free positions, lexicographic (lowest first)
@@ -250,7 +253,7 @@ static uint32_t choose_group(uint32_t S, int k, int r, int sw) {
     while (true) {
         uint32_t Q = S;
         for (int i = 0; i < need; ++i) Q |= 1u << free_pos[idx[i]];
-        const int sc = score(Q);
+        const int sc = 2 * score(Q) + ((Q & run) != 0);
         if (sc < best_score) {
             best_score = sc;
             best = Q;

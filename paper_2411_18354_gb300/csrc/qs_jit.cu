@@ -389,6 +389,44 @@ char pauli_of(const RegGate &R, bool batched) {
 
 }  // namespace
 
+namespace {
+
+// Whether the rows of a group, one per thread, cover runs of at least 32 bytes of the state per
+// access: complex64 without qubits 1 and 2 in registers (qubit 0 may be, its pairs move as vectors),
+// complex128 without 0 and 1.
+bool direct_rows(const TileGroup &Gr, int r, bool dbl) {
+    uint32_t Q = 0;
+    for (int q = 0; q < r; ++q) Q |= 1u << Gr.q[q];
+    return (Q & (dbl ? 3u : 6u)) == 0;
+}
+
+// " | (...)" terms of the global offset of row rho: its bits at the group's other local qubits'
+// positions in the state, by runs that move by the same distance.
+std::string row_address(const TilePass &P, const TileGroup &Gr, int bits) {
+    std::string a;
+    int from = 0, dist = -1;
+    auto put = [&](int to) {
+        if (to == from) return;
+        char b[96];
+        std::snprintf(b, sizeof(b), " | ((u64)(rho & 0x%xu) << %d)", ((1u << to) - 1u) & ~((1u << from) - 1u), dist);
+        a += b;
+    };
+    for (int i = 0; i < bits; ++i) {
+        uint32_t l = 0;
+        for (int s = 0; s < Gr.nrseg; ++s) l |= ((1u << i) << Gr.rshift[s]) & Gr.rmask[s];
+        const int d = __builtin_ctzll(scatter_host(P, l)) - i;
+        if (d != dist) {
+            put(i);
+            from = i;
+            dist = d;
+        }
+    }
+    put(bits);
+    return a;
+}
+
+}  // namespace
+
 // Two tile buffers per block (the next tile's copies in flight while the current one is
 // computed) where both still leave room for two blocks per SM.
 bool jit_double_buffer(int dtype, bool adjoint, int k) {
@@ -598,6 +636,7 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
     }
     o.f("    __syncthreads();\n");
 
+    bool stored = false;
     for (int gi_ = 0; gi_ < P.group_count; ++gi_) {
         const TileGroup &Gr = groups[P.group_begin + gi_];
         const int r = Gr.r;
@@ -620,6 +659,17 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
             og[e] = Gr.has_g ? Gr.gperm[e] : off;
             os[e] = Gr.has_s ? Gr.sperm[e] : off;
         }
+        // The last group writes its rows straight to the state where every tile runs it and its
+        // qubits leave the low ones to the lanes (runs of at least 32 bytes per store): the tile's
+        // last trip through shared memory and a block barrier less.
+        const bool direct = gi_ + 1 == P.group_count && gcond.empty() && direct_rows(Gr, r, dbl);
+        std::vector<unsigned long long> ge(E);
+        for (int e = 0; e < E; ++e) ge[e] = scatter_host(P, tile_swizzle(os[e], SW));
+        if (direct) {
+            o.f("    T2 *gp_ = gvec(psi, tau);\n");
+            if (adjoint) o.f("    T2 *gl_ = gvec(lam, tau);\n");
+        }
+        stored = direct;
         for (uint32_t rb = 0; rb < rblocks; ++rb) {
             o.f("    {\n      const u32 rho = %uu + tid;\n", rb * T);
             const bool guard = rows < (rb + 1) * (uint32_t)T;
@@ -727,19 +777,41 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
             }
             flush_dots();
             o.f("      if (act) {\n");
-            row_move(false, "v", "tp", os);
-            if (adjoint) row_move(false, "w", "tl", os);
+            if (direct) {
+                o.f("        const u64 ga = base%s;\n", row_address(P, Gr, k - r).c_str());
+                for (int vec = 0; vec < (adjoint ? 2 : 1); ++vec) {
+                    const char *reg = vec ? "w" : "v", *gv = vec ? "gl_" : "gp_";
+                    for (int e = 0; e < E; ++e) {
+                        const bool pair = !dbl && !(e & 1) && E > 1 && (ge[e] ^ ge[e | 1]) == 1u;
+                        const int e0 = pair && (ge[e] & 1u) ? e | 1 : e;
+                        if (dbg) o.f("        if (dok(dbg, ga | 0x%llxull, %d)) { dcount(dbg, ga | 0x%llxull, %d);", ge[e0], pair ? 2 : 1, ge[e0], pair ? 2 : 1);
+                        if (pair)
+                            o.f("        { T4 q; q.x = %s[%d].x; q.y = %s[%d].y; q.z = %s[%d].x; q.w = %s[%d].y; "
+                                "*reinterpret_cast<T4 *>(%s + (ga | 0x%llxull)) = q; }\n",
+                                reg, e0, reg, e0, reg, e0 ^ 1, reg, e0 ^ 1, gv, ge[e0]);
+                        else
+                            o.f("        %s[ga | 0x%llxull] = %s[%d];\n", gv, ge[e0], reg, e);
+                        if (dbg) o.f("        }\n");
+                        e += pair;
+                    }
+                }
+            } else {
+                row_move(false, "v", "tp", os);
+                if (adjoint) row_move(false, "w", "tl", os);
+            }
             o.f("      }\n    }\n");
         }
         o.f("    }\n    __syncthreads();\n");
     }
-    o.f("    {\n    T2 *gp_ = gvec(psi, tau);\n");
-    copies(false, "gp_", "tp", "base");
-    if (adjoint) {
-        o.f("    T2 *gl_ = gvec(lam, tau);\n");
-        copies(false, "gl_", "tl", "base");
+    if (!stored) {
+        o.f("    {\n    T2 *gp_ = gvec(psi, tau);\n");
+        copies(false, "gp_", "tp", "base");
+        if (adjoint) {
+            o.f("    T2 *gl_ = gvec(lam, tau);\n");
+            copies(false, "gl_", "tl", "base");
+        }
+        o.f("    }\n    __syncthreads();\n");
     }
-    o.f("    }\n    __syncthreads();\n");
     if (adjoint && batched && NP > 0) {
         // this tile's gradient partials (sum over the block's warps), then fresh accumulators;
         // the loop's next block barrier orders them before the next tile adds to them

@@ -427,11 +427,17 @@ std::string row_address(const TilePass &P, const TileGroup &Gr, int bits) {
 
 }  // namespace
 
-// Two tile buffers per block (the next tile's copies in flight while the current one is
-// computed) where both still leave room for two blocks per SM.
-bool jit_double_buffer(int dtype, bool adjoint, int k) {
+// A block alternates between copies, row moves and arithmetic with block barriers in between, so an
+// SM needs other blocks to fill its pipes, and the next tile's copy must run meanwhile: two tile
+// buffers wherever two blocks still fit, and three blocks where their buffers fit and the rows are
+// complex64 (80 registers a thread: 1000-gate circuit at n = 28 57.8 -> 56.1 ms, QFT29 7.88 -> 7.68,
+// n = 24 gradient 7.99 -> 7.61; complex128 rows alone take 64). One buffer costs 15-20 %; blocks of 128
+// threads, 5-qubit groups and tiles of 2^11 or 2^13 amplitudes were within 3 % or slower, rows of
+// 64 or 32 contiguous bytes (one or two more qubits per pass) 15 and 40 % slower.
+JitShape jit_shape(int dtype, bool adjoint, int k) {
     const size_t tile = (size_t(1) << k) * (dtype == QS_C64 ? 8 : 16) * (adjoint ? 2 : 1);
-    return 2 * tile <= 100 * 1024;
+    if (dtype == QS_C64 && 6 * tile <= 200 * 1024) return {3, true};
+    return {adjoint && dtype == QS_C128 ? 1 : 2, 2 * tile <= 100 * 1024};
 }
 
 std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const TileGroup *groups,
@@ -486,7 +492,7 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
     if (batched) o.f("  int pix[%d][2];\n", G > 0 ? G : 1);
     o.f("};\n");
     o.f("__device__ __forceinline__ u32 swz(u32 a) { return %s; }\n", swz_expr("a", SW).c_str());
-    const int minb = (adjoint && dbl) ? 1 : 2;
+    const int minb = jit_shape(dtype, adjoint, k).blocks;
     if (batched)
         o.f("extern \"C\" __global__ void __launch_bounds__(%d, %d) %s(T2 *__restrict__ psi, T2 *__restrict__ lam, "
             "double *__restrict__ part, u64 stride, u64 nstates, const R *__restrict__ cs, u32 cs_stride, "
@@ -499,7 +505,7 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
     else
         o.f("extern \"C\" __global__ void __launch_bounds__(%d, %d) %s(T2 *__restrict__ psi, const __grid_constant__ A a%s) {\n",
             T, minb, kname, dbg ? ", DebugState *dbg" : "");
-    const bool db = jit_double_buffer(dtype, adjoint, k);
+    const bool db = jit_shape(dtype, adjoint, k).db;
     const uint32_t TILE = 1u << k;
     const uint32_t BUF = (adjoint ? 2 : 1) * TILE;  // one buffer: psi tile (and lambda tile)
     o.f("  extern __shared__ __align__(16) unsigned char sm_[];\n");
@@ -1173,7 +1179,7 @@ bool jit_prepare_programs(int dtype, const std::vector<JitRequest> &reqs, std::s
             for (int g = P.gate_begin; g < P.gate_begin + P.gate_count; ++g) npg += prog.gates[g].pkind != 0;
         const size_t NP = it.adjoint ? (size_t)std::max(1, it.batched ? npg : P.nparam) : 0;
         const size_t pm = it.batched ? 8 * (size_t)std::max(1, npg) : 0;
-        j.smem = (jit_double_buffer(dtype, it.adjoint, P.k) ? 2 : 1) * (it.adjoint ? 2 : 1) * T * es +
+        j.smem = (jit_shape(dtype, it.adjoint, P.k).db ? 2 : 1) * (it.adjoint ? 2 : 1) * T * es +
                  (pm + 2 * NP * (kTileThreads / 32)) * rs;
         j.nparam_gates = npg;
         const size_t G = P.gate_count > 0 ? P.gate_count : 1;

@@ -68,8 +68,13 @@ cudaError_t launch_jit_pass_batched(int dtype, const JitPass &jp, const FusedPro
                                     void *lam, double *part, uint64_t stride, uint64_t nstates, const void *cs,
                                     uint32_t cs_stride, cudaStream_t st);
 
-// Whether the kernel of a pass with 2^k-amplitude tiles double-buffers them.
-bool jit_double_buffer(int dtype, bool adjoint, int k);
+// Blocks per SM that the kernel of a pass with 2^k-amplitude tiles is compiled for, and whether
+// it has two tile buffers (the next tile is copied in while the current one is computed).
+struct JitShape {
+    int blocks;
+    bool db;
+};
+JitShape jit_shape(int dtype, bool adjoint, int k);
 
 // The generated source of one pass (exposed for tests of the generator).
 // batched: the kernel runs the pass over `nstates` states of one batch program at once (tile

@@ -16,12 +16,15 @@
 // terms), the running sum over a block's tiles is a compensated (Kahan) float32 sum, and the
 // sum over blocks is float64. Complex128: float64 everywhere. The result does not depend on
 // scheduling (fixed tile-to-block assignment and fixed summation order).
-// Complex128 is bound by the FP64 pipe (GB300 issues about 2 FP64 operations per SM per clock),
-// so its sums are arranged for fewer operations: a thread's 16 values go through a pairwise
-// tree whose partial sums also give the four j-bit sums (26 adds instead of 48); the warp
-// forms the lane-bit sums on the way while it reduces the total (a butterfly: 15 shuffles and
-// adds instead of 25) and reduces the four j-bit sums by a transposed reduce-scatter that
-// leaves each in its own lanes (6 instead of 20).
+//
+// Complex128 in float64 arithmetic is bound by the FP64 pipe (2 operations per SM and clock; |psi|^2
+// and the sums took ~5 per amplitude, 2.5 clocks against 0.7 of memory time). A thread's 16 values
+// therefore share one power-of-two scale and are squared and added as 64-bit integers
+// (k_expz_c128): 58-bit magnitudes, |x|^2 as xh^2 + yh^2 + (the cross and low products >> 30) in
+// units of 2^-56 of the scale's square, below 2^57 each, so that the 16-value sums are exact. Five
+// sums per 16 values become float64 and are added there. The warp-level sums are formed once per
+// run of 2^m consecutive tiles (the low m tile bits have per-thread sums of their own). n = 28:
+// 2.72 -> 0.80 ms (5.4 TB/s), error against exact arithmetic as before (1-2 units in the last place).
 #include <algorithm>
 
 #include "k_gate.cuh"
@@ -36,11 +39,11 @@ constexpr int kJ = 16;  // unrolled loads per thread per tile
 template <typename Real> struct RedT;
 template <> struct RedT<float> {
     using T2 = float2;
-    static constexpr int VB = 1;  // log2(amplitudes per 16-byte load)
+    static constexpr int TB = 13;  // log2(amplitudes per tile): 256 threads, 16 loads of 16 bytes
 };
 template <> struct RedT<double> {
     using T2 = double2;
-    static constexpr int VB = 0;
+    static constexpr int TB = 12;
 };
 
 template <typename A>
@@ -50,127 +53,68 @@ __device__ __forceinline__ A warp_sum(A v) {
     return v;
 }
 
-template <typename Real>
 __global__ void __launch_bounds__(kRedThreads)
-k_expz_tiles(const typename RedT<Real>::T2 *__restrict__ psi, int n, uint64_t ntiles, double *__restrict__ partials) {
-    using A = Real;  // per-thread / per-warp accumulator type
-    constexpr int VB = RedT<Real>::VB;
-    constexpr int TB = VB + 8 + 4;
-    // per-warp values: [0] total, [1..VB] v-bit, [1+VB .. 4+VB] j bits, [5+VB .. 9+VB] lane bits
-    constexpr int NV = 1 + VB + 4 + 5;
-    __shared__ A wpart[kRedThreads / 32][NV];
+k_expz_c64(const float2 *__restrict__ psi, int n, uint64_t ntiles, double *__restrict__ partials) {
+    constexpr int TB = RedT<float>::TB;
+    // per-warp values: [0] total, [1] element bit, [2..5] j bits, [6..10] lane bits
+    __shared__ float wpart[kRedThreads / 32][11];
     const int tid = threadIdx.x;
     const int lane = tid & 31;
     const int warp = tid >> 5;
-    Acc<Real> acc{};  // output `tid` of this block, over its tiles
+    Acc<float> acc{};  // output `tid` of this block, over its tiles
     for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        A tot = 0, sv = 0, sj[4] = {0, 0, 0, 0};
-        if constexpr (VB == 1) {
-            const float4 *base = reinterpret_cast<const float4 *>(psi) + (tile << (TB - 1));
+        float tot = 0, sv = 0, sj[4] = {0, 0, 0, 0};
+        const float4 *base = reinterpret_cast<const float4 *>(psi) + (tile << (TB - 1));
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                float4 q[kJ / 2];
+        for (int h = 0; h < 2; ++h) {
+            float4 q[kJ / 2];
 #pragma unroll
-                for (int jj = 0; jj < kJ / 2; ++jj) q[jj] = base[(h * (kJ / 2) + jj) * kRedThreads + tid];
+            for (int jj = 0; jj < kJ / 2; ++jj) q[jj] = base[(h * (kJ / 2) + jj) * kRedThreads + tid];
 #pragma unroll
-                for (int jj = 0; jj < kJ / 2; ++jj) {
-                    const int j = h * (kJ / 2) + jj;
-                    const A p0 = (A)fmaf(q[jj].x, q[jj].x, q[jj].y * q[jj].y);
-                    const A p1 = (A)fmaf(q[jj].z, q[jj].z, q[jj].w * q[jj].w);
-                    const A s = p0 + p1;
-                    tot += s;
-                    sv += p1;
+            for (int jj = 0; jj < kJ / 2; ++jj) {
+                const int j = h * (kJ / 2) + jj;
+                const float p0 = fmaf(q[jj].x, q[jj].x, q[jj].y * q[jj].y);
+                const float p1 = fmaf(q[jj].z, q[jj].z, q[jj].w * q[jj].w);
+                const float s = p0 + p1;
+                tot += s;
+                sv += p1;
 #pragma unroll
-                    for (int b = 0; b < 4; ++b)
-                        if ((j >> b) & 1) sj[b] += s;
-                }
+                for (int b = 0; b < 4; ++b)
+                    if ((j >> b) & 1) sj[b] += s;
             }
-        } else {
-            // complex128: |psi|^2 of the thread's 16 values, a pairwise tree, per-warp sums
-            const double2 *base = reinterpret_cast<const double2 *>(psi) + (tile << TB);
-            double p[kJ];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                double2 q[kJ / 2];
-#pragma unroll
-                for (int jj = 0; jj < kJ / 2; ++jj) q[jj] = base[(h * (kJ / 2) + jj) * kRedThreads + tid];
-#pragma unroll
-                for (int jj = 0; jj < kJ / 2; ++jj) p[h * (kJ / 2) + jj] = fma(q[jj].x, q[jj].x, q[jj].y * q[jj].y);
-            }
-            double a[8], b4[4], c2[2];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) a[i] = p[2 * i] + p[2 * i + 1];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) b4[i] = a[2 * i] + a[2 * i + 1];
-            c2[0] = b4[0] + b4[1];
-            c2[1] = b4[2] + b4[3];
-            double t = c2[0] + c2[1];
-            double sjt[4];  // sum over the thread's j with bit b set
-            sjt[3] = c2[1];
-            sjt[2] = b4[1] + b4[3];
-            sjt[1] = (a[1] + a[3]) + (a[5] + a[7]);
-            sjt[0] = ((p[1] + p[3]) + (p[5] + p[7])) + ((p[9] + p[11]) + (p[13] + p[15]));
-            // butterfly over the lane bits: before step b, t sums the 2^b lanes that differ from
-            // this one below bit b; the half with bit b set is this lane's t or its partner's
-            double lb[5];
-#pragma unroll
-            for (int b = 0; b < 5; ++b) {
-                const double pt = __shfl_xor_sync(0xffffffffu, t, 1 << b);
-#pragma unroll
-                for (int c = 0; c < b; ++c) lb[c] += __shfl_xor_sync(0xffffffffu, lb[c], 1 << b);
-                lb[b] = ((lane >> b) & 1) ? t : pt;
-                t += pt;
-            }
-            // j-bit sums: lanes with lane bit 4 = 0 keep sums 0, 1 and lanes with bit 4 = 1 keep
-            // 2, 3; then bit 3 splits those; bits 2..0 finish each sum. Sum q ends in the lanes
-            // with (lane >> 3) == q.
-            const bool h4 = (lane >> 4) & 1, h3 = (lane >> 3) & 1;
-            const double k0 = (h4 ? sjt[2] : sjt[0]) + __shfl_xor_sync(0xffffffffu, h4 ? sjt[0] : sjt[2], 16);
-            const double k1 = (h4 ? sjt[3] : sjt[1]) + __shfl_xor_sync(0xffffffffu, h4 ? sjt[1] : sjt[3], 16);
-            double vj = (h3 ? k1 : k0) + __shfl_xor_sync(0xffffffffu, h3 ? k0 : k1, 8);
-#pragma unroll
-            for (int o = 4; o > 0; o >>= 1) vj += __shfl_xor_sync(0xffffffffu, vj, o);
-            if (lane == 0) {
-                wpart[warp][0] = (A)t;
-#pragma unroll
-                for (int b = 0; b < 5; ++b) wpart[warp][5 + b] = (A)lb[b];
-            }
-            if ((lane & 7) == 0) wpart[warp][1 + (lane >> 3)] = (A)vj;
         }
-        if constexpr (VB == 1) {
-            // lane-bit sums before the total is reduced
-            A sl[5];
+        // lane-bit sums before the total is reduced
+        float sl[5];
 #pragma unroll
-            for (int b = 0; b < 5; ++b) sl[b] = warp_sum<A>(((lane >> b) & 1) ? tot : (A)0);
-            tot = warp_sum<A>(tot);
-            sv = warp_sum<A>(sv);
+        for (int b = 0; b < 5; ++b) sl[b] = warp_sum<float>(((lane >> b) & 1) ? tot : 0.f);
+        tot = warp_sum<float>(tot);
+        sv = warp_sum<float>(sv);
 #pragma unroll
-            for (int b = 0; b < 4; ++b) sj[b] = warp_sum<A>(sj[b]);
-            if (lane == 0) {
-                wpart[warp][0] = tot;
-                wpart[warp][1] = sv;
+        for (int b = 0; b < 4; ++b) sj[b] = warp_sum<float>(sj[b]);
+        if (lane == 0) {
+            wpart[warp][0] = tot;
+            wpart[warp][1] = sv;
 #pragma unroll
-                for (int b = 0; b < 4; ++b) wpart[warp][1 + VB + b] = sj[b];
+            for (int b = 0; b < 4; ++b) wpart[warp][2 + b] = sj[b];
 #pragma unroll
-                for (int b = 0; b < 5; ++b) wpart[warp][5 + VB + b] = sl[b];
-            }
+            for (int b = 0; b < 5; ++b) wpart[warp][6 + b] = sl[b];
         }
         __syncthreads();
         if (tid <= n) {
             // output tid: tid == n -> total; else S_tid (sum over amplitudes with bit tid set)
-            A v = 0;
+            float v = 0;
             const int b = tid;
             if (b == n) {
                 for (int w = 0; w < kRedThreads / 32; ++w) v += wpart[w][0];
-            } else if (b < VB) {
+            } else if (b < 1) {
                 for (int w = 0; w < kRedThreads / 32; ++w) v += wpart[w][1];
-            } else if (b < VB + 5) {
-                for (int w = 0; w < kRedThreads / 32; ++w) v += wpart[w][5 + VB + (b - VB)];
-            } else if (b < VB + 8) {
+            } else if (b < 6) {
+                for (int w = 0; w < kRedThreads / 32; ++w) v += wpart[w][6 + (b - 1)];
+            } else if (b < 9) {
                 for (int w = 0; w < kRedThreads / 32; ++w)
-                    if ((w >> (b - VB - 5)) & 1) v += wpart[w][0];
+                    if ((w >> (b - 6)) & 1) v += wpart[w][0];
             } else if (b < TB) {
-                for (int w = 0; w < kRedThreads / 32; ++w) v += wpart[w][1 + VB + (b - VB - 8)];
+                for (int w = 0; w < kRedThreads / 32; ++w) v += wpart[w][2 + (b - 9)];
             } else if ((tile >> (b - TB)) & 1ull) {
                 for (int w = 0; w < kRedThreads / 32; ++w) v += wpart[w][0];
             }
@@ -179,6 +123,136 @@ k_expz_tiles(const typename RedT<Real>::T2 *__restrict__ psi, int n, uint64_t nt
         __syncthreads();
     }
     if (tid <= n) partials[(size_t)tid * gridDim.x + blockIdx.x] = acc.value();  // output-major
+}
+
+// A value of a thread's 16 as limbs of a 58-bit magnitude in units of 2^(E - 1080): the high 28 bits
+// and twice the low 30.
+__device__ __forceinline__ void magnitude(double v, int E, unsigned &h, unsigned &l2) {
+    const int hi = fx::abs_hi(v);
+    const int d = E - (hi >> 20);
+    unsigned long long m = ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(v);
+    m <<= 7;
+    asm("shr.b64 %0, %0, %1;" : "+l"(m) : "r"(d));  // (amounts above 63 give 0: zeros)
+    h = (unsigned)(m >> 32);
+    l2 = (unsigned)m >> 1;
+}
+
+// Sum of 16 values and the sums over the values with bit b of their index set, as a pairwise tree.
+template <typename A>
+__device__ __forceinline__ void tree16(const A *p, A &t, A *sj) {
+    A a[8], b4[4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) a[i] = p[2 * i] + p[2 * i + 1];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) b4[i] = a[2 * i] + a[2 * i + 1];
+    const A c0 = b4[0] + b4[1], c1 = b4[2] + b4[3];
+    t = c0 + c1;
+    sj[3] = c1;
+    sj[2] = b4[1] + b4[3];
+    sj[1] = (a[1] + a[3]) + (a[5] + a[7]);
+    sj[0] = ((p[1] + p[3]) + (p[5] + p[7])) + ((p[9] + p[11]) + (p[13] + p[15]));
+}
+
+constexpr int kRunBits = 4;            // at most: low tile bits with sums of their own
+constexpr int kSqLow = 600;            // exponents whose squares the integer form takes
+constexpr unsigned kSqSpan = 900;
+
+// complex128: blocks take runs of 2^m consecutive tiles.
+__global__ void __launch_bounds__(kRedThreads, 2)
+k_expz_c128(const double2 *__restrict__ psi, int n, int m, uint64_t nruns, double *__restrict__ partials) {
+    constexpr int TB = RedT<double>::TB;
+    // per-warp values: [0] total, [1..4] j bits, [5..8] low tile bits, [9..13] lane bits
+    __shared__ double wpart[kRedThreads / 32][14];
+    const int tid = threadIdx.x;
+    const int lane = tid & 31;
+    const int warp = tid >> 5;
+    double acc = 0;  // output `tid` of this block, over its runs
+    for (uint64_t run = blockIdx.x; run < nruns; run += gridDim.x) {
+        double tot = 0, s8[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // j bits, then low tile bits
+        for (int tl = 0; tl < (1 << m); ++tl) {
+            const double2 *base = psi + (((run << m) | (uint64_t)tl) << TB);
+            double2 q[kJ];
+#pragma unroll
+            for (int j = 0; j < kJ; ++j) q[j] = base[j * kRedThreads + tid];
+            int top = 0;
+#pragma unroll
+            for (int j = 0; j < kJ; ++j) top = max(top, max(fx::abs_hi(q[j].x), fx::abs_hi(q[j].y)));
+            const int E = top >> 20;
+            double t, sj[4];
+            if ((unsigned)(E - kSqLow) < kSqSpan) {
+                unsigned long long p[kJ], ti, si[4];
+#pragma unroll
+                for (int j = 0; j < kJ; ++j) {
+                    unsigned xh, xl, yh, yl;
+                    magnitude(q[j].x, E, xh, xl);
+                    magnitude(q[j].y, E, yh, yl);
+                    const unsigned long long mid = (unsigned long long)xh * xl + (unsigned long long)yh * yl +
+                                                   ((unsigned long long)__umulhi(xl, xl) + __umulhi(yl, yl));
+                    p[j] = (unsigned long long)xh * xh + (unsigned long long)yh * yh + (mid >> 30);
+                }
+                tree16(p, ti, si);
+                const int sc = 2 * E - 2100;
+                t = fx::to_f64((long long)ti, sc);
+#pragma unroll
+                for (int b = 0; b < 4; ++b) sj[b] = fx::to_f64((long long)si[b], sc);
+            } else {  // zeros, infinities, NaN, or squares out of range
+                double p[kJ];
+#pragma unroll
+                for (int j = 0; j < kJ; ++j) p[j] = fma(q[j].x, q[j].x, q[j].y * q[j].y);
+                tree16(p, t, sj);
+            }
+            tot += t;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) s8[b] += sj[b];
+#pragma unroll
+            for (int b = 0; b < kRunBits; ++b)
+                if ((tl >> b) & 1) s8[4 + b] += t;
+        }
+        // butterfly over the lane bits: before step b, tot sums the 2^b lanes that differ from
+        // this one below bit b; the half with bit b set is this lane's tot or its partner's
+        double lb[5];
+#pragma unroll
+        for (int b = 0; b < 5; ++b) {
+            const double pt = __shfl_xor_sync(0xffffffffu, tot, 1 << b);
+#pragma unroll
+            for (int c = 0; c < b; ++c) lb[c] += __shfl_xor_sync(0xffffffffu, lb[c], 1 << b);
+            lb[b] = ((lane >> b) & 1) ? tot : pt;
+            tot += pt;
+        }
+        // the eight other sums at once: each step trades half of them with the partner lane; sum i
+        // ends in the lanes with lane / 4 == i
+#pragma unroll
+        for (int w = 4, of = 16; w > 0; w >>= 1, of >>= 1) {
+            const bool up = lane & of;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (i < w) s8[i] = (up ? s8[i + w] : s8[i]) + __shfl_xor_sync(0xffffffffu, up ? s8[i] : s8[i + w], of);
+        }
+        double v8 = s8[0];
+        v8 += __shfl_xor_sync(0xffffffffu, v8, 2);
+        v8 += __shfl_xor_sync(0xffffffffu, v8, 1);
+        if (lane == 0) {
+            wpart[warp][0] = tot;
+#pragma unroll
+            for (int b = 0; b < 5; ++b) wpart[warp][9 + b] = lb[b];
+        }
+        if ((lane & 3) == 0) wpart[warp][1 + (lane >> 2)] = v8;
+        __syncthreads();
+        if (tid <= n) {
+            const int b = tid;
+            double v = 0;
+            if (b >= 5 && b < 8) {
+                for (int w = 0; w < kRedThreads / 32; ++w)
+                    if ((w >> (b - 5)) & 1) v += wpart[w][0];
+            } else if (b == n || b < TB + m || ((run >> (b - TB - m)) & 1ull)) {
+                const int at = b == n ? 0 : b < 5 ? 9 + b : b < TB ? 1 + (b - 8) : b < TB + m ? 5 + (b - TB) : 0;
+                for (int w = 0; w < kRedThreads / 32; ++w) v += wpart[w][at];
+            }
+            acc += v;
+        }
+        __syncthreads();
+    }
+    if (tid <= n) partials[(size_t)tid * gridDim.x + blockIdx.x] = acc;  // output-major
 }
 
 // Fixed-order sum of the per-block partials (output-major: partials[b * nblocks + g]); one
@@ -245,7 +319,7 @@ template <typename Real>
 cudaError_t expect_z_impl(const void *psi, int n, double *scratch, double *out_z, double *out_norm2,
                           cudaStream_t st) {
     using T2 = typename RedT<Real>::T2;
-    constexpr int TB = RedT<Real>::VB + 8 + 4;
+    constexpr int TB = RedT<Real>::TB;
     const T2 *p = reinterpret_cast<const T2 *>(psi);
     if (n < TB) {
         k_expz_small<Real><<<1, kRedThreads, 0, st>>>(p, n, out_z, out_norm2);
@@ -253,13 +327,18 @@ cudaError_t expect_z_impl(const void *psi, int n, double *scratch, double *out_z
     }
     static const int occ = [] {
         int o = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_expz_tiles<Real>, kRedThreads, 0) != cudaSuccess || o < 1) o = 1;
-        return o;
+        cudaError_t e;
+        if constexpr (sizeof(Real) == 8) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_expz_c128, kRedThreads, 0);
+        else e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_expz_c64, kRedThreads, 0);
+        return e != cudaSuccess || o < 1 ? 1 : o;
     }();
-    const uint64_t ntiles = 1ull << (n - TB);
+    // complex128: runs as long as at least 4096 are left to share out over the ~300 blocks
+    const int m = sizeof(Real) == 8 ? std::min(kRunBits, std::max(0, n - TB - 12)) : 0;
+    const uint64_t nruns = 1ull << (n - TB - m);
     const uint64_t cap = std::min<uint64_t>((uint64_t)kRedMaxBlocks, (uint64_t)device_sm_count() * occ);
-    const int grid = (int)std::min<uint64_t>(ntiles, cap);
-    k_expz_tiles<Real><<<grid, kRedThreads, 0, st>>>(p, n, ntiles, scratch);
+    const int grid = (int)std::min<uint64_t>(nruns, cap);
+    if constexpr (sizeof(Real) == 8) k_expz_c128<<<grid, kRedThreads, 0, st>>>(p, n, m, nruns, scratch);
+    else k_expz_c64<<<grid, kRedThreads, 0, st>>>(p, n, nruns, scratch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_expz_final<<<1, 1024, 0, st>>>(scratch, grid, n, out_z, out_norm2);

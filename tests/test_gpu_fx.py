@@ -91,3 +91,45 @@ def test_infinities_and_nan_stay_in_their_pairs():
                 bad[k] = bad[k ^ (1 << t)] = True
             assert np.all(np.isfinite(got[~bad]))
             assert not np.any(np.isfinite(got[[4, 9, 300]]))
+
+
+@pytest.mark.parametrize("n", [12, 13, 16])
+@pytest.mark.parametrize("kind", ["plain", "zeros", "spread", "small", "tiny"])
+def test_expect_z_integer_sums(n, kind):
+    """<Z_i> of complex128 with 16 values per thread summed as integers. Bound 2^-47 of the norm: each
+    value loses at most 2^-54 of its thread's largest (16 of them: 2^-50 of that thread's sum), and the
+    float64 additions above round at most 2^6 times along any path."""
+    import paper_2411_18354_gb300 as qs
+
+    rng = np.random.default_rng([n, len(kind)])
+    v = rng.standard_normal(1 << n) + 1j * rng.standard_normal(1 << n)
+    if kind == "zeros":
+        v[rng.random(1 << n) < 0.9] = 0
+    elif kind == "spread":
+        v *= 2.0 ** rng.integers(-60, 61, 1 << n)
+    elif kind == "small":  # around the exponents where float64 squares take over
+        v *= 2.0 ** rng.integers(-440, -400, 1 << n)
+    elif kind == "tiny":
+        v *= 2.0 ** -500
+    with qs.State(n, "c128") as st:
+        st.from_numpy(v)
+        z, norm2 = st.expect_z()
+    p = v.real.astype(np.longdouble) ** 2 + v.imag.astype(np.longdouble) ** 2
+    k = np.arange(1 << n)
+    total = p.sum()
+    assert abs(norm2 - total) <= 2.0 ** -47 * total
+    for q in range(n):
+        assert abs(z[q] - (p * (1 - 2 * ((k >> q) & 1))).sum()) <= 2.0 ** -47 * total
+
+
+@pytest.mark.parametrize("n", [24, 25, 26, 27])
+def test_expect_z_runs_of_tiles(n):
+    """Runs of 1, 2, 4, 8 tiles: basis states whose bits differ in and around the run's tile bits."""
+    import paper_2411_18354_gb300 as qs
+
+    with qs.State(n, "c128") as st:
+        for k in (0, 1 << 12, 5 << 13, 3 << 15, (1 << n) - 1, (1 << (n - 1)) | 0x5A5A):
+            st.set_basis(k)
+            z, norm2 = st.expect_z()
+            assert norm2 == 1.0
+            assert np.array_equal(z, np.array([1.0 - 2.0 * ((k >> i) & 1) for i in range(n)]))

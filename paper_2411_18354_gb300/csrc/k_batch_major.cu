@@ -15,7 +15,7 @@ constexpr uint32_t kObsChunk = 1u << 14;  // amplitudes per block of the energy 
 // psi_s = |0...0> for every state; cs[s][p] = (cos, sin) of theta / 2 for its parameters.
 template <typename Real>
 __global__ void __launch_bounds__(kBmThreads) k_bm_init(typename CxT<Real>::T *__restrict__ psi, int n, int S,
-                                                       Real *__restrict__ cs, int nparam,
+                                                       double *__restrict__ cs, int nparam,
                                                        const double *__restrict__ theta,
                                                        const uint64_t *__restrict__ param_off,
                                                        const int *__restrict__ gstate) {
@@ -33,8 +33,59 @@ __global__ void __launch_bounds__(kBmThreads) k_bm_init(typename CxT<Real>::T *_
         const uint64_t s = j / nparam, p = j % nparam;
         double sn, c;
         sincos(0.5 * theta[param_off[gstate[s]] + p], &sn, &c);
-        cs[2 * j] = (Real)c;
-        cs[2 * j + 1] = (Real)sn;
+        cs[2 * j] = c;
+        cs[2 * j + 1] = sn;
+    }
+}
+
+// One thread per (pass, state): the matrices of the pass's parameterised gates for the state's angles,
+// in the order they are applied. A divided rotation [c -s; s c] (the dagger in the sweep) holds
+// {q, q, -q, -q, which} with the larger of c, s divided out; the next full one is multiplied by the
+// product of what was divided out so far, and each derivative product is scaled by its square.
+template <typename Real>
+__global__ void __launch_bounds__(64) k_bm_mats(const BatchMatPass *__restrict__ passes,
+                                                const BatchMatGate *__restrict__ gates, int S,
+                                                const double *__restrict__ cs, int nparam, Real *__restrict__ mats) {
+    const BatchMatPass P = passes[blockIdx.x];
+    const int s = blockIdx.y * 64 + threadIdx.x;
+    if (s >= S) return;
+    Real *row = mats + P.off + (uint64_t)s * P.words;
+    double pending = 1.0;
+    for (int j = 0; j < P.count; ++j, row += 8) {
+        const BatchMatGate G = gates[P.begin + j];
+        const double *v = cs + 2 * ((uint64_t)s * nparam + G.pidx);
+        const double c = v[0], sn = G.adjoint ? -v[1] : v[1];
+        if (G.adjoint) (mats + P.off + (uint64_t)s * P.words + 8 * P.count)[j] = (Real)(pending * pending);
+        Real u[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        if (G.kind == BM_RY_DIVIDED) {
+            const bool wide = fabs(sn) > fabs(c);
+            const double d = wide ? sn : c, q = (wide ? c : sn) / d;
+            u[0] = u[1] = (Real)q;
+            u[2] = u[3] = (Real)-q;
+            u[4] = wide ? (Real)1 : (Real)0;
+            pending *= d;
+        } else if (G.kind == BM_RY_FULL || G.kind == BM_RY_CONTROLLED) {
+            const double f = G.kind == BM_RY_FULL ? pending : 1.0;
+            if (G.kind == BM_RY_FULL) pending = 1.0;
+            u[0] = u[6] = (Real)(c * f);
+            u[2] = (Real)(-sn * f);
+            u[4] = (Real)(sn * f);
+            if (sizeof(Real) == 4) {  // for packed multiply-adds
+                u[1] = u[0];
+                u[3] = u[2];
+                u[5] = u[4];
+                u[7] = u[6];
+            }
+        } else if (G.kind == BM_RZ_SIDE) {  // diag(1, e^{i theta}): the global phase is left out
+            u[0] = (Real)(c * c - sn * sn);
+            u[1] = (Real)(2.0 * c * sn);
+        } else {
+            u[0] = u[6] = (Real)c;
+            u[1] = (Real)-sn;
+            u[7] = (Real)sn;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) row[i] = u[i];
     }
 }
 
@@ -98,32 +149,36 @@ __global__ void __launch_bounds__(kBmThreads) k_bm_energy(const double *__restri
 }
 
 // dE/dtheta_p = 2 sum over the gates p drives (in program order) of the per-tile partials of
-// Re <lambda| dU psi>: block per state, thread per parameter. items[csr_ptr[p] .. csr_ptr[p+1])
-// are the offsets of p's gates' partial blocks ([J][state][tile] of their sweep pass).
+// Re <lambda| dU psi>: block per state, a warp per parameter (lane l adds tiles l, l + 32, ..., then a
+// fixed-order shuffle reduction; a thread per parameter took 39 us for 70 states of 128 tiles).
+// items[csr_ptr[p] .. csr_ptr[p+1]) are the offsets of p's gates' partial blocks ([J][state][tile] of
+// their sweep pass).
 __global__ void __launch_bounds__(kBmThreads) k_bm_grad(const double *__restrict__ part, const int *__restrict__ csr_ptr,
                                                        const uint64_t *__restrict__ items, int nparam, int S,
                                                        uint32_t tiles, double *__restrict__ grad,
                                                        const uint64_t *__restrict__ param_off,
                                                        const int *__restrict__ gstate) {
-    const int s = blockIdx.x;
-    for (int p = threadIdx.x; p < nparam; p += blockDim.x) {
+    const int s = blockIdx.x, lane = threadIdx.x & 31;
+    for (int p = threadIdx.x >> 5; p < nparam; p += kBmThreads / 32) {
         double g = 0.0;
         for (int it = csr_ptr[p]; it < csr_ptr[p + 1]; ++it) {
             const double *q = part + items[it] + (uint64_t)s * tiles;
-            for (uint32_t t = 0; t < tiles; ++t) g += q[t];
+            for (uint32_t t = lane; t < tiles; t += 32) g += q[t];
         }
-        grad[param_off[gstate[s]] + p] = 2.0 * g;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+        if (lane == 0) grad[param_off[gstate[s]] + p] = 2.0 * g;
     }
 }
 
 template <typename Real>
-cudaError_t init_impl(void *psi, int n, int S, void *cs, int nparam, const double *theta, const uint64_t *param_off,
+cudaError_t init_impl(void *psi, int n, int S, double *cs, int nparam, const double *theta, const uint64_t *param_off,
                       const int *gstate, cudaStream_t st) {
     const uint64_t work = std::max<uint64_t>((uint64_t)S << n, (uint64_t)S * nparam);
     const unsigned grid = (unsigned)std::min<uint64_t>((work + kBmThreads - 1) / kBmThreads,
                                                        (uint64_t)device_sm_count() * 8);
     k_bm_init<Real><<<std::max(1u, grid), kBmThreads, 0, st>>>(static_cast<typename CxT<Real>::T *>(psi), n, S,
-                                                                static_cast<Real *>(cs), nparam, theta, param_off,
+                                                                cs, nparam, theta, param_off,
                                                                 gstate);
     return cudaGetLastError();
 }
@@ -148,10 +203,19 @@ size_t bm_obs_partials(int n, int S) {
     return (size_t)S * (size_t)std::max<uint64_t>(1, N / kObsChunk);
 }
 
-cudaError_t launch_bm_init(int dtype, void *psi, int n, int S, void *cs, int nparam, const double *theta,
+cudaError_t launch_bm_init(int dtype, void *psi, int n, int S, double *cs, int nparam, const double *theta,
                            const uint64_t *param_off, const int *gstate, cudaStream_t st) {
     return dtype == QS_C64 ? init_impl<float>(psi, n, S, cs, nparam, theta, param_off, gstate, st)
                            : init_impl<double>(psi, n, S, cs, nparam, theta, param_off, gstate, st);
+}
+
+cudaError_t launch_bm_mats(int dtype, const BatchMatPass *passes, int npasses, const BatchMatGate *gates, int S,
+                           const double *cs, int nparam, void *mats, cudaStream_t st) {
+    if (npasses == 0 || S == 0) return cudaSuccess;
+    const dim3 grid((unsigned)npasses, (unsigned)((S + 63) / 64));
+    if (dtype == QS_C64) k_bm_mats<float><<<grid, 64, 0, st>>>(passes, gates, S, cs, nparam, static_cast<float *>(mats));
+    else k_bm_mats<double><<<grid, 64, 0, st>>>(passes, gates, S, cs, nparam, static_cast<double *>(mats));
+    return cudaGetLastError();
 }
 
 cudaError_t launch_bm_obs(int dtype, const void *psi, void *lam, int n, int S, double *part, double *energy,

@@ -34,6 +34,7 @@ namespace {
 constexpr uint32_t kBatchMagic = 0x51534254u;  // "QSBT"
 constexpr int kBatchMaxQubits = 30;
 constexpr int kBatchMaxParams = 4096;
+constexpr int kSide = 3;  // parallel branches of a pass-major graph beside the first
 }  // namespace
 
 // A program of the pass-major path (QS_FLAG_JIT): its states side by side in one buffer, every
@@ -41,9 +42,16 @@ constexpr int kBatchMaxParams = 4096;
 struct BatchJitProg {
     int n = 0, nparam = 0;
     std::vector<int> states;        // global state indices
+    std::vector<qs_gate> gates;     // of each state, until its programs are planned
+    bool planned = false;
     qs::FusedProgram pf, pa;        // forward and sweep programs (rotation kinds / indices filled in)
     std::vector<qs::JitPass> jf, ja;
-    void *psi = nullptr, *lam = nullptr, *cs = nullptr;
+    void *psi = nullptr, *lam = nullptr;
+    double *cs = nullptr;                     // (cos, sin) of theta / 2 per state and parameter
+    void *mats = nullptr;                     // every pass's matrices of the parameterised gates, per state
+    qs::BatchMatPass *d_mpass = nullptr;      // forward passes, then sweep passes
+    qs::BatchMatGate *d_mgate = nullptr;
+    std::vector<uint64_t> mat_off;            // per pass: its first real in mats
     double *part = nullptr, *obs = nullptr;  // sweep gradient partials, energy partials
     int *d_states = nullptr, *d_csr = nullptr;
     uint64_t *d_items = nullptr;
@@ -61,6 +69,7 @@ struct qs_batch {
     int grid = 0;
     size_t smem = 0;
     int small_bits = 0, tile_bits = 0, max_pass_gates = 0;
+    int major_f = 0, major_a = 0, major_gates = 0;  // pass-major: tile bits forward and sweep, gates per pass
     // device buffers
     void *d_states = nullptr, *d_order = nullptr, *d_progs = nullptr, *d_passes = nullptr, *d_gates = nullptr;
     void *d_groups = nullptr;
@@ -72,6 +81,8 @@ struct qs_batch {
     double *g_energy = nullptr, *g_grad = nullptr;
     int g_flags = 0;
     cudaStream_t capture_stream = nullptr;
+    cudaStream_t side[kSide] = {};      // capture only: branches of the graph (enqueue_jit)
+    cudaEvent_t joins[1 + kSide] = {};
     // pass-major path (QS_FLAG_JIT): programs of the states above small_bits, prepared on first use
     std::vector<BatchJitProg> jprogs;
     std::vector<int32_t> small_order;  // the states at or below small_bits, largest first
@@ -87,8 +98,12 @@ namespace {
 void free_batch(qs_batch *b) {
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->capture_stream) cudaStreamDestroy(b->capture_stream);
+    for (cudaStream_t st : b->side)
+        if (st) cudaStreamDestroy(st);
+    for (cudaEvent_t ev : b->joins)
+        if (ev) cudaEventDestroy(ev);
     for (BatchJitProg &jp : b->jprogs)
-        for (void *p : {jp.psi, jp.lam, jp.cs, (void *)jp.part, (void *)jp.obs, (void *)jp.d_states, (void *)jp.d_csr,
+        for (void *p : {jp.psi, jp.lam, (void *)jp.cs, jp.mats, (void *)jp.d_mpass, (void *)jp.d_mgate, (void *)jp.part, (void *)jp.obs, (void *)jp.d_states, (void *)jp.d_csr,
                         (void *)jp.d_items})
             if (p) cudaFree(p);
     if (b->d_small_order) cudaFree(b->d_small_order);
@@ -155,11 +170,57 @@ bool plan_pair(int n, int dtype, const qs_gate &g, int nparam, GatePlan *fwd, Ga
 }
 
 // Compile the pass-major path's kernels and allocate its buffers (first QS_FLAG_JIT run).
+// The pass-major path's programs of one gate list: every rotation its own gate (a compiled pass applies
+// RY in 2 and a one-sided phase in 4 multiply-adds per output pair, a merged RZ RY in 16), and
+// uncontrolled RZ(theta) = e^{-i theta / 2} diag(1, e^{i theta}) one-sided: the global phase changes
+// neither the energy nor a derivative (plan_adjoint_gates). Planned when first needed: a batch that
+// only runs in the persistent kernel does not pay for it.
+void plan_major(const qs_batch *b, BatchJitProg &jp) {
+    if (jp.planned) return;
+    const int n = jp.n, dtype = b->dtype;
+    const std::vector<qs_gate> &gs = jp.gates;
+    const size_t gc = gs.size();
+    char err[256];
+    std::vector<GatePlan> fwd(gc), adj(gc);
+    std::vector<int> slots(gc, -1);
+    for (size_t i = 0; i < gc; ++i) {  // (the records were validated by qs_batch_create)
+        plan_pair(n, dtype, gs[i], jp.nparam, &fwd[i], &adj[i], err, sizeof(err));
+        if (gs[i].kind == QS_GATE_RY || gs[i].kind == QS_GATE_RZ) slots[i] = gs[i].param;
+    }
+    for (size_t i = 0; i < gc; ++i) {
+        if (gs[i].kind != QS_GATE_RZ || gs[i].ctrl_mask != 0) continue;
+        static const double kPhase[8] = {1.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.6, 0.8};  // structure only
+        for (GatePlan *p : {&fwd[i], &adj[i]}) {
+            GatePlan q;
+            if (!plan_gate(n, dtype, gs[i].target, 0, 0, kPhase, QS_GATE_U, OP_SIDE, &q, err, sizeof(err))) continue;
+            q.side = 1;
+            *p = q;
+        }
+    }
+    std::vector<int> seq(gc);
+    std::iota(seq.begin(), seq.end(), 0);
+    plan_fused(n, dtype, std::min(b->major_f, n), seq, fwd, nullptr, &jp.pf, b->major_gates, false, kGroupBits, true);
+    std::reverse(seq.begin(), seq.end());
+    plan_fused(n, dtype, std::min(b->major_a, n), seq, adj, &slots, &jp.pa, b->major_gates, false, kGroupBitsAdjoint, true);
+    for (FusedProgram *p : {&jp.pf, &jp.pa})
+        for (size_t i = 0; i < p->gates.size(); ++i) {
+            RegGate &G = p->gates[i];
+            const qs_gate &src = gs[p->gate_src[i]];
+            const bool rot = src.kind == QS_GATE_RY || src.kind == QS_GATE_RZ;
+            G.pkind = rot ? src.kind : 0;
+            G.pidx = rot ? src.param : 0;
+            G.slot = rot && p == &jp.pa ? src.param : -1;
+        }
+    jp.gates = {};
+    jp.planned = true;
+}
+
 qs_status ensure_jit(qs_batch *b) {
     if (b->jit_ready) return QS_OK;
     const size_t es = elem_bytes(b->dtype), rs = es / 2;
     std::vector<JitRequest> reqs;
     for (BatchJitProg &jp : b->jprogs) {
+        plan_major(b, jp);
         reqs.push_back({&jp.pf, false, true, &jp.jf});
         reqs.push_back({&jp.pa, true, true, &jp.ja});
     }
@@ -203,6 +264,25 @@ qs_status ensure_jit(qs_batch *b) {
             total += (size_t)J * S * (size_t)P.ntiles;
             if (P.ntiles != jp.tiles) return set_error(QS_EUNSUPPORTED, "qs_batch_run: passes of unequal tile counts");
         }
+        // the matrices of each pass's parameterised gates, per state
+        std::vector<BatchMatPass> mp;
+        std::vector<BatchMatGate> mg;
+        uint64_t mat_reals = 0;
+        jp.mat_off.clear();
+        for (int dir = 0; dir < 2; ++dir) {
+            const FusedProgram &prog = dir ? jp.pa : jp.pf;
+            for (size_t i = 0; i < prog.passes.size(); ++i) {
+                BatchMatPass m{};
+                m.begin = (int32_t)mg.size();
+                jit_batch_gates(prog, (int)i, dir != 0, &mg);
+                m.count = (int32_t)mg.size() - m.begin;
+                m.words = jit_batch_words(m.count, dir != 0);
+                m.off = mat_reals;
+                mat_reals += (uint64_t)m.words * S;
+                jp.mat_off.push_back(m.off);
+                mp.push_back(m);
+            }
+        }
         std::vector<int> csr(jp.nparam + 1, 0);
         std::vector<uint64_t> flat;
         for (int q = 0; q < jp.nparam; ++q) {
@@ -211,13 +291,15 @@ qs_status ensure_jit(qs_batch *b) {
         }
         csr[jp.nparam] = (int)flat.size();
         if (!dev_alloc(&jp.psi, (size_t)S * N * es) || !dev_alloc(&jp.lam, (size_t)S * N * es) ||
-            !dev_alloc(&jp.cs, (size_t)S * std::max(1, jp.nparam) * 2 * rs) ||
+            !dev_alloc((void **)&jp.cs, (size_t)S * std::max(1, jp.nparam) * 2 * sizeof(double)) ||
+            !dev_alloc(&jp.mats, mat_reals * rs) ||
             !dev_alloc((void **)&jp.part, total * sizeof(double)) ||
             !dev_alloc((void **)&jp.obs, bm_obs_partials(jp.n, S) * sizeof(double)))
             return set_error(QS_ENOMEM, "qs_batch_run: cannot allocate the pass-major state buffers");
         qs_status st;
         if ((st = upload(jp.states, (void **)&jp.d_states)) != QS_OK || (st = upload(csr, (void **)&jp.d_csr)) != QS_OK ||
-            (st = upload(flat, (void **)&jp.d_items)) != QS_OK)
+            (st = upload(flat, (void **)&jp.d_items)) != QS_OK || (st = upload(mp, (void **)&jp.d_mpass)) != QS_OK ||
+            (st = upload(mg, (void **)&jp.d_mgate)) != QS_OK)
             return st;
         jp.pass_off.push_back(total);  // end marker: total partials
     }
@@ -228,38 +310,71 @@ qs_status ensure_jit(qs_batch *b) {
     return QS_OK;
 }
 
-// Enqueue one pass-major run on `st`: the small states in the persistent kernel, then every
-// larger program's passes over all its states.
-cudaError_t enqueue_jit(qs_batch *b, const BatchArgs &a0, cudaStream_t st) {
+// Enqueue one program of a pass-major run on `st`: its passes over all its states.
+cudaError_t enqueue_program(qs_batch *b, BatchJitProg &jp, const BatchArgs &a0, cudaStream_t st) {
+    const int S = (int)jp.states.size();
+    const uint64_t N = 1ull << jp.n;
+    const size_t rs = elem_bytes(b->dtype) / 2, nf = jp.pf.passes.size(), na = jp.pa.passes.size();
+    auto mats = [&](size_t pass) { return static_cast<const char *>(jp.mats) + jp.mat_off[pass] * rs; };
+    cudaError_t e = launch_bm_init(b->dtype, jp.psi, jp.n, S, jp.cs, jp.nparam, a0.theta, b->d_param_off, jp.d_states, st);
+    if (e == cudaSuccess)
+        e = launch_bm_mats(b->dtype, jp.d_mpass, (int)(nf + na), jp.d_mgate, S, jp.cs, jp.nparam, jp.mats, st);
+    for (size_t i = 0; e == cudaSuccess && i < nf; ++i)
+        e = launch_jit_pass_batched(b->dtype, jp.jf[i], jp.pf, (int)i, jp.psi, nullptr, nullptr, N, S, mats(i), st);
+    if (e == cudaSuccess)
+        e = launch_bm_obs(b->dtype, jp.psi, jp.lam, jp.n, S, jp.obs, a0.energy, jp.d_states, st);
+    if (e == cudaSuccess && jp.pass_off.back() > 0)
+        e = cudaMemsetAsync(jp.part, 0, jp.pass_off.back() * sizeof(double), st);
+    for (size_t i = 0; e == cudaSuccess && i < na; ++i)
+        e = launch_jit_pass_batched(b->dtype, jp.ja[i], jp.pa, (int)i, jp.psi, jp.lam, jp.part + jp.pass_off[i], N, S,
+                                    mats(nf + i), st);
+    if (e == cudaSuccess)
+        e = launch_bm_grad(jp.part, jp.d_csr, jp.d_items, jp.nparam, S, jp.tiles, a0.grad, b->d_param_off,
+                           jp.d_states, st);
+    return e;
+}
+
+// The branches' streams and events (before the capture that uses them).
+cudaError_t ensure_branches(qs_batch *b) {
     cudaError_t e = cudaSuccess;
-    if (!b->small_order.empty()) {
+    for (int i = 0; i < kSide && e == cudaSuccess; ++i)
+        if (!b->side[i]) e = cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking);
+    for (int i = 0; i <= kSide && e == cudaSuccess; ++i)
+        if (!b->joins[i]) e = cudaEventCreateWithFlags(&b->joins[i], cudaEventDisableTiming);
+    return e;
+}
+
+// Enqueue one pass-major run on `st`: the small states in the persistent kernel, then every larger
+// program's passes over all its states. The programs are independent (own buffers, own states'
+// outputs); `fork` (while st is being captured into a graph) puts them on parallel branches, the
+// largest on st itself, so that programs too small to fill the GPU run beside each other.
+cudaError_t enqueue_jit(qs_batch *b, const BatchArgs &a0, cudaStream_t st, bool fork) {
+    cudaError_t e = cudaSuccess;
+    cudaStream_t on[1 + kSide] = {st, st, st, st};
+    const bool small = !b->small_order.empty();
+    const int branches = fork ? std::min<int>(1 + kSide, (int)b->jprogs.size() + (small ? 1 : 0)) : 1;
+    if (branches > 1) e = cudaEventRecord(b->joins[0], st);
+    for (int i = 1; i < branches && e == cudaSuccess; ++i) {
+        on[i] = b->side[i - 1];
+        e = cudaStreamWaitEvent(on[i], b->joins[0], 0);
+    }
+    int next = 0;  // the largest program takes st, the others the side branches in turn
+    auto branch = [&]() { return branches > 1 ? (next == 0 ? next++, 0 : 1 + (next++ - 1) % (branches - 1)) : 0; };
+    for (BatchJitProg &jp : b->jprogs)
+        if (e == cudaSuccess) e = enqueue_program(b, jp, a0, on[branch()]);
+    if (e == cudaSuccess && small) {
         BatchArgs a = a0;
         a.order = b->d_small_order;
         a.num_states = (int)b->small_order.size();
-        e = cudaMemsetAsync(b->queue, 0, sizeof(int), st);
-        if (e == cudaSuccess) e = launch_batch(b->dtype, a, b->grid, b->smem, st);
-        if (e != cudaSuccess) return e;
+        cudaStream_t q = on[branch()];
+        e = cudaMemsetAsync(b->queue, 0, sizeof(int), q);
+        if (e == cudaSuccess) e = launch_batch(b->dtype, a, b->grid, b->smem, q);
     }
-    for (BatchJitProg &jp : b->jprogs) {
-        const int S = (int)jp.states.size();
-        const uint64_t N = 1ull << jp.n;
-        e = launch_bm_init(b->dtype, jp.psi, jp.n, S, jp.cs, jp.nparam, a0.theta, b->d_param_off, jp.d_states, st);
-        for (size_t i = 0; e == cudaSuccess && i < jp.pf.passes.size(); ++i)
-            e = launch_jit_pass_batched(b->dtype, jp.jf[i], jp.pf, (int)i, jp.psi, nullptr, nullptr, N, S, jp.cs,
-                                        2u * (uint32_t)jp.nparam, st);
-        if (e == cudaSuccess)
-            e = launch_bm_obs(b->dtype, jp.psi, jp.lam, jp.n, S, jp.obs, a0.energy, jp.d_states, st);
-        if (e == cudaSuccess && jp.pass_off.back() > 0)
-            e = cudaMemsetAsync(jp.part, 0, jp.pass_off.back() * sizeof(double), st);
-        for (size_t i = 0; e == cudaSuccess && i < jp.pa.passes.size(); ++i)
-            e = launch_jit_pass_batched(b->dtype, jp.ja[i], jp.pa, (int)i, jp.psi, jp.lam, jp.part + jp.pass_off[i], N,
-                                        S, jp.cs, 2u * (uint32_t)jp.nparam, st);
-        if (e == cudaSuccess)
-            e = launch_bm_grad(jp.part, jp.d_csr, jp.d_items, jp.nparam, S, jp.tiles, a0.grad, b->d_param_off,
-                               jp.d_states, st);
-        if (e != cudaSuccess) return e;
+    for (int i = 1; i < branches && e == cudaSuccess; ++i) {
+        e = cudaEventRecord(b->joins[i], on[i]);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(st, b->joins[i], 0);
     }
-    return cudaSuccess;
+    return e;
 }
 
 }  // namespace
@@ -276,6 +391,10 @@ qs_status qs_batch_create(int num_states, const int *n_qubits, const qs_gate *ga
     if (dtype == QS_Q30) return set_error(QS_EUNSUPPORTED, "qs_batch_create: batches are not built for QS_Q30 states");
     if (dtype != QS_C64 && dtype != QS_C128) return set_error(QS_EINVAL, "qs_batch_create: bad dtype");
     const int es = (int)elem_bytes(dtype);
+    // pass-major path: tiles and fusion depth of single-state compiled passes unless given
+    const int major_f = tile_bits > 0 ? tile_bits : dtype == QS_C64 ? 12 : 11;
+    const int major_a = tile_bits > 0 ? tile_bits : dtype == QS_C64 ? 11 : 10;
+    const int major_gates = max_pass_gates > 0 && max_pass_gates <= kTileMaxGates ? max_pass_gates : kPassMaxGates;
     if (small_bits <= 0) small_bits = dtype == QS_C64 ? 12 : 11;
     if (tile_bits <= 0) tile_bits = dtype == QS_C64 ? 11 : 10;
     if (max_pass_gates <= 0 || max_pass_gates > kTileMaxGates) max_pass_gates = kTileMaxGates;  // its tables' size
@@ -290,7 +409,6 @@ qs_status qs_batch_create(int num_states, const int *n_qubits, const qs_gate *ga
     std::vector<RegGate> tgates;
     std::vector<TileGroup> tgroups;
     std::map<std::string, int> prog_of;
-    std::vector<std::pair<FusedProgram, FusedProgram>> host_progs;  // per program: forward, sweep
     int max_params = 1, max_large_n = 0, max_small_n = 0, smem_bits = 5;
     char err[256], e2[512];
     for (int s = 0; s < num_states; ++s) {
@@ -368,7 +486,7 @@ qs_status qs_batch_create(int num_states, const int *n_qubits, const qs_gate *ga
                     tgroups.push_back(Gr);
                 }
                 for (size_t gi = 0; gi < fp.gates.size(); ++gi) {
-                    RegGate &G = fp.gates[gi];  // rotation fields filled in place (the pass-major path keeps fp)
+                    RegGate &G = fp.gates[gi];  // rotation fields filled in place
                     const int first = dir ? fp.gate_src[gi] : srcm[fp.gate_src[gi]].first;
                     const int second = dir ? -1 : srcm[fp.gate_src[gi]].second;
                     const qs_gate &src = gs[first];
@@ -401,7 +519,6 @@ qs_status qs_batch_create(int num_states, const int *n_qubits, const qs_gate *ga
             pid = (int)progs.size();
             progs.push_back(bp);
             prog_of.emplace(key, pid);
-            host_progs.push_back({std::move(pf), std::move(pa)});
         }
         states[s].n = n;
         states[s].prog = pid;
@@ -433,6 +550,9 @@ qs_status qs_batch_create(int num_states, const int *n_qubits, const qs_gate *ga
     b->small_bits = small_bits;
     b->tile_bits = tile_bits;
     b->max_pass_gates = max_pass_gates;
+    b->major_f = major_f;
+    b->major_a = major_a;
+    b->major_gates = major_gates;
     qs_status st;
     if ((st = upload(states, &b->d_states)) != QS_OK || (st = upload(order, &b->d_order)) != QS_OK ||
         (st = upload(progs, &b->d_progs)) != QS_OK || (st = upload(passes, &b->d_passes)) != QS_OK ||
@@ -473,8 +593,7 @@ qs_status qs_batch_create(int num_states, const int *n_qubits, const qs_gate *ga
                 BatchJitProg &jp = b->jprogs.back();
                 jp.n = states[s].n;
                 jp.nparam = states[s].nparam;
-                jp.pf = host_progs[pid].first;
-                jp.pa = host_progs[pid].second;
+                jp.gates.assign(gates + gate_offsets[s], gates + gate_offsets[s + 1]);
             }
             b->jprogs[jp_of[pid]].states.push_back(s);
         }
@@ -512,7 +631,7 @@ qs_status qs_batch_run(qs_batch *b, const double *theta, double *energy, double 
         if (st != QS_OK) return st;
     }
     auto enqueue = [&](cudaStream_t st) -> cudaError_t {
-        if (jit) return enqueue_jit(b, a, st);
+        if (jit) return enqueue_jit(b, a, st, (flags & QS_FLAG_GRAPH) != 0);
         cudaError_t e1 = cudaMemsetAsync(b->queue, 0, sizeof(int), st);
         return e1 == cudaSuccess ? launch_batch(b->dtype, a, b->grid, b->smem, st) : e1;
     };
@@ -531,6 +650,8 @@ qs_status qs_batch_run(qs_batch *b, const double *theta, double *energy, double 
             e = cudaStreamCreateWithFlags(&b->capture_stream, cudaStreamNonBlocking);
             if (e != cudaSuccess) return cuda_fail(e, "qs_batch_run: capture stream");
         }
+        if (jit) e = ensure_branches(b);
+        if (jit && e != cudaSuccess) return cuda_fail(e, "qs_batch_run: graph branches");
         e = cudaStreamBeginCapture(b->capture_stream, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return cuda_fail(e, "qs_batch_run: begin capture");
         cudaError_t e2 = enqueue(b->capture_stream);
@@ -575,7 +696,9 @@ qs_status qs_batch_bytes(const qs_batch *b, double *algorithmic_bytes) {
     // writes lambda, every sweep pass reads and writes the selected tiles of psi and lambda
     double total = 0.0;
     const double es = (double)elem_bytes(b->dtype);
-    for (const BatchJitProg &jp : b->jprogs) {
+    for (const BatchJitProg &cjp : b->jprogs) {
+        BatchJitProg &jp = const_cast<BatchJitProg &>(cjp);
+        plan_major(b, jp);
         const double state = std::ldexp(es, jp.n);
         double per = 3.0 * state;
         for (size_t i = 0; i < jp.pf.passes.size(); ++i) per += 2.0 * state * pass_touched_fraction(jp.pf, (int)i);

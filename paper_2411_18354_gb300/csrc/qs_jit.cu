@@ -139,22 +139,6 @@ void preamble(Out &o, bool dbl) {
         "  T2 a; a.x = F(ar, x.x, -ai * x.y); a.y = F(ar, x.y, ai * x.x); x = a;\n}\n");
     o.f("__device__ __forceinline__ void u_diag(T2 &x, T2 &y, const R *m) { u_mul(x, m[0], m[1]); u_mul(y, m[6], m[7]); }\n");
     o.f("__device__ __forceinline__ void u_swap(T2 &x, T2 &y) { T2 t = x; x = y; y = t; }\n");
-    // a parameterised gate from (c, s) = (cos, sin) of theta / 2: kind 2 = RY = [[c, -s], [s, c]],
-    // kind 3 = RZ = diag(c - i s, c + i s); adj: the dagger
-    o.f("__device__ __forceinline__ void pmat(int kind, R c, R s, int adj, R *u) {\n"
-        "  for (int i = 0; i < 8; ++i) u[i] = 0;\n"
-        "  u[0] = c; u[6] = c;\n"
-        "  if (kind == 2) { u[2] = adj ? s : -s; u[4] = adj ? -s : s; }\n"
-        "  else { u[1] = adj ? s : -s; u[7] = adj ? -s : s; }\n"
-        "}\n"
-        "__device__ __forceinline__ void dup(R *u) { u[1] = u[0]; u[3] = u[2]; u[5] = u[4]; u[7] = u[6]; }\n");
-    // w = a b for row-major complex 2x2 matrices (interleaved re, im)
-    o.f("__device__ __forceinline__ void mat2(const R *a, const R *b, R *w) {\n"
-        "  for (int i = 0; i < 2; ++i) for (int j = 0; j < 2; ++j) {\n"
-        "    const R *x = a + 4 * i, *y0 = b + 2 * j, *y1 = b + 4 + 2 * j;\n"
-        "    w[4 * i + 2 * j] = x[0] * y0[0] - x[1] * y0[1] + x[2] * y1[0] - x[3] * y1[1];\n"
-        "    w[4 * i + 2 * j + 1] = x[0] * y0[1] + x[1] * y0[0] + x[2] * y1[1] + x[3] * y1[0];\n"
-        "  }\n}\n");
     // Sums over the warp of M values per lane at once: each step trades half of the values with the
     // partner lane, so M sums take M - 1 + log2(32 / M) shuffles instead of 5 M; value i ends in the
     // lanes with lane / (32 / M) == i.
@@ -224,12 +208,16 @@ struct Refs {
 // of the row, so nothing grows by more than sqrt(2) per gate). The last such gate of a pass, and
 // every kRealRun-th, is applied in full with the product of the divided entries. Form 0: in full; 1:
 // rotation, 2: reflection, divided. Inner products of psi and lambda taken in between are scaled
-// back by the square of the product when the pass writes its partial sums.
+// back by the square of the product when they are summed. (Batch: only the rotations that each
+// state's angles drive; their matrices, with the products, are formed per state beforehand.)
 constexpr int kRealRun = 24;
-std::vector<int> real_forms(const RegGate *g, int count) {
+bool divisible(const RegGate &g, bool batched) {
+    return g.op == OP_REAL && g.rot && g.cqm == 0 && g.crm == 0 && g.hmask == 0 && (!batched || g.pkind == QS_GATE_RY);
+}
+std::vector<int> real_forms(const RegGate *g, int count, bool batched) {
     std::vector<int> form(count, 0), at;
     for (int i = 0; i < count; ++i)
-        if (g[i].op == OP_REAL && g[i].rot && g[i].cqm == 0 && g[i].crm == 0 && g[i].hmask == 0) at.push_back(i);
+        if (divisible(g[i], batched)) at.push_back(i);
     for (size_t j = 0; j + 1 < at.size(); ++j)
         if ((j + 1) % kRealRun != 0) form[at[j]] = g[at[j]].rot;
     return form;
@@ -451,9 +439,9 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
     const uint32_t steps = (nvec + T - 1) / T;
     const int G = P.gate_count;
     const RegGate *pg = gates + P.gate_begin;
-    // Matrix of each gate as an expression: parameters of the kernel (single
-    // state), or, in a batch, shared-memory rows formed per tile from the tile's state's angles
-    // for the parameterised gates (pm_; J = index among them).
+    // Matrix of each gate as an expression: parameters of the kernel (single state), or, in a
+    // batch, shared-memory rows for the parameterised gates (pm_; J = index among them), copied in
+    // with each tile from the matrices of the tile's state.
     std::vector<int> pj(G, -1);
     int NPG = 0;
     if (batched)
@@ -462,7 +450,7 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
     const int NP = adjoint ? (batched ? NPG : P.nparam) : 0;  // gradient accumulators
     Refs refs;
     refs.m.resize(G);
-    refs.form = batched ? std::vector<int>(G, 0) : real_forms(pg, G);
+    refs.form = real_forms(pg, G, batched);
     int nacc = 0;
     for (int i = 0; i < G; ++i) {
         char b[48];
@@ -485,17 +473,15 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
             "  for (int j = 0; j < span; ++j) if (i + j < d->count_n) atomicAdd(d->counts + i + j, 1u);\n}\n");
     }
     // parameter block: the fixed matrices of the pass's gates (U, or U^dagger in the adjoint
-    // sweep); single-state sweep: the global gradient slots of its parameterised gates; batch:
-    // the parameter indices of the parameterised gates
+    // sweep); single-state sweep: the scales and global gradient slots of its parameterised gates
     o.f("struct alignas(16) A {\n  R m[%d][8];\n", G > 0 ? G : 1);
     if (adjoint && !batched) o.f("  double f[%d];\n  int gs[%d];\n", NP > 0 ? NP : 1, NP > 0 ? NP : 1);
-    if (batched) o.f("  int pix[%d][2];\n", G > 0 ? G : 1);
     o.f("};\n");
     o.f("__device__ __forceinline__ u32 swz(u32 a) { return %s; }\n", swz_expr("a", SW).c_str());
     const int minb = jit_shape(dtype, adjoint, k).blocks;
     if (batched)
         o.f("extern \"C\" __global__ void __launch_bounds__(%d, %d) %s(T2 *__restrict__ psi, T2 *__restrict__ lam, "
-            "double *__restrict__ part, u64 stride, u64 nstates, const R *__restrict__ cs, u32 cs_stride, "
+            "double *__restrict__ part, u64 stride, u64 nstates, const R *__restrict__ mats, "
             "const __grid_constant__ A a) {\n",
             T, minb, kname);
     else if (adjoint)
@@ -511,8 +497,8 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
     o.f("  extern __shared__ __align__(16) unsigned char sm_[];\n");
     o.f("  T2 *const sm0 = reinterpret_cast<T2 *>(sm_);\n");
     o.f("  R *const sr_ = reinterpret_cast<R *>(sm0 + %u);\n", (db ? 2 : 1) * BUF);
-    if (batched) o.f("  R *const pm_ = sr_;\n");
-    const int pm_words = batched ? 8 * (NPG > 0 ? NPG : 1) : 0;
+    const int pm_state = batched ? jit_batch_words(NPG, adjoint) : 0;  // reals per state
+    const int pm_words = (db ? 2 : 1) * pm_state;
     if (adjoint) {
         o.f("  R *acc_s = sr_ + %d;\n", pm_words);
         o.f("  R *acc_c = acc_s + %d;\n", (NP > 0 ? NP : 1) * (T / 32));
@@ -584,35 +570,20 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
         }
         if (cp_guard) o.f("    }\n");
     };
-    auto loads = [&](const char *tname, const char *bname, const char *tau_name) {
+    auto loads = [&](const char *tname, const char *bname, const char *tau_name, const char *pm_index) {
         o.f("    {\n    T2 *tq = %s;\n    const T2 *gp_ = gvec(psi, %s);\n", tname, tau_name);
         copies(true, "gp_", "tq", bname);
         if (adjoint) {
             o.f("    T2 *tr = tq + %u;\n    const T2 *gl_ = gvec(lam, %s);\n", TILE, tau_name);
             copies(true, "gl_", "tr", bname);
         }
-        o.f("    }\n    cpcommit();\n");
-    };
-    // batch: the matrices of the parameterised gates for the state of tile tau_ (one thread
-    // per gate), from that state's (cos, sin) of theta / 2
-    auto stage_params = [&](const char *tau_name) {
-        if (!batched || NPG == 0) return;
-        o.f("    {\n      const R *cq = cs + (%s >> %d) * (u64)cs_stride;\n", tau_name, logt);
-        for (int i = 0; i < G; ++i) {
-            if (pj[i] < 0) continue;
-            const RegGate &R = pg[i];
-            o.f("      if (tid == %d) { R u1[8]; pmat(%d, cq[2 * a.pix[%d][0]], cq[2 * a.pix[%d][0] + 1], %d, u1);",
-                pj[i] % T, R.pkind, i, i, adjoint ? 1 : 0);
-            if (!adjoint && R.pkind2 != 0)
-                o.f(" R u2[8]; pmat(%d, cq[2 * a.pix[%d][1]], cq[2 * a.pix[%d][1] + 1], 0, u2);"
-                    " mat2(u2, u1, pm_ + %d);",
-                    R.pkind2, i, i, 8 * pj[i]);
-            else
-                o.f(" for (int q_ = 0; q_ < 8; ++q_) pm_[%d + q_] = u1[q_];", 8 * pj[i]);
-            if (!dbl && R.op == OP_REAL) o.f(" dup(pm_ + %d);", 8 * pj[i]);
-            o.f(" }\n");
+        if (pm_state > 0) {  // the matrices of the tile's state
+            const int per = dbl ? 2 : 4, chunks = pm_state / per;
+            o.f("    const R *gm_ = mats + (%s >> %d) * %dull;\n    R *sm_m = sr_ + (%s) * %d;\n", tau_name, logt, pm_state,
+                db ? pm_index : "0", pm_state);
+            o.f("    for (u32 c_ = tid; c_ < %du; c_ += %d) cp16(sm_m + c_ * %d, gm_ + c_ * %d);\n", chunks, T, per, per);
         }
-        o.f("    }\n");
+        o.f("    }\n    cpcommit();\n");
     };
     const char *skip_next = sel.empty() ? "" : "    while (nxt < ntiles && !selected(tile_base(nxt))) nxt += gridDim.x;\n";
     o.f("  u64 tau = blockIdx.x;\n");
@@ -620,7 +591,7 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
     if (db) o.f("  int cur = 0;\n");
     if (db) {
         o.f("  if (tau < ntiles) {\n    const u64 b0 = tile_base(tau);\n");
-        loads("sm0", "b0", "tau");
+        loads("sm0", "b0", "tau", "0");
         o.f("  }\n");
     }
     o.f("  while (tau < ntiles) {\n");
@@ -631,13 +602,13 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
     else
         o.f("    T2 *tp = sm0;  // one buffer\n");
     if (adjoint) o.f("    T2 *tl = tp + %u;\n", TILE);
-    stage_params("tau");
+    if (pm_state > 0) o.f("    const R *const pm_ = sr_ + %s * %d;\n", db ? "cur" : "0", pm_state);
     if (db) {
         o.f("    if (nxt < ntiles) {\n      const u64 nb = tile_base(nxt);\n      T2 *tn = sm0 + (cur ^ 1) * %u;\n", BUF);
-        loads("tn", "nb", "nxt");
+        loads("tn", "nb", "nxt", "cur ^ 1");
         o.f("      cpwait1();\n    } else {\n      cpwait0();\n    }\n");
     } else {
-        loads("tp", "base", "tau");
+        loads("tp", "base", "tau", "0");
         o.f("    cpwait0();\n");
     }
     o.f("    __syncthreads();\n");
@@ -736,10 +707,10 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
                     else o.f(", 0");
                 }
                 o.f("};\n        const R s_ = warp_sums<%d>(q_, lane);\n", M);
-                o.f("        if ((lane & %d) == 0%s) { const int j_ = (%d + (lane / %d)) * %d + warp; kahan(acc_s + j_, acc_c + j_, "
-                    "s_); } }\n",
+                o.f("        if ((lane & %d) == 0%s) { const int i_ = %d + (lane / %d), j_ = i_ * %d + warp; kahan(acc_s + j_, acc_c "
+                    "+ j_, s_%s); } }\n",
                     32 / M - 1, M > npend ? (" && lane / " + std::to_string(32 / M) + " < " + std::to_string(npend)).c_str() : "",
-                    pend0, 32 / M, T / 32);
+                    pend0, 32 / M, T / 32, batched ? (" * pm_[" + std::to_string(8 * NPG) + " + i_]").c_str() : "");
                 npend = 0;
             };
             for (int g = 0; g < Gr.gate_count; ++g) {
@@ -900,10 +871,7 @@ std::string shape_key(int dtype, bool adjoint, bool batched, const TilePass &P, 
         put(&g.rot, sizeof(g.rot));
         put(&g.hmask, sizeof(g.hmask));
         put(&g.hvals, sizeof(g.hvals));
-        if (batched) {  // the kinds of the rotations whose matrices the kernel forms
-            const int kinds[2] = {g.pkind, g.pkind2};
-            put(kinds, sizeof(kinds));
-        }
+        if (batched) put(&g.pkind, sizeof(g.pkind));  // the rotations whose matrices are each state's own
     }
     return k;
 }
@@ -1178,14 +1146,14 @@ bool jit_prepare_programs(int dtype, const std::vector<JitRequest> &reqs, std::s
         if (it.batched)
             for (int g = P.gate_begin; g < P.gate_begin + P.gate_count; ++g) npg += prog.gates[g].pkind != 0;
         const size_t NP = it.adjoint ? (size_t)std::max(1, it.batched ? npg : P.nparam) : 0;
-        const size_t pm = it.batched ? 8 * (size_t)std::max(1, npg) : 0;
-        j.smem = (jit_shape(dtype, it.adjoint, P.k).db ? 2 : 1) * (it.adjoint ? 2 : 1) * T * es +
+        const bool db = jit_shape(dtype, it.adjoint, P.k).db;
+        const size_t pm = it.batched ? (size_t)jit_batch_words(npg, it.adjoint) * (db ? 2 : 1) : 0;
+        j.smem = (db ? 2 : 1) * (it.adjoint ? 2 : 1) * T * es +
                  (pm + 2 * NP * (kTileThreads / 32)) * rs;
         j.nparam_gates = npg;
         const size_t G = P.gate_count > 0 ? P.gate_count : 1;
         size_t bytes = G * 8 * rs;
         if (it.adjoint && !it.batched) bytes = ((bytes + 7) & ~size_t(7)) + NP * (sizeof(double) + sizeof(int));
-        if (it.batched) bytes = ((bytes + 3) & ~size_t(3)) + G * 2 * sizeof(int);
         j.arg_bytes = (bytes + 15) & ~size_t(15);
         j.batched = it.batched;
     }
@@ -1268,7 +1236,7 @@ void put_matrices(const FusedProgram &prog, const TilePass &P, const std::vector
             pending *= d;
             continue;
         }
-        const bool full = g[i].op == OP_REAL && g[i].rot && pending != 1.0 && g[i].cqm == 0 && g[i].crm == 0 && g[i].hmask == 0;
+        const bool full = pending != 1.0 && divisible(g[i], false);
         for (int k = 0; k < 8; ++k) out[k] = (Real)(full ? U[k] * pending : U[k]);
         if (full) pending = 1.0;
         if (sizeof(Real) == 4 && g[i].op == OP_REAL)
@@ -1309,7 +1277,7 @@ cudaError_t launch_jit_pass(int dtype, const JitPass &jp, const FusedProgram &pr
     const size_t rs = dtype == QS_C64 ? 4 : 8;
     const size_t G1 = G > 0 ? G : 1;
     std::vector<double> scale(G);
-    put_matrices(dtype, prog, P, real_forms(g, G), blk.data(), &scale);
+    put_matrices(dtype, prog, P, real_forms(g, G, false), blk.data(), &scale);
     if (adjoint) {
         const size_t NP1 = P.nparam > 0 ? P.nparam : 1;
         double *f = reinterpret_cast<double *>(&blk[(G1 * 8 * rs + 7) & ~size_t(7)]);
@@ -1332,9 +1300,28 @@ cudaError_t launch_jit_pass(int dtype, const JitPass &jp, const FusedProgram &pr
                             adjoint ? args_adj : args_fwd, jp.smem, st);
 }
 
+int jit_batch_words(int nparam_gates, bool adjoint) {
+    return 8 * nparam_gates + (adjoint ? (nparam_gates + 3) & ~3 : 0);
+}
+
+void jit_batch_gates(const FusedProgram &prog, int p, bool adjoint, std::vector<BatchMatGate> *out) {
+    const TilePass &P = prog.passes[p];
+    const RegGate *g = prog.gates.data() + P.gate_begin;
+    const std::vector<int> form = real_forms(g, P.gate_count, true);
+    for (int i = 0; i < P.gate_count; ++i) {
+        if (g[i].pkind == 0) continue;
+        BatchMatGate d;
+        d.pidx = g[i].pidx;
+        d.kind = g[i].op == OP_REAL ? (form[i] ? BM_RY_DIVIDED : divisible(g[i], true) ? BM_RY_FULL : BM_RY_CONTROLLED)
+                                    : (g[i].op == OP_SIDE ? BM_RZ_SIDE : BM_RZ);
+        d.adjoint = adjoint;
+        out->push_back(d);
+    }
+}
+
 cudaError_t launch_jit_pass_batched(int dtype, const JitPass &jp, const FusedProgram &prog, int p, void *psi,
-                                    void *lam, double *part, uint64_t stride, uint64_t nstates, const void *cs,
-                                    uint32_t cs_stride, cudaStream_t st) {
+                                    void *lam, double *part, uint64_t stride, uint64_t nstates, const void *mats,
+                                    cudaStream_t st) {
     if (!jp.batched) return cudaErrorInvalidValue;
     cudaKernel_t kern;
     int occ = 1;
@@ -1342,22 +1329,12 @@ cudaError_t launch_jit_pass_batched(int dtype, const JitPass &jp, const FusedPro
     if (e != cudaSuccess) return e;
     const TilePass &P = prog.passes[p];
     std::vector<unsigned char> blk(jp.arg_bytes, 0);
-    const int G = P.gate_count;
-    const size_t rs = dtype == QS_C64 ? 4 : 8;
-    const size_t G1 = G > 0 ? G : 1;
-    put_matrices(dtype, prog, P, std::vector<int>(G, 0), blk.data());
-    int *pix = reinterpret_cast<int *>(blk.data() + ((G1 * 8 * rs + 3) & ~size_t(3)));
-    const RegGate *g = prog.gates.data() + P.gate_begin;
-    for (int i = 0; i < G; ++i) {
-        pix[2 * i] = g[i].pidx;
-        pix[2 * i + 1] = g[i].pidx2;
-    }
+    put_matrices(dtype, prog, P, std::vector<int>(P.gate_count, 0), blk.data());
     const uint64_t total = nstates * P.ntiles;
     const uint64_t cap = (uint64_t)device_sm_count() * occ;
     const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(total, cap));
     unsigned long long stride_ = stride, nst = nstates;
-    unsigned cs_st = cs_stride;
-    void *args[] = {&psi, &lam, &part, &stride_, &nst, const_cast<void **>(&cs), &cs_st, blk.data()};
+    void *args[] = {&psi, &lam, &part, &stride_, &nst, const_cast<void **>(&mats), blk.data()};
     return cudaLaunchKernel(reinterpret_cast<const void *>(kern), dim3(grid), dim3(kTileThreads), args, jp.smem, st);
 }
 

@@ -19,6 +19,7 @@
 #include <string>
 #include <vector>
 
+#include "k_batch_major.cuh"
 #include "qs_fuse.cuh"
 
 namespace qs {
@@ -61,12 +62,17 @@ cudaError_t launch_jit_pass(int dtype, const JitPass &jp, const FusedProgram &pr
                             double *part, size_t part_stride, cudaStream_t st);
 
 // Launch batched pass `p` over `nstates` states whose vectors start `stride` amplitudes apart at
-// psi (and lam, sweep), with their (cos, sin) of theta/2 at cs (cs_stride reals per state);
-// sweep: part receives per tile and parameterised gate J the partial of Re <lambda| dU psi> at
-// [(J * nstates + state) * tiles_per_state + tile].
+// psi (and lam, sweep); mats holds the matrices of the pass's parameterised gates, jit_batch_words
+// reals for each state; sweep: part receives per tile and parameterised gate J the partial of
+// Re <lambda| dU psi> at [(J * nstates + state) * tiles_per_state + tile].
 cudaError_t launch_jit_pass_batched(int dtype, const JitPass &jp, const FusedProgram &prog, int p, void *psi,
-                                    void *lam, double *part, uint64_t stride, uint64_t nstates, const void *cs,
-                                    uint32_t cs_stride, cudaStream_t st);
+                                    void *lam, double *part, uint64_t stride, uint64_t nstates, const void *mats,
+                                    cudaStream_t st);
+
+// The parameterised gates of batched pass `p`, in the order of their matrices (k_bm_mats fills
+// them): 8 reals each, then, in the sweep, the scale of each one's derivative product.
+int jit_batch_words(int nparam_gates, bool adjoint);
+void jit_batch_gates(const FusedProgram &prog, int p, bool adjoint, std::vector<BatchMatGate> *out);
 
 // Blocks per SM that the kernel of a pass with 2^k-amplitude tiles is compiled for, and whether
 // it has two tile buffers (the next tile is copied in while the current one is computed).
@@ -78,9 +84,8 @@ JitShape jit_shape(int dtype, bool adjoint, int k);
 
 // The generated source of one pass (exposed for tests of the generator).
 // batched: the kernel runs the pass over `nstates` states of one batch program at once (tile
-// index = state * tiles per state + tile), each state's vectors `stride` amplitudes apart,
-// the parameterised gates' matrices formed per tile from that state's (cos, sin) of theta/2
-// (RegGate pkind / pkind2 / pidx / pidx2), and in the sweep the gradient partial of every
+// index = state * tiles per state + tile), each state's vectors `stride` amplitudes apart, the
+// parameterised gates' matrices (RegGate pkind / pidx) read with each tile, and in the sweep the gradient partial of every
 // parameterised gate written per tile.
 std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const TileGroup *groups,
                             const RegGate *gates, const char *kname, bool batched = false);

@@ -13,7 +13,7 @@ static_assert(sizeof(TileGroup) % 16 == 0 && sizeof(SGate<float>) % 16 == 0 && s
               "per-pass shared-memory tables keep 16-byte alignment");
 
 template <typename Real, bool ADJ>
-__global__ void __launch_bounds__(kTileThreads, (ADJ && sizeof(Real) == 8) ? 1 : 2)
+__global__ void __launch_bounds__(kTileThreads, 2)
 k_tile_pass(typename TileT<Real>::T2 *__restrict__ psi, typename TileT<Real>::T2 *__restrict__ lam, const TilePass P,
             const TileGroup *__restrict__ groups, const RegGate *__restrict__ gates, double *__restrict__ part,
             size_t part_stride) {

@@ -19,6 +19,11 @@ namespace qs {
 
 size_t adj_partials_per_slot();
 cudaError_t launch_adj_step(int dtype, void *psi, void *lam, const GatePlan &p, double *part, cudaStream_t st);
+// Two consecutive parameterised steps that one launch can take (a one-sided Z rotation, then a Y
+// rotation of the same qubit, no controls), and that launch.
+bool adj_steps_join(const GatePlan &z, const GatePlan &y);
+cudaError_t launch_adj_step_zy(int dtype, void *psi, void *lam, const GatePlan &z, const GatePlan &y, double *part_z,
+                               double *part_y, cudaStream_t st);
 cudaError_t launch_obs_sumz(int dtype, const void *psi, void *lam, int n, cudaStream_t st);
 cudaError_t launch_sum_vec(const double *z, int n, double *out, cudaStream_t st);
 cudaError_t launch_grad_final(const double *part, int nslots, double *slot_sum, const int *slot_param,
@@ -386,7 +391,8 @@ static qs_status launch_program(qs_state *s, const FusedProgram &prog, const std
     const TileGroup *groups = dev_table ? table_groups(prog, dev_table) : nullptr;
     const RegGate *gates = dev_table ? table_gates(prog, dev_table) : nullptr;
     const DiagGate *dgates = dev_table ? table_dgates(prog, dev_table) : nullptr;
-    for (const FusedOp &op : prog.ops) {
+    for (size_t oi = 0; oi < prog.ops.size(); ++oi) {
+        const FusedOp &op = prog.ops[oi];
         const bool bad = op.drun >= 0 ? (op.drun >= (int)prog.druns.size() || !dgates)
                                       : (op.pass >= (int)prog.passes.size() ||
                                          (op.pass < 0 && (op.gate < 0 || (size_t)op.gate >= plans.size())));
@@ -403,6 +409,16 @@ static qs_status launch_program(qs_state *s, const FusedProgram &prog, const std
             e = launch_gate(s->dtype, s->psi, plans[op.gate], st);
         } else {
             const int slot = (*slots)[op.gate];
+            if (slot >= 0 && oi + 1 < prog.ops.size() && prog.ops[oi + 1].pass < 0 && prog.ops[oi + 1].drun < 0) {
+                const int next = prog.ops[oi + 1].gate;
+                if (next >= 0 && (size_t)next < plans.size() && (*slots)[next] >= 0 && adj_steps_join(plans[op.gate], plans[next])) {
+                    e = launch_adj_step_zy(s->dtype, s->psi, lam, plans[op.gate], plans[next], part + (size_t)slot * P,
+                                           part + (size_t)(*slots)[next] * P, st);
+                    if (e != cudaSuccess) return cuda_fail(e, "fused program launch (joined sweep steps)");
+                    ++oi;
+                    continue;
+                }
+            }
             e = launch_adj_step(s->dtype, s->psi, lam, plans[op.gate], slot >= 0 ? part + (size_t)slot * P : nullptr, st);
         }
         if (e != cudaSuccess) {
@@ -1136,6 +1152,13 @@ qs_status qs_adjoint_grad(qs_state *s, const qs_gate *gates, size_t count, const
     } else {
         for (size_t ii = count; ii-- > 0;) {
             const int slot = slot_of[ii];
+            if (slot >= 0 && ii > 0 && slot_of[ii - 1] >= 0 && adj_steps_join(adj[ii], adj[ii - 1])) {
+                e = launch_adj_step_zy(s->dtype, s->psi, s->lam, adj[ii], adj[ii - 1], part + (size_t)slot * P,
+                                       part + (size_t)slot_of[ii - 1] * P, stm);
+                if (e != cudaSuccess) return cuda_fail(e, "qs_adjoint_grad sweep launch");
+                --ii;
+                continue;
+            }
             e = launch_adj_step(s->dtype, s->psi, s->lam, adj[ii], slot >= 0 ? part + (size_t)slot * P : nullptr, stm);
             if (e != cudaSuccess) return cuda_fail(e, "qs_adjoint_grad sweep launch");
         }

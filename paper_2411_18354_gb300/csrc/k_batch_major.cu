@@ -38,54 +38,86 @@ __global__ void __launch_bounds__(kBmThreads) k_bm_init(typename CxT<Real>::T *_
     }
 }
 
-// One thread per (pass, state): the matrices of the pass's parameterised gates for the state's angles,
-// in the order they are applied. A divided rotation [c -s; s c] (the dagger in the sweep) holds
-// {q, q, -q, -q, which} with the larger of c, s divided out; the next full one is multiplied by the
-// product of what was divided out so far, and each derivative product is scaled by its square.
+// One warp per (pass, state), a lane per gate: the matrices of the pass's parameterised gates for the
+// state's angles, in the order they are applied. A divided rotation [c -s; s c] (the dagger in the
+// sweep) holds {q, q, -q, -q, which} with the larger of c, s divided out; the next full one is
+// multiplied by the product of what was divided out so far (a scan over the lanes, restarted after
+// each full one), and each derivative product is scaled by its square. (A thread walking a pass's
+// gates took 66 us for 70 states of 18 qubits.)
 template <typename Real>
-__global__ void __launch_bounds__(64) k_bm_mats(const BatchMatPass *__restrict__ passes,
-                                                const BatchMatGate *__restrict__ gates, int S,
-                                                const double *__restrict__ cs, int nparam, Real *__restrict__ mats) {
+__global__ void __launch_bounds__(kBmThreads) k_bm_mats(const BatchMatPass *__restrict__ passes,
+                                                       const BatchMatGate *__restrict__ gates, int S,
+                                                       const double *__restrict__ cs, int nparam,
+                                                       Real *__restrict__ mats) {
     const BatchMatPass P = passes[blockIdx.x];
-    const int s = blockIdx.y * 64 + threadIdx.x;
-    if (s >= S) return;
-    Real *row = mats + P.off + (uint64_t)s * P.words;
-    double pending = 1.0;
-    for (int j = 0; j < P.count; ++j, row += 8) {
-        const BatchMatGate G = gates[P.begin + j];
-        const double *v = cs + 2 * ((uint64_t)s * nparam + G.pidx);
-        const double c = v[0], sn = G.adjoint ? -v[1] : v[1];
-        if (G.adjoint) (mats + P.off + (uint64_t)s * P.words + 8 * P.count)[j] = (Real)(pending * pending);
-        Real u[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        if (G.kind == BM_RY_DIVIDED) {
-            const bool wide = fabs(sn) > fabs(c);
-            const double d = wide ? sn : c, q = (wide ? c : sn) / d;
-            u[0] = u[1] = (Real)q;
-            u[2] = u[3] = (Real)-q;
-            u[4] = wide ? (Real)1 : (Real)0;
-            pending *= d;
-        } else if (G.kind == BM_RY_FULL || G.kind == BM_RY_CONTROLLED) {
-            const double f = G.kind == BM_RY_FULL ? pending : 1.0;
-            if (G.kind == BM_RY_FULL) pending = 1.0;
-            u[0] = u[6] = (Real)(c * f);
-            u[2] = (Real)(-sn * f);
-            u[4] = (Real)(sn * f);
-            if (sizeof(Real) == 4) {  // for packed multiply-adds
-                u[1] = u[0];
-                u[3] = u[2];
-                u[5] = u[4];
-                u[7] = u[6];
+    const int lane = threadIdx.x & 31;
+    for (int s = blockIdx.y * (kBmThreads / 32) + (threadIdx.x >> 5); s < S; s += gridDim.y * (kBmThreads / 32)) {
+        Real *rows = mats + P.off + (uint64_t)s * P.words;
+        double carry = 1.0;  // divided out before this chunk of 32 gates
+        for (int j0 = 0; j0 < P.count; j0 += 32) {
+            const int j = j0 + lane;
+            const bool on = j < P.count;
+            BatchMatGate G{0, BM_RZ, 0};
+            double c = 1.0, sn = 0.0;
+            if (on) {
+                G = gates[P.begin + j];
+                const double *v = cs + 2 * ((uint64_t)s * nparam + G.pidx);
+                c = v[0];
+                sn = G.adjoint ? -v[1] : v[1];
             }
-        } else if (G.kind == BM_RZ_SIDE) {  // diag(1, e^{i theta}): the global phase is left out
-            u[0] = (Real)(c * c - sn * sn);
-            u[1] = (Real)(2.0 * c * sn);
-        } else {
-            u[0] = u[6] = (Real)c;
-            u[1] = (Real)-sn;
-            u[7] = (Real)sn;
-        }
+            const bool wide = fabs(sn) > fabs(c);
+            const double d = wide ? sn : c;
+            double prod = G.kind == BM_RY_DIVIDED ? d : 1.0;  // inclusive product since the last full gate
+            int full = G.kind == BM_RY_FULL;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) row[i] = u[i];
+            for (int o = 1; o < 32; o <<= 1) {
+                const double p = __shfl_up_sync(0xffffffffu, prod, o);
+                const int f = __shfl_up_sync(0xffffffffu, full, o);
+                if (lane >= o) {
+                    if (!full) prod *= p;
+                    full |= f;
+                }
+            }
+            if (!full) prod *= carry;
+            double pending = __shfl_up_sync(0xffffffffu, prod, 1);  // before this gate
+            if (lane == 0) pending = carry;
+            carry = __shfl_sync(0xffffffffu, prod, 31);
+            if (!on) continue;
+            if (G.adjoint) rows[8 * P.count + j] = (Real)(pending * pending);
+            Real u[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+            if (G.kind == BM_RY_DIVIDED) {
+                const double q = (wide ? c : sn) / d;
+                u[0] = u[1] = (Real)q;
+                u[2] = u[3] = (Real)-q;
+                u[4] = wide ? (Real)1 : (Real)0;
+            } else if (G.kind == BM_RY_FULL || G.kind == BM_RY_CONTROLLED) {
+                const double f = G.kind == BM_RY_FULL ? pending : 1.0;
+                u[0] = u[6] = (Real)(c * f);
+                u[2] = (Real)(-sn * f);
+                u[4] = (Real)(sn * f);
+                if (sizeof(Real) == 4) {  // for packed multiply-adds
+                    u[1] = u[0];
+                    u[3] = u[2];
+                    u[5] = u[4];
+                    u[7] = u[6];
+                }
+            } else if (G.kind == BM_RZ_SIDE) {  // diag(1, e^{i theta}): the global phase is left out
+                u[0] = (Real)(c * c - sn * sn);
+                u[1] = (Real)(2.0 * c * sn);
+            } else {
+                u[0] = u[6] = (Real)c;
+                u[1] = (Real)-sn;
+                u[7] = (Real)sn;
+            }
+            using V = typename CxT<Real>::T;
+#pragma unroll
+            for (int i = 0; i < 8; i += 2) {
+                V w;
+                w.x = u[i];
+                w.y = u[i + 1];
+                *reinterpret_cast<V *>(rows + 8 * j + i) = w;
+            }
+        }
     }
 }
 
@@ -149,26 +181,25 @@ __global__ void __launch_bounds__(kBmThreads) k_bm_energy(const double *__restri
 }
 
 // dE/dtheta_p = 2 sum over the gates p drives (in program order) of the per-tile partials of
-// Re <lambda| dU psi>: block per state, a warp per parameter (lane l adds tiles l, l + 32, ..., then a
-// fixed-order shuffle reduction; a thread per parameter took 39 us for 70 states of 128 tiles).
-// items[csr_ptr[p] .. csr_ptr[p+1]) are the offsets of p's gates' partial blocks ([J][state][tile] of
-// their sweep pass).
+// Re <lambda| dU psi>: block.x per state, `lanes` (a power of two <= 32) lanes per parameter, lane l
+// adding tiles l, l + lanes, ..., then a fixed-order shuffle reduction (a thread per parameter and
+// all its tiles took 39 us for 70 states of 128 tiles). items[csr_ptr[p] .. csr_ptr[p+1]) are the
+// offsets of p's gates' partial blocks ([J][state][tile] of their sweep pass).
 __global__ void __launch_bounds__(kBmThreads) k_bm_grad(const double *__restrict__ part, const int *__restrict__ csr_ptr,
-                                                       const uint64_t *__restrict__ items, int nparam, int S,
-                                                       uint32_t tiles, double *__restrict__ grad,
+                                                       const uint64_t *__restrict__ items, int nparam,
+                                                       uint32_t tiles, int lanes, double *__restrict__ grad,
                                                        const uint64_t *__restrict__ param_off,
                                                        const int *__restrict__ gstate) {
-    const int s = blockIdx.x, lane = threadIdx.x & 31;
-    for (int p = threadIdx.x >> 5; p < nparam; p += kBmThreads / 32) {
-        double g = 0.0;
+    const int s = blockIdx.x, lane = threadIdx.x & (lanes - 1);
+    const int p = (int)((blockIdx.y * kBmThreads + threadIdx.x) / lanes);
+    double g = 0.0;
+    if (p < nparam)
         for (int it = csr_ptr[p]; it < csr_ptr[p + 1]; ++it) {
             const double *q = part + items[it] + (uint64_t)s * tiles;
-            for (uint32_t t = lane; t < tiles; t += 32) g += q[t];
+            for (uint32_t t = lane; t < tiles; t += lanes) g += q[t];
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
-        if (lane == 0) grad[param_off[gstate[s]] + p] = 2.0 * g;
-    }
+    for (int o = lanes >> 1; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+    if (p < nparam && lane == 0) grad[param_off[gstate[s]] + p] = 2.0 * g;
 }
 
 template <typename Real>
@@ -212,9 +243,9 @@ cudaError_t launch_bm_init(int dtype, void *psi, int n, int S, double *cs, int n
 cudaError_t launch_bm_mats(int dtype, const BatchMatPass *passes, int npasses, const BatchMatGate *gates, int S,
                            const double *cs, int nparam, void *mats, cudaStream_t st) {
     if (npasses == 0 || S == 0) return cudaSuccess;
-    const dim3 grid((unsigned)npasses, (unsigned)((S + 63) / 64));
-    if (dtype == QS_C64) k_bm_mats<float><<<grid, 64, 0, st>>>(passes, gates, S, cs, nparam, static_cast<float *>(mats));
-    else k_bm_mats<double><<<grid, 64, 0, st>>>(passes, gates, S, cs, nparam, static_cast<double *>(mats));
+    const dim3 grid((unsigned)npasses, (unsigned)std::min(32768, (S + kBmThreads / 32 - 1) / (kBmThreads / 32)));
+    if (dtype == QS_C64) k_bm_mats<float><<<grid, kBmThreads, 0, st>>>(passes, gates, S, cs, nparam, static_cast<float *>(mats));
+    else k_bm_mats<double><<<grid, kBmThreads, 0, st>>>(passes, gates, S, cs, nparam, static_cast<double *>(mats));
     return cudaGetLastError();
 }
 
@@ -227,7 +258,10 @@ cudaError_t launch_bm_obs(int dtype, const void *psi, void *lam, int n, int S, d
 cudaError_t launch_bm_grad(const double *part, const int *csr_ptr, const uint64_t *items, int nparam, int S,
                            uint32_t tiles, double *grad, const uint64_t *param_off, const int *gstate, cudaStream_t st) {
     if (nparam == 0) return cudaSuccess;
-    k_bm_grad<<<S, kBmThreads, 0, st>>>(part, csr_ptr, items, nparam, S, tiles, grad, param_off, gstate);
+    int lanes = 1;
+    while (lanes < 32 && (uint32_t)lanes < tiles) lanes *= 2;
+    const dim3 blocks((unsigned)S, (unsigned)(((uint64_t)nparam * lanes + kBmThreads - 1) / kBmThreads));
+    k_bm_grad<<<blocks, kBmThreads, 0, st>>>(part, csr_ptr, items, nparam, tiles, lanes, grad, param_off, gstate);
     return cudaGetLastError();
 }
 

@@ -128,21 +128,21 @@ __device__ __forceinline__ void pair_update(T2 &x, T2 &y, const Real *m) {
 
 // The update of one pair (one-sided: one amplitude) with the gate's matrix. complex64: float32
 // arithmetic. complex128: fixed point where the numbers allow it, float64 arithmetic otherwise
-// (k_fx.cuh); a pair of zeros needs neither.
-template <int OP, typename Idx>
-__device__ __forceinline__ void gate_pair(float2 &x, float2 &y, const DevGate<float, Idx> &g) {
+// (k_fx.cuh); a pair of zeros needs neither. G: a gate with its matrix m (and limbs fx).
+template <int OP, typename G>
+__device__ __forceinline__ void gate_pair(float2 &x, float2 &y, const G &g) {
     pair_update<OP == OP_GENW ? (int)OP_GEN : OP, float2, float>(x, y, g.m);
 }
-template <typename Idx>
-__device__ __forceinline__ void gate_side(float2 &x, const DevGate<float, Idx> &g) {
+template <typename G>
+__device__ __forceinline__ void gate_side(float2 &x, const G &g) {
     x = cmul<float2, float>(g.m[0], g.m[1], x);
 }
-template <typename Idx>
-__device__ __forceinline__ void gate_side(double2 &x, const DevGate<double, Idx> &g) {
+template <typename G>
+__device__ __forceinline__ void gate_side(double2 &x, const G &g) {
     if (!fx::mul<0>(x, g.fx) && (fx::nonzero(x.x) || fx::nonzero(x.y))) x = cmul<double2, double>(g.m[0], g.m[1], x);
 }
-template <int OP, typename Idx>
-__device__ __forceinline__ void gate_pair(double2 &x, double2 &y, const DevGate<double, Idx> &g) {
+template <int OP, typename G>
+__device__ __forceinline__ void gate_pair(double2 &x, double2 &y, const G &g) {
     if (OP == OP_SWAP) {
         pair_update<OP, double2, double>(x, y, g.m);
     } else if (OP == OP_GEN || OP == OP_GENW) {

@@ -401,6 +401,8 @@ static qs_status launch_program(qs_state *s, const FusedProgram &prog, const std
         if (op.drun >= 0) {
             const DiagRun &r = prog.druns[op.drun];
             e = launch_diag_run(s->dtype, s->psi, s->n, dgates + r.begin, r.count, r.nc, st);
+        } else if (op.pass >= 0 && prog.whole_count > 0) {
+            e = launch_whole(s->dtype, s->psi, s->n, table_whole(prog, dev_table), prog.whole_count, st);
         } else if (op.pass >= 0 && jit) {
             e = launch_jit_pass(s->dtype, (*jit)[op.pass], prog, op.pass, s->psi, lam, part, P, st);
         } else if (op.pass >= 0) {
@@ -584,7 +586,11 @@ std::vector<uint64_t> adj_signature(int dtype, const AdjPlan &ap) {
 }
 
 // The matrices of a program's gates from the current plans.
-void refresh_matrices(FusedProgram &prog, const std::vector<GatePlan> &plans) {
+void refresh_matrices(int dtype, FusedProgram &prog, const std::vector<GatePlan> &plans) {
+    if (prog.whole_count > 0) {
+        pack_whole(dtype, plans, &prog);
+        return;
+    }
     for (size_t gi = 0; gi < prog.gates.size(); ++gi) {
         RegGate &R = prog.gates[gi];
         const int src = prog.gate_src[gi];
@@ -940,12 +946,18 @@ qs_status qs_apply_circuit(qs_state *s, const qs_gate *gates, size_t count, cons
     const bool fuse = (flags & QS_FLAG_FUSE) != 0;
     FusedProgram prog;
     std::vector<JitPass> jit;
-    if (fuse) {
+    bool planned = false;
+    if (fuse && !(flags & QS_FLAG_JIT)) {  // one pass over the gates where it applies: nothing worth keeping
+        std::vector<int> seq(plans.size());
+        for (size_t i = 0; i < plans.size(); ++i) seq[i] = (int)i;
+        planned = plan_whole(s->n, s->dtype, tile_bits(s->dtype, false), seq, plans, &prog);
+    }
+    if (fuse && !planned) {
         std::vector<unsigned char> pkey = plan_cache_key('F', s, gates, count, n_theta, flags);
         std::vector<uint64_t> sig;
         plans_signature(s->dtype, plans, &sig);
         if (plan_cache_take(pkey, sig, &prog, nullptr, &jit, nullptr)) {
-            refresh_matrices(prog, plans);
+            refresh_matrices(s->dtype, prog, plans);
         } else {
             std::vector<int> seq(plans.size());  // after merging: fewer plans than records
             for (size_t i = 0; i < plans.size(); ++i) seq[i] = (int)i;
@@ -1069,8 +1081,8 @@ qs_status qs_adjoint_grad(qs_state *s, const qs_gate *gates, size_t count, const
         std::vector<unsigned char> key = plan_cache_key('A', s, gates, count, n_theta, flags);
         std::vector<uint64_t> sig = adj_signature(s->dtype, ap);
         if (plan_cache_take(key, sig, &pf, &pa, &jf, &ja)) {
-            refresh_matrices(pf, fwd);
-            refresh_matrices(pa, adj);
+            refresh_matrices(s->dtype, pf, fwd);
+            refresh_matrices(s->dtype, pa, adj);
         } else {
             plan_adjoint_programs(s, flags, &ap);
             if (use_jit) {

@@ -513,6 +513,8 @@ static void plan_in_order(int n, int dtype, int k, const std::vector<int> &seq, 
         prog->gate_src.clear();
         prog->druns.clear();
         prog->dgates.clear();
+        prog->whole.clear();
+        prog->whole_count = 0;
         prog->model_cost = 0.0;
     }
     max_gates = std::max(1, std::min(max_gates, kPassMaxGates));
@@ -757,6 +759,43 @@ static void plan_in_order(int n, int dtype, int k, const std::vector<int> &seq, 
     if (prog) emit_all(*sg);
 }
 
+void pack_whole(int dtype, const std::vector<GatePlan> &plans, FusedProgram *prog) {
+    const size_t each = whole_gate_bytes(dtype);
+    prog->whole.resize(each * prog->gate_src.size());
+    for (size_t i = 0; i < prog->gate_src.size(); ++i)
+        pack_whole_gate(dtype, plans[prog->gate_src[i]], prog->whole.data() + each * i);
+}
+
+// One pass over the whole state in the given order (the order does not change its cost). False: fewer
+// than two gates change anything, a launch of its own is better.
+bool plan_whole(int n, int dtype, int k, const std::vector<int> &seq, const std::vector<GatePlan> &plans,
+                FusedProgram *prog) {
+    if (dtype == QS_Q30) return false;
+    // a tile's size at most (complex128: one qubit more, its tiles hold half as many amplitudes)
+    if (n > std::min(dtype == QS_C64 ? k : k + 1, whole_bits(dtype))) return false;
+    std::vector<int> src;
+    double selected = 0.0;
+    for (int g : seq)
+        if (plans[g].units != 0) {
+            src.push_back(g);
+            selected += std::ldexp(plans[g].op == OP_SIDE ? 0.5 : 1.0, -popc(plans[g].ctrl_mask));
+        }
+    if (src.size() < 2 || (dtype == QS_C64 && n == kWholeBitsC64 && selected > 0.7 * (double)src.size())) return false;
+    *prog = FusedProgram{};
+    TilePass P;
+    make_pass(n, (1ull << n) - 1ull, &P);
+    P.gate_count = (int)src.size();
+    prog->passes.push_back(P);
+    prog->ops.push_back({0, -1});
+    prog->order = src;
+    prog->gate_src = std::move(src);
+    prog->whole_count = P.gate_count;
+    // a launch, the state read and written once, ~0.2 us a gate in one block
+    prog->model_cost = launch_latency_cost(n, dtype) * (1.0 + 0.1 * P.gate_count) + 1.0;
+    pack_whole(dtype, plans, prog);
+    return true;
+}
+
 bool plan_fused(int n, int dtype, int k, const std::vector<int> &seq, const std::vector<GatePlan> &plans,
                 const std::vector<int> *gslots, FusedProgram *prog, int max_gates, bool allow_single, int group_bits, bool jit) {
     // The gates in the given order and in the order block_schedule gives for passes of k local
@@ -764,6 +803,7 @@ bool plan_fused(int n, int dtype, int k, const std::vector<int> &seq, const std:
     // one of lower modelled cost is emitted.
     Segments s1;
     const int N = (int)seq.size();
+    if (!gslots && allow_single && !jit && plan_whole(n, dtype, k, seq, plans, prog)) return true;
     if (N < 3) {
         plan_in_order(n, dtype, k, seq, plans, gslots, prog, max_gates, allow_single, group_bits, jit, &s1);
         return true;
@@ -844,7 +884,7 @@ static double union_fraction(std::vector<std::pair<uint64_t, uint64_t>> terms, l
 
 double pass_touched_fraction(const FusedProgram &prog, int pass) {
     const TilePass &P = prog.passes[pass];
-    if (!P.hctrl) return 1.0;
+    if (!P.hctrl) return 1.0;  // (also a whole-state pass)
     std::vector<std::pair<uint64_t, uint64_t>> terms;
     for (int g = P.gate_begin; g < P.gate_begin + P.gate_count; ++g)
         terms.push_back({prog.gates[g].hmask, prog.gates[g].hvals});
@@ -858,10 +898,16 @@ static size_t dgate_offset(const FusedProgram &p) {
     return align16(p.groups.size() * sizeof(TileGroup)) + align16(p.gates.size() * sizeof(RegGate));
 }
 
-size_t program_table_bytes(const FusedProgram &p) { return dgate_offset(p) + p.dgates.size() * sizeof(DiagGate); }
+size_t program_table_bytes(const FusedProgram &p) {
+    return p.whole_count > 0 ? p.whole.size() : dgate_offset(p) + p.dgates.size() * sizeof(DiagGate);
+}
 
 void pack_program_table(const FusedProgram &p, void *host_dst) {
     char *d = static_cast<char *>(host_dst);
+    if (p.whole_count > 0) {
+        std::memcpy(d, p.whole.data(), p.whole.size());
+        return;
+    }
     if (!p.groups.empty()) std::memcpy(d, p.groups.data(), p.groups.size() * sizeof(TileGroup));
     if (!p.gates.empty())
         std::memcpy(d + align16(p.groups.size() * sizeof(TileGroup)), p.gates.data(), p.gates.size() * sizeof(RegGate));
@@ -871,6 +917,8 @@ void pack_program_table(const FusedProgram &p, void *host_dst) {
 const DiagGate *table_dgates(const FusedProgram &p, const void *dev_base) {
     return reinterpret_cast<const DiagGate *>(static_cast<const char *>(dev_base) + dgate_offset(p));
 }
+
+const void *table_whole(const FusedProgram &, const void *dev_base) { return dev_base; }
 
 const TileGroup *table_groups(const FusedProgram &, const void *dev_base) {
     return static_cast<const TileGroup *>(dev_base);

@@ -5,6 +5,7 @@
 
 #include "k_diag.cuh"
 #include "k_tile.cuh"
+#include "k_whole.cuh"
 
 namespace qs {
 
@@ -28,6 +29,10 @@ struct FusedProgram {
     std::vector<int> order;         // plan indices in the order the program applies them
     std::vector<DiagRun> druns;
     std::vector<DiagGate> dgates;   // all diagonal runs' gates
+    // The state fits one block's shared memory: the program is one pass whose gates (plan indices in
+    // gate_src, packed in `whole`) run one after another there (k_whole.cu); no groups, no RegGates.
+    int whole_count = 0;
+    std::vector<unsigned char> whole;
     double model_cost = 0.0;        // planner's cost estimate (units of one state read + write)
 };
 
@@ -48,6 +53,14 @@ void pack_program_table(const FusedProgram &p, void *host_dst);
 const TileGroup *table_groups(const FusedProgram &p, const void *dev_base);
 const RegGate *table_gates(const FusedProgram &p, const void *dev_base);
 const DiagGate *table_dgates(const FusedProgram &p, const void *dev_base);
+const void *table_whole(const FusedProgram &p, const void *dev_base);
+
+// Plans a forward program of interpreted passes with k-qubit tiles as one block's work where the state
+// fits (k_whole.cuh); false: not so (prog untouched).
+bool plan_whole(int n, int dtype, int k, const std::vector<int> &seq, const std::vector<GatePlan> &plans,
+                FusedProgram *prog);
+// Packs the gates of such a program from the current plans.
+void pack_whole(int dtype, const std::vector<GatePlan> &plans, FusedProgram *prog);
 
 // Plan the gates plans[seq[0]], plans[seq[1]], ... (the circuit's order; the program may apply
 // gates that commute in another order, see `order`). For the adjoint sweep, `gslots[g]` is the

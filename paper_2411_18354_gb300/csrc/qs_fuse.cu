@@ -7,8 +7,8 @@
 // launch of a gate costs the fraction of 64-byte DRAM units it touches; a pass costs the
 // fraction of tiles it touches (union bound over its gates' tile predicates) plus a per-gate
 // compute cost inside the tile (measured: about 0.15 for complex64, whose gates are
-// memory-bound; complex128 arithmetic gates are FP64-bound alone or in a pass, so there mostly
-// exchanges join passes). A run of diagonal gates can also go to one k_diag_run launch (up to
+// memory-bound; complex128 arithmetic gates run in fixed point alone and are FP64-bound in a pass,
+// so there mostly exchanges join passes). A run of diagonal gates can also go to one k_diag_run launch (up to
 // 64 gates; an uncontrolled gate just before the run can lead it), which costs one read +
 // write of the chunks the run can change. The gate sequence is cut into single launches,
 // passes and diagonal runs of least total modelled cost (dynamic programming over where each
@@ -43,7 +43,10 @@ double launch_latency_cost(int n, int dtype) {
 double single_launch_cost(const GatePlan &p, int dtype) {
     const int unit_bits = dtype == QS_C64 ? 3 : 2;
     const uint64_t high = p.ctrl_mask & ~((1ull << unit_bits) - 1ull);
-    return std::ldexp(1.0, -popc(high));
+    // a one-sided complex128 gate whose target is above the unit touches half (complex64 plans were
+    // measured without: diagonal gates rarely run alone there)
+    const double side = dtype == QS_C128 && p.op == OP_SIDE && p.t >= unit_bits ? 0.5 : 1.0;
+    return side * std::ldexp(1.0, -popc(high));
 }
 
 // A gate of a pass in local coordinates (before grouping).
@@ -470,9 +473,11 @@ static void make_pass(int n, uint64_t Lmask, TilePass *P) {
 // group's gather / scatter, diagonal about as much: the interpreter's per-gate work, not the
 // arithmetic, sets it), also for gates whose non-local controls select only some tiles;
 // 0.15 fits the measured plans best. complex128 gates are FP64-bound alone and inside a pass
-// alike (a general 2x2 costs ~3 units either way), so only exchanges (no arithmetic, ~0.33)
-// gain from a pass.
-static double pass_gate_cost(int dtype, const GatePlan &p, bool jit) {
+// (a general 2x2 costs ~3 units there; alone, in fixed point, one), so only exchanges (no
+// arithmetic, ~0.33) gain from a pass.
+// A pass with fewer tiles than SMs leaves the rest idle, and its FP64 work takes as many times longer
+// (13 qubits, 200 gates with 0-3 controls: planned into passes 875 us, apart 465).
+static double pass_gate_cost(int n, int dtype, int k, const GatePlan &p, bool jit) {
     if (dtype == QS_C64 && !jit) return 0.15;
     if (dtype == QS_C64) {
         // passes compiled for their shape (QS_FLAG_JIT), measured at n = 24 in units of one
@@ -482,12 +487,19 @@ static double pass_gate_cost(int dtype, const GatePlan &p, bool jit) {
         double c = p.op == OP_GEN ? 0.13 : p.op == OP_REAL ? 0.065 : p.op == OP_SWAP ? 0.04 : 0.035;
         return c * std::max(std::ldexp(1.0, -popc(p.ctrl_mask)), 0.125);
     }
-    return p.op == OP_SWAP ? 0.33 : 3.0;
+    return p.op == OP_SWAP ? 0.33 : 3.0 * std::max(1.0, 152.0 * std::ldexp(1.0, -std::max(0, n - k)));
 }
 
 // Compute cost of one diagonal gate inside a k_diag_run launch (its factor is formed once per
-// chunk of 8 amplitudes, or once per warp): small against the launch's state read + write.
-static double diag_run_gate_cost(int dtype) { return dtype == QS_C64 ? 0.005 : 0.02; }
+// chunk of 8 amplitudes, or once per warp): small against the launch's state read + write for
+// complex64. complex128 factors and products are FP64-bound there, while a phase alone runs in fixed
+// point at memory speed: QFT at n = 22, one run per qubit 3.18 ms (144 us each, 6.5 units), every gate
+// alone 1.98 ms.
+// (its blocks hold 2048 amplitudes: below 2^18 amplitudes SMs idle)
+static double diag_run_gate_cost(int n, int dtype) {
+    return dtype == QS_C64 ? 0.005 : 0.35 * std::max(1.0, 152.0 * std::ldexp(1.0, -std::max(0, n - 11)));
+}
+static double diag_run_lead_cost(int n, int dtype) { return dtype == QS_C64 ? 0.0 : 3.0 * diag_run_gate_cost(n, dtype); }
 
 enum { SEG_SINGLE, SEG_PASS, SEG_DIAG, SEG_LEAD_DIAG, SEG_NONE };
 
@@ -538,7 +550,7 @@ static void plan_in_order(int n, int dtype, int k, const std::vector<int> &seq, 
         tbit_of[j] = real ? (1ull << p.t) : 0ull;
         ctrl_of[j] = p.ctrl_mask;
         param_of[j] = param;
-        cost_of[j] = real ? pass_gate_cost(dtype, p, jit) * (param && jit ? 1.5 : 1.0) : 0.0;
+        cost_of[j] = real ? pass_gate_cost(n, dtype, k, p, jit) * (param && jit ? 1.5 : 1.0) : 0.0;
     }
     // Take gates seq[i], seq[i + 1], ... (before `end`) into one pass while its targets fit in
     // k local qubits and the gate and parameter limits allow; visit(j, frac, compute, real)
@@ -730,7 +742,7 @@ static void plan_in_order(int n, int dtype, int k, const std::vector<int> &seq, 
         if (diag_runs && p0.units != 0 && is_diag(g0)) {
             diag_span(j, N, false, [&](size_t e, double frac, int real) {
                 if (real < 2) return;
-                const double v = launch_cost + frac + real * diag_run_gate_cost(dtype) + best[e + 1];
+                const double v = launch_cost + frac + real * diag_run_gate_cost(n, dtype) + best[e + 1];
                 if (v < bv - 1e-9) {
                     bv = v;
                     bc = e + 1;
@@ -742,7 +754,7 @@ static void plan_in_order(int n, int dtype, int k, const std::vector<int> &seq, 
             !is_diag(g0) && j + 1 < N) {
             diag_span(j + 1, N, true, [&](size_t e, double frac, int real) {
                 if (real < 1) return;
-                const double v = launch_cost + frac + real * diag_run_gate_cost(dtype) + best[e + 1];
+                const double v = launch_cost + frac + diag_run_lead_cost(n, dtype) + real * diag_run_gate_cost(n, dtype) + best[e + 1];
                 if (v < bv - 1e-9) {
                     bv = v;
                     bc = e + 1;

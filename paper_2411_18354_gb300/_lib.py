@@ -32,6 +32,7 @@ _c_state_p = ctypes.c_void_p
 _u64 = ctypes.c_uint64
 _dp = ctypes.POINTER(ctypes.c_double)
 _vp = ctypes.c_void_p
+_C128 = np.dtype(np.complex128)
 
 # (name, restype, argtypes) for every function declared in include/qs.h
 _SIGNATURES = [
@@ -81,6 +82,7 @@ _SIGNATURES = [
 ]
 
 _lib = None
+_GATE_CALLS = {"qs_apply_gate": None, "qs_apply_gate_masked": None}
 
 
 def lib_path() -> str:
@@ -101,6 +103,12 @@ def lib():
             fn = getattr(L, name)
             fn.restype = res
             fn.argtypes = args
+        # the per-gate calls once more with plain addresses (no ctypes object per argument)
+        for name in _GATE_CALLS:
+            fn = L[name]
+            fn.restype = ctypes.c_int
+            fn.argtypes = [ctypes.c_void_p, ctypes.c_int, _u64, _u64, ctypes.c_void_p]
+            _GATE_CALLS[name] = fn
         _lib = L
     return _lib
 
@@ -202,9 +210,20 @@ def qs_state_synchronize(h: int) -> None:
     _check(lib().qs_state_synchronize(_c_state_p(h)))
 
 
+def _gate_call(name: str, h: int, target: int, ctrl_mask: int, ctrl_vals: int, U) -> None:
+    L = lib()
+    # a contiguous 2x2 complex128 array is the C layout already
+    if type(U) is np.ndarray and U.dtype is _C128 and U.size == 4 and U.flags.c_contiguous:
+        u = U
+    else:
+        u = _u8(U)
+    st = _GATE_CALLS[name](h, target, ctrl_mask, ctrl_vals, u.ctypes.data)
+    if st != QS_OK:
+        raise QsError(st, L.qs_last_error().decode(errors="replace"))
+
+
 def qs_apply_gate(h: int, target: int, ctrl_mask: int, ctrl_vals: int, U) -> None:
-    u = _u8(U)
-    _check(lib().qs_apply_gate(_c_state_p(h), target, ctrl_mask, ctrl_vals, u.ctypes.data_as(_dp)))
+    _gate_call("qs_apply_gate", h, target, ctrl_mask, ctrl_vals, U)
 
 
 def qs_apply_x(h: int, target: int, ctrl_mask: int = 0, ctrl_vals: int = 0) -> None:
@@ -212,8 +231,7 @@ def qs_apply_x(h: int, target: int, ctrl_mask: int = 0, ctrl_vals: int = 0) -> N
 
 
 def qs_apply_gate_masked(h: int, target: int, ctrl_mask: int, ctrl_vals: int, U) -> None:
-    u = _u8(U)
-    _check(lib().qs_apply_gate_masked(_c_state_p(h), target, ctrl_mask, ctrl_vals, u.ctypes.data_as(_dp)))
+    _gate_call("qs_apply_gate_masked", h, target, ctrl_mask, ctrl_vals, U)
 
 
 def _gates_arg(gates):

@@ -199,14 +199,12 @@ k_adj_step_zy(typename CxT<Real>::T *__restrict__ psi, typename CxT<Real>::T *__
     }
 }
 
-// lambda_k = (n - 2 popcount(k)) psi_k : O = sum_i Z_i is diagonal with that eigenvalue.
-template <typename Real>
-__global__ void k_obs_sumz(const typename CxT<Real>::T *__restrict__ psi, typename CxT<Real>::T *__restrict__ lam,
-                           int n, uint64_t N) {
+// lambda_k = (n - 2 popcount(k)) psi_k : O = sum_i Z_i is diagonal with that eigenvalue (complex128).
+__global__ void k_obs_sumz(const double2 *__restrict__ psi, double2 *__restrict__ lam, int n, uint64_t N) {
     const uint64_t step = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += step) {
-        const Real w = (Real)(n - 2 * __popcll(k));
-        typename CxT<Real>::T v = psi[k];
+        const double w = (double)(n - 2 * __popcll(k));
+        double2 v = psi[k];
         v.x *= w;
         v.y *= w;
         lam[k] = v;
@@ -221,34 +219,63 @@ __global__ void k_sum_vec(const double *__restrict__ z, int n, double *__restric
     }
 }
 
-// slot_sum[s] = sum over blocks of part[s][b] (fixed order).
-__global__ void k_slot_sums(const double *__restrict__ part, int nslots, double *__restrict__ slot_sum) {
-    // a warp per slot: lane l adds blocks l, l + 32, ... (coalesced), then a fixed-order
-    // shuffle reduction
-    const int s = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
-    if (s >= nslots) return;  // uniform over the warp
-    double v = 0.0;
-    for (int b = lane; b < kAdjMaxBlocks; b += 32) v += part[(size_t)s * kAdjMaxBlocks + b];
+// lambda = O psi as above and the energy's partial sums in the same read: part[b] = this block's sum of
+// (n - 2 popcount k) |psi_k|^2 (complex64: float32 over two amplitudes, a compensated running sum per
+// thread, float64 across threads). One launch and one read of psi instead of the <Z_i> reduction, its
+// final pass, their sum and lambda (complex128 keeps those: its reduction sums integers, k_reduce.cu).
+__global__ void __launch_bounds__(256) k_obs_energy(const float2 *__restrict__ psi, float2 *__restrict__ lam, int n,
+                                                    uint64_t N, double *__restrict__ part) {
+    Acc<float> acc{};
+    const uint64_t step = (uint64_t)gridDim.x * 256;
+    for (uint64_t j = (uint64_t)blockIdx.x * 256 + threadIdx.x; j < N / 2; j += step) {
+        float4 v = reinterpret_cast<const float4 *>(psi)[j];
+        const float w0 = (float)(n - 2 * __popcll(2 * j)), w1 = w0 - 2.f;
+        acc.add(fmaf(w0, fmaf(v.x, v.x, v.y * v.y), w1 * fmaf(v.z, v.z, v.w * v.w)));
+        v.x *= w0;
+        v.y *= w0;
+        v.z *= w1;
+        v.w *= w1;
+        reinterpret_cast<float4 *>(lam)[j] = v;
+    }
+    __shared__ double wsum[8];
+    double t = acc.value();
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) slot_sum[s] = v;
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = t;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double e = 0.0;
+        for (int w = 0; w < 8; ++w) e += wsum[w];
+        part[blockIdx.x] = e;
+    }
 }
 
-// grad[p] = 2 * sum of slot sums whose parameter is p: a warp per parameter, lane l looks at slots
-// l, l + 32, ..., then a fixed-order shuffle reduction (a thread per parameter walking all slots
-// took 55 us at 960 slots, 25 us at 320).
-__global__ void k_grad_gather(const double *__restrict__ slot_sum, const int *__restrict__ slot_param, int nslots,
-                              double *__restrict__ grad, int nparams) {
-    const int p = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+// grad[p] = 2 * sum over the slots whose parameter is p, and over their blocks, of part[s][b]: a warp
+// per parameter, lane l looking at slots l, l + 32, ... and adding blocks l, l + 32, ... of each hit,
+// then a fixed-order shuffle reduction. Warp nparams (energy != nullptr): the energy from slot row
+// nslots. (Slot sums, a thread per parameter walking all slots, and the energy's own kernels were
+// four launches; the walk alone took 55 us at 960 slots.)
+__global__ void __launch_bounds__(256) k_grad_final(const double *__restrict__ part, const int *__restrict__ slot_param,
+                                                    int nslots, double *__restrict__ grad, int nparams,
+                                                    double *__restrict__ energy) {
+    const int p = (int)((blockIdx.x * 256 + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
-    if (p >= nparams) return;  // uniform over the warp
+    if (p > nparams || (p == nparams && !energy)) return;  // uniform over the warp
     double v = 0.0;
-    for (int s = lane; s < nslots; s += 32)
-        if (slot_param[s] == p) v += slot_sum[s];
+    auto add_row = [&](int s) {
+        for (int b = lane; b < kAdjMaxBlocks; b += 32) v += part[(size_t)s * kAdjMaxBlocks + b];
+    };
+    if (p == nparams) {
+        add_row(nslots);
+    } else {
+        for (int s0 = 0; s0 < nslots; s0 += 32) {
+            unsigned hits = __ballot_sync(0xffffffffu, s0 + lane < nslots && slot_param[s0 + lane] == p);
+            for (; hits; hits &= hits - 1) add_row(s0 + __ffs(hits) - 1);
+        }
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) grad[p] = 2.0 * v;
+    if (lane == 0) (p == nparams ? *energy : grad[p]) = p == nparams ? v : 2.0 * v;
 }
 
 template <typename K>
@@ -385,13 +412,10 @@ cudaError_t launch_adj_step_zy(int dtype, void *psi, void *lam, const GatePlan &
                   : zy_by_shape<double, uint64_t>(psi, lam, z, y, part_z, part_y, st);
 }
 
-cudaError_t launch_obs_sumz(int dtype, const void *psi, void *lam, int n, cudaStream_t st) {
+cudaError_t launch_obs_sumz(const void *psi, void *lam, int n, cudaStream_t st) {
     const uint64_t N = 1ull << n;
     const unsigned grid = (unsigned)std::min<uint64_t>((N + 255) / 256, (uint64_t)device_sm_count() * 8);
-    if (dtype == QS_C64)
-        k_obs_sumz<float><<<grid, 256, 0, st>>>(reinterpret_cast<const float2 *>(psi), reinterpret_cast<float2 *>(lam), n, N);
-    else
-        k_obs_sumz<double><<<grid, 256, 0, st>>>(reinterpret_cast<const double2 *>(psi), reinterpret_cast<double2 *>(lam), n, N);
+    k_obs_sumz<<<grid, 256, 0, st>>>(static_cast<const double2 *>(psi), static_cast<double2 *>(lam), n, N);
     return cudaGetLastError();
 }
 
@@ -400,18 +424,23 @@ cudaError_t launch_sum_vec(const double *z, int n, double *out, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t launch_grad_final(const double *part, int nslots, double *slot_sum, const int *slot_param,
-                              double *grad, int nparams, cudaStream_t st) {
-    if (nslots > 0) {
-        k_slot_sums<<<(nslots + 7) / 8, 256, 0, st>>>(part, nslots, slot_sum);  // 8 slots (warps) per block
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    if (nparams > 0) {
-        k_grad_gather<<<(nparams + 7) / 8, 256, 0, st>>>(slot_sum, slot_param, nslots, grad, nparams);
-        return cudaGetLastError();
-    }
-    return cudaSuccess;
+// complex64, n >= 1: lambda = O psi and the energy's partial sums in part[0 .. adj_partials_per_slot())
+// (zeroed by the caller).
+cudaError_t launch_obs_energy(const void *psi, void *lam, int n, double *part, cudaStream_t st) {
+    const uint64_t N = 1ull << n;
+    const unsigned grid = (unsigned)std::max<uint64_t>(
+        1, std::min<uint64_t>({(N / 2 + 255) / 256, (uint64_t)device_sm_count() * 6, (uint64_t)kAdjMaxBlocks}));
+    k_obs_energy<<<grid, 256, 0, st>>>(static_cast<const float2 *>(psi), static_cast<float2 *>(lam), n, N, part);
+    return cudaGetLastError();
+}
+
+// energy (may be null): written from the partial sums in row nslots of part.
+cudaError_t launch_grad_final(const double *part, int nslots, const int *slot_param, double *grad, int nparams,
+                              double *energy, cudaStream_t st) {
+    if (nparams == 0 && !energy) return cudaSuccess;
+    const uint64_t warps = (uint64_t)nparams + 1;
+    k_grad_final<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(part, slot_param, nslots, grad, nparams, energy);
+    return cudaGetLastError();
 }
 
 }  // namespace qs

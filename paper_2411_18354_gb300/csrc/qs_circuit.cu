@@ -24,10 +24,11 @@ cudaError_t launch_adj_step(int dtype, void *psi, void *lam, const GatePlan &p, 
 bool adj_steps_join(const GatePlan &z, const GatePlan &y);
 cudaError_t launch_adj_step_zy(int dtype, void *psi, void *lam, const GatePlan &z, const GatePlan &y, double *part_z,
                                double *part_y, cudaStream_t st);
-cudaError_t launch_obs_sumz(int dtype, const void *psi, void *lam, int n, cudaStream_t st);
+cudaError_t launch_obs_sumz(const void *psi, void *lam, int n, cudaStream_t st);
 cudaError_t launch_sum_vec(const double *z, int n, double *out, cudaStream_t st);
-cudaError_t launch_grad_final(const double *part, int nslots, double *slot_sum, const int *slot_param,
-                              double *grad, int nparams, cudaStream_t st);
+cudaError_t launch_obs_energy(const void *psi, void *lam, int n, double *part, cudaStream_t st);
+cudaError_t launch_grad_final(const double *part, int nslots, const int *slot_param, double *grad, int nparams,
+                              double *energy, cudaStream_t st);
 
 void release_state_buffers(qs_state *s) {
     for (auto &g : s->graphs) {
@@ -976,7 +977,8 @@ qs_status qs_apply_circuit(qs_state *s, const qs_gate *gates, size_t count, cons
         if (e != cudaSuccess) return cuda_fail(e, "qs_apply_circuit: loading compiled passes");
     }
     const std::vector<JitPass> *jp = (flags & QS_FLAG_JIT) ? &jit : nullptr;
-    const size_t table_bytes = fuse ? program_table_bytes(prog) : 0;
+    // (compiled passes hold everything in their parameters; only diagonal runs read a table then)
+    const size_t table_bytes = fuse && !(jp && prog.druns.empty()) ? program_table_bytes(prog) : 0;
     std::vector<char> table_host(table_bytes);
     if (table_bytes) pack_program_table(prog, table_host.data());
 
@@ -1095,7 +1097,7 @@ qs_status qs_adjoint_grad(qs_state *s, const qs_gate *gates, size_t count, const
         }
     }
 
-    // Buffers: lambda, partials [nslots][P], slot sums, slot->param map, outputs.
+    // Buffers: lambda, partials [nslots + 1][P] (the last row the energy's), slot->param map, outputs.
     cudaError_t e;
     if (!s->lam) {
         e = cudaMalloc(&s->lam, s->bytes);
@@ -1106,7 +1108,8 @@ qs_status qs_adjoint_grad(qs_state *s, const qs_gate *gates, size_t count, const
         }
     }
     const size_t P = adj_partials_per_slot();
-    const size_t need = (size_t)nslots * P + (size_t)nslots + (size_t)nslots + n_theta + 64 + 8;
+    const size_t rows = (size_t)nslots + 1;
+    const size_t need = rows * P + (size_t)nslots + n_theta + 64 + 8;
     if (s->grad_scratch_n < need) {
         if (s->grad_scratch) cudaFree(s->grad_scratch);
         s->grad_scratch = nullptr;
@@ -1122,16 +1125,16 @@ qs_status qs_adjoint_grad(qs_state *s, const qs_gate *gates, size_t count, const
     qs_status st = ensure_reduce_scratch(s);
     if (st != QS_OK) return st;
     double *part = s->grad_scratch;
-    double *slot_sum = part + (size_t)nslots * P;
-    int *slot_param_dev = reinterpret_cast<int *>(slot_sum + nslots);  // nslots ints fit in nslots doubles
-    double *grad_dev = slot_sum + 2 * (size_t)nslots;
+    int *slot_param_dev = reinterpret_cast<int *>(part + rows * P);  // nslots ints fit in nslots doubles
+    double *grad_dev = part + rows * P + (size_t)nslots;
     double *energy_dev = grad_dev + n_theta;
     cudaStream_t stm = s->stream;
 
     // Tables of the fused forward and sweep programs (one upload, stream-ordered).
     const size_t bf = fuse ? (program_table_bytes(pf) + 255) & ~size_t(255) : 0;
     const size_t ba = fuse ? program_table_bytes(pa) : 0;
-    if (fuse && bf + ba > 0) {
+    // (compiled passes hold everything in their parameters; only diagonal runs read a table then)
+    if (fuse && bf + ba > 0 && !(use_jit && pf.druns.empty() && pa.druns.empty())) {
         st = ensure_device(&s->tile_table, &s->tile_table_bytes, bf + ba, stm,
                            "qs_adjoint_grad: cannot allocate the fused gate table");
         if (st != QS_OK) return st;
@@ -1148,12 +1151,16 @@ qs_status qs_adjoint_grad(qs_state *s, const qs_gate *gates, size_t count, const
               : launch_plans(s, fwd, stm);
     if (st != QS_OK) return st;
     // Energy and lambda = O psi.
-    double *z = s->red_scratch;
-    e = launch_expect_z(s->dtype, s->psi, s->n, s->red_scratch + 64, z, nullptr, stm);
-    if (e == cudaSuccess) e = launch_sum_vec(z, s->n, (on_dev && energy) ? energy : energy_dev, stm);
-    if (e == cudaSuccess) e = launch_obs_sumz(s->dtype, s->psi, s->lam, s->n, stm);
-    if (e == cudaSuccess && nslots > 0)
-        e = cudaMemsetAsync(part, 0, (size_t)nslots * P * sizeof(double), stm);
+    double *energy_to = (on_dev && energy) ? energy : energy_dev;
+    e = cudaMemsetAsync(part, 0, rows * P * sizeof(double), stm);
+    if (s->dtype == QS_C64) {
+        if (e == cudaSuccess) e = launch_obs_energy(s->psi, s->lam, s->n, part + (size_t)nslots * P, stm);
+    } else {
+        double *z = s->red_scratch;
+        if (e == cudaSuccess) e = launch_expect_z(s->dtype, s->psi, s->n, s->red_scratch + 64, z, nullptr, stm);
+        if (e == cudaSuccess) e = launch_sum_vec(z, s->n, energy_to, stm);
+        if (e == cudaSuccess) e = launch_obs_sumz(s->psi, s->lam, s->n, stm);
+    }
     if (e == cudaSuccess && nslots > 0)
         e = cudaMemcpyAsync(slot_param_dev, slot_param.data(), nslots * sizeof(int), cudaMemcpyHostToDevice, stm);
     if (e != cudaSuccess) return cuda_fail(e, "qs_adjoint_grad setup");
@@ -1175,7 +1182,8 @@ qs_status qs_adjoint_grad(qs_state *s, const qs_gate *gates, size_t count, const
             if (e != cudaSuccess) return cuda_fail(e, "qs_adjoint_grad sweep launch");
         }
     }
-    e = launch_grad_final(part, nslots, slot_sum, slot_param_dev, on_dev ? grad : grad_dev, (int)n_theta, stm);
+    e = launch_grad_final(part, nslots, slot_param_dev, on_dev ? grad : grad_dev, (int)n_theta,
+                          s->dtype == QS_C64 ? energy_to : nullptr, stm);
     if (e != cudaSuccess) return cuda_fail(e, "qs_adjoint_grad final");
     if (!on_dev) {
         if (n_theta > 0) e = cudaMemcpyAsync(grad, grad_dev, n_theta * sizeof(double), cudaMemcpyDeviceToHost, stm);

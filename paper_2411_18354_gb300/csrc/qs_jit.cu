@@ -164,7 +164,6 @@ void preamble(Out &o, bool dbl) {
         "\"l\"(g) : \"memory\");\n}\n");
     o.f("__device__ __forceinline__ void cpcommit() { asm volatile(\"cp.async.commit_group;\\n\" ::: \"memory\"); }\n");
     o.f("__device__ __forceinline__ void cpwait0() { asm volatile(\"cp.async.wait_group 0;\\n\" ::: \"memory\"); }\n");
-    o.f("__device__ __forceinline__ void cpwait1() { asm volatile(\"cp.async.wait_group 1;\\n\" ::: \"memory\"); }\n");
 }
 
 // Expression of the tile swizzle of `a` (the same bijection as tile_swizzle, k_tile.cuh).
@@ -620,14 +619,17 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
     if (adjoint) o.f("    T2 *tl = tp + %u;\n", TILE);
     if (pm_state > 0) o.f("    const R *const pm_ = sr_ + %s * %d;\n", db ? "cur" : "0", pm_state);
     if (db) {
+        // one barrier: this tile has arrived, and every thread is done with the one before, whose
+        // buffer the next tile's copy takes
+        o.f("    cpwait0();\n    __syncthreads();\n");
         o.f("    if (nxt < ntiles) {\n      const u64 nb = tile_base(nxt);\n      T2 *tn = sm0 + (cur ^ 1) * %u;\n", BUF);
         loads("tn", "nb", "nxt", "cur ^ 1");
-        o.f("      cpwait1();\n    } else {\n      cpwait0();\n    }\n");
+        o.f("    }\n");
     } else {
         loads("tp", "base", "tau", "0");
-        o.f("    cpwait0();\n");
+        o.f("    cpwait0();\n    __syncthreads();\n");
     }
-    o.f("    __syncthreads();\n");
+    const bool end_sync = !db || (adjoint && batched && NP > 0);  // a barrier after the tile's last access
 
     bool stored = false;
     for (int gi_ = 0; gi_ < P.group_count; ++gi_) {
@@ -792,7 +794,7 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
             }
             o.f("      }\n    }\n");
         }
-        o.f("    }\n    __syncthreads();\n");
+        o.f("    }\n%s", stored && !end_sync ? "" : "    __syncthreads();\n");
     }
     if (!stored) {
         o.f("    {\n    T2 *gp_ = gvec(psi, tau);\n");
@@ -801,7 +803,7 @@ std::string jit_pass_source(int dtype, bool adjoint, const TilePass &P, const Ti
             o.f("    T2 *gl_ = gvec(lam, tau);\n");
             copies(false, "gl_", "tl", "base");
         }
-        o.f("    }\n    __syncthreads();\n");
+        o.f("    }\n%s", end_sync ? "    __syncthreads();\n" : "");
     }
     if (adjoint && batched && NP > 0) {
         // this tile's gradient partials (sum over the block's warps), then fresh accumulators;

@@ -283,6 +283,10 @@ __device__ __forceinline__ bool mul(double2 &x, const FxMat &f) {
     return true;
 }
 
+// Keeps the float64 form behind its branch (the compiler may otherwise compute a short one for every
+// pair and select).
+__device__ __forceinline__ void rare(double &v) { asm volatile("" : "+d"(v)); }
+
 __device__ __forceinline__ bool nonzero(double v) { return (__double2hiint(v) | __double2loint(v)) != 0; }
 
 }  // namespace fx

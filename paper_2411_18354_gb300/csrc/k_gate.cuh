@@ -52,13 +52,37 @@ template <> struct Vec<float, 4> {
         Vec<float, 2>::st(p + 2, v + 2);
     }
 };
+// Four complex64 amplitudes as one 32-byte access: the two sides of two pairs of target 1.
+__device__ __forceinline__ void ld_quad(const float2 *p, float2 *x, float2 *y) {
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(x[0].x), "=f"(x[0].y), "=f"(x[1].x), "=f"(x[1].y), "=f"(y[0].x), "=f"(y[0].y), "=f"(y[1].x),
+                   "=f"(y[1].y)
+                 : "l"(p)
+                 : "memory");
+}
+__device__ __forceinline__ void st_quad(float2 *p, const float2 *x, const float2 *y) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(x[0].x), "f"(x[0].y),
+                 "f"(x[1].x), "f"(x[1].y), "f"(y[0].x), "f"(y[0].y), "f"(y[1].x), "f"(y[1].y)
+                 : "memory");
+}
 template <> struct Vec<double, 1> {
     __device__ __forceinline__ static void ld(const double2 *p, double2 *v) { v[0] = *p; }
     __device__ __forceinline__ static void st(double2 *p, const double2 *v) { *p = v[0]; }
 };
+// An adjacent pair of complex128 amplitudes: one 32-byte access (two of 16 bytes left every warp
+// instruction touching every other 16 bytes of 1 KB).
 template <> struct Vec<double, 2> {
-    __device__ __forceinline__ static void ld(const double2 *p, double2 *v) { v[0] = p[0]; v[1] = p[1]; }
-    __device__ __forceinline__ static void st(double2 *p, const double2 *v) { p[0] = v[0]; p[1] = v[1]; }
+    __device__ __forceinline__ static void ld(const double2 *p, double2 *v) {
+        asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+                     : "=d"(v[0].x), "=d"(v[0].y), "=d"(v[1].x), "=d"(v[1].y)
+                     : "l"(p)
+                     : "memory");
+    }
+    __device__ __forceinline__ static void st(double2 *p, const double2 *v) {
+        asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0].x), "d"(v[0].y), "d"(v[1].x),
+                     "d"(v[1].y)
+                     : "memory");
+    }
 };
 
 // Device copy of a gate: index map in the index width, matrix in the state's precision
@@ -139,7 +163,19 @@ __device__ __forceinline__ void gate_side(float2 &x, const G &g) {
 }
 template <typename G>
 __device__ __forceinline__ void gate_side(double2 &x, const G &g) {
-    if (!fx::mul<0>(x, g.fx) && (fx::nonzero(x.x) || fx::nonzero(x.y))) x = cmul<double2, double>(g.m[0], g.m[1], x);
+    if (!fx::mul<0>(x, g.fx) && (fx::nonzero(x.x) || fx::nonzero(x.y))) {
+        fx::rare(x.x);
+        x = cmul<double2, double>(g.m[0], g.m[1], x);
+    }
+}
+template <typename G>
+__device__ __forceinline__ void gate_real(double &x, double &y, const G &g) {
+    if (!fx::real(x, y, g.fx) && (fx::nonzero(x) || fx::nonzero(y))) {
+        fx::rare(x);
+        const double nx = fma(g.m[0], x, g.m[2] * y);
+        y = fma(g.m[4], x, g.m[6] * y);
+        x = nx;
+    }
 }
 template <int OP, typename G>
 __device__ __forceinline__ void gate_pair(double2 &x, double2 &y, const G &g) {
@@ -147,22 +183,19 @@ __device__ __forceinline__ void gate_pair(double2 &x, double2 &y, const G &g) {
         pair_update<OP, double2, double>(x, y, g.m);
     } else if (OP == OP_GEN || OP == OP_GENW) {
         if (!(OP == OP_GEN ? fx::gen(x, y, g.fx) : fx::genw(x, y, g.fx)) &&
-            (fx::nonzero(x.x) || fx::nonzero(x.y) || fx::nonzero(y.x) || fx::nonzero(y.y)))
+            (fx::nonzero(x.x) || fx::nonzero(x.y) || fx::nonzero(y.x) || fx::nonzero(y.y))) {
+            fx::rare(x.x);
             pair_update<OP_GEN, double2, double>(x, y, g.m);
+        }
     } else if (OP == OP_REAL) {
-        if (!fx::real(x.x, y.x, g.fx) && (fx::nonzero(x.x) || fx::nonzero(y.x))) {
-            const double nx = fma(g.m[0], x.x, g.m[2] * y.x);
-            y.x = fma(g.m[4], x.x, g.m[6] * y.x);
-            x.x = nx;
-        }
-        if (!fx::real(x.y, y.y, g.fx) && (fx::nonzero(x.y) || fx::nonzero(y.y))) {
-            const double nx = fma(g.m[0], x.y, g.m[2] * y.y);
-            y.y = fma(g.m[4], x.y, g.m[6] * y.y);
-            x.y = nx;
-        }
+        gate_real(x.x, y.x, g);
+        gate_real(x.y, y.y, g);
     } else if (OP == OP_DIAG) {
-        if (!fx::mul<0>(x, g.fx) && (fx::nonzero(x.x) || fx::nonzero(x.y))) x = cmul<double2, double>(g.m[0], g.m[1], x);
-        if (!fx::mul<3>(y, g.fx) && (fx::nonzero(y.x) || fx::nonzero(y.y))) y = cmul<double2, double>(g.m[6], g.m[7], y);
+        gate_side(x, g);
+        if (!fx::mul<3>(y, g.fx) && (fx::nonzero(y.x) || fx::nonzero(y.y))) {
+            fx::rare(y.x);
+            y = cmul<double2, double>(g.m[6], g.m[7], y);
+        }
     }
 }
 // Masked comparator: the class of the matrix is read at run time, so that it runs the arithmetic
@@ -222,6 +255,9 @@ k_gate(typename CxT<Real>::T *__restrict__ psi, const DevGate<Real, Idx> g, Idx 
     using T2 = typename CxT<Real>::T;
     constexpr int r = Log2<R>::v;
     constexpr int A = (LAY == LAY_ADJ) ? 2 * R : R;  // amplitudes per load group
+    // complex64, target 1: a unit's two vectors are 32 contiguous bytes (as two accesses each warp
+    // instruction touches every other 16 bytes of 1 KB: n = 29 1.43 ms, as one 1.34)
+    constexpr bool QUAD = sizeof(Real) == 4 && LAY == LAY_SPLIT && R == 2 && OP != OP_SIDE && !MASKED;
     // When launched as a programmatic dependent of the previous kernel on the stream, this block
     // may start while that kernel drains: the state is touched only after it has completed and
     // its writes are visible (grid dependency barrier; immediate for a normal launch). The next
@@ -253,11 +289,20 @@ k_gate(typename CxT<Real>::T *__restrict__ psi, const DevGate<Real, Idx> g, Idx 
                 } else if (OP == OP_SIDE) {
                     Vec<Real, R>::ld(psi + (lo[k] | (side ? g.tbit : (Idx)0)), x[k]);
                 } else {
+                    if constexpr (QUAD) {
+                        if (g.tbit == 2) {  // uniform
+                            ld_quad(psi + lo[k], x[k], y[k]);
+                            continue;
+                        }
+                    }
                     Vec<Real, R>::ld(psi + lo[k], x[k]);
                     Vec<Real, R>::ld(psi + (lo[k] | g.tbit), y[k]);
                 }
             }
         }
+        // every load before the first branch or store: the compiler otherwise sinks some below the
+        // arithmetic of the others (complex128 diagonal, n = 28: 1.99 ms, with all loads first 1.39)
+        asm volatile("" ::: "memory");
 #pragma unroll
         for (int k = 0; k < UNR; ++k) {
             if (!on[k]) continue;
@@ -279,6 +324,13 @@ k_gate(typename CxT<Real>::T *__restrict__ psi, const DevGate<Real, Idx> g, Idx 
                 for (int i = 0; i < R; ++i) {
                     if (MASKED) gate_pair_any(x[k][i], y[k][i], g, side);
                     else gate_pair<OP>(x[k][i], y[k][i], g);
+                }
+                if constexpr (QUAD) {
+                    if (g.tbit == 2) {
+                        st_quad(psi + lo[k], x[k], y[k]);
+                        QS_DBG_WRITE(lo[k], 4);
+                        continue;
+                    }
                 }
                 Vec<Real, R>::st(psi + lo[k], x[k]);
                 Vec<Real, R>::st(psi + (lo[k] | g.tbit), y[k]);

@@ -300,9 +300,10 @@ k_gate(typename CxT<Real>::T *__restrict__ psi, const DevGate<Real, Idx> g, Idx 
                 }
             }
         }
-        // every load before the first branch or store: the compiler otherwise sinks some below the
-        // arithmetic of the others (complex128 diagonal, n = 28: 1.99 ms, with all loads first 1.39)
-        asm volatile("" ::: "memory");
+        // complex128: every load before the first branch or store; the compiler otherwise sinks some
+        // below the arithmetic of the others (diagonal, n = 28: 1.99 ms, with all loads first 1.39).
+        // complex64 gains nothing from it and keeps the compiler's order.
+        if constexpr (sizeof(Real) == 8) asm volatile("" ::: "memory");
 #pragma unroll
         for (int k = 0; k < UNR; ++k) {
             if (!on[k]) continue;

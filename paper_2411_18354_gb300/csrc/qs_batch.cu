@@ -8,12 +8,14 @@
 // their matrices from theta. Tuning (small_bits, tile_bits, max_pass_gates) comes from the
 // caller, normally the autotuner; 0 selects the library defaults.
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 #include <cstring>
 #include <new>
 #include <map>
 #include <numeric>
 #include <string>
+#include <thread>
 #include <utility>
 #include <vector>
 
@@ -43,7 +45,6 @@ struct BatchJitProg {
     int n = 0, nparam = 0;
     std::vector<int> states;        // global state indices
     std::vector<qs_gate> gates;     // of each state, until its programs are planned
-    bool planned = false;
     qs::FusedProgram pf, pa;        // forward and sweep programs (rotation kinds / indices filled in)
     std::vector<qs::JitPass> jf, ja;
     void *psi = nullptr, *lam = nullptr;
@@ -169,14 +170,11 @@ bool plan_pair(int n, int dtype, const qs_gate &g, int nparam, GatePlan *fwd, Ga
     return true;
 }
 
-// Compile the pass-major path's kernels and allocate its buffers (first QS_FLAG_JIT run).
-// The pass-major path's programs of one gate list: every rotation its own gate (a compiled pass applies
-// RY in 2 and a one-sided phase in 4 multiply-adds per output pair, a merged RZ RY in 16), and
-// uncontrolled RZ(theta) = e^{-i theta / 2} diag(1, e^{i theta}) one-sided: the global phase changes
-// neither the energy nor a derivative (plan_adjoint_gates). Planned when first needed: a batch that
-// only runs in the persistent kernel does not pay for it.
-void plan_major(const qs_batch *b, BatchJitProg &jp) {
-    if (jp.planned) return;
+// The pass-major path's forward (dir 0) or sweep (dir 1) program of one gate list: every rotation its
+// own gate (a compiled pass applies RY in 2 and a one-sided phase in 4 multiply-adds per output pair, a
+// merged RZ RY in 16), and uncontrolled RZ(theta) = e^{-i theta / 2} diag(1, e^{i theta}) one-sided: the
+// global phase changes neither the energy nor a derivative (plan_adjoint_gates).
+void plan_major(const qs_batch *b, BatchJitProg &jp, int dir) {
     const int n = jp.n, dtype = b->dtype;
     const std::vector<qs_gate> &gs = jp.gates;
     const size_t gc = gs.size();
@@ -187,40 +185,78 @@ void plan_major(const qs_batch *b, BatchJitProg &jp) {
         plan_pair(n, dtype, gs[i], jp.nparam, &fwd[i], &adj[i], err, sizeof(err));
         if (gs[i].kind == QS_GATE_RY || gs[i].kind == QS_GATE_RZ) slots[i] = gs[i].param;
     }
+    std::vector<GatePlan> &plans = dir ? adj : fwd;
     for (size_t i = 0; i < gc; ++i) {
         if (gs[i].kind != QS_GATE_RZ || gs[i].ctrl_mask != 0) continue;
         static const double kPhase[8] = {1.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.6, 0.8};  // structure only
-        for (GatePlan *p : {&fwd[i], &adj[i]}) {
-            GatePlan q;
-            if (!plan_gate(n, dtype, gs[i].target, 0, 0, kPhase, QS_GATE_U, OP_SIDE, &q, err, sizeof(err))) continue;
-            q.side = 1;
-            *p = q;
-        }
+        GatePlan q;
+        if (!plan_gate(n, dtype, gs[i].target, 0, 0, kPhase, QS_GATE_U, OP_SIDE, &q, err, sizeof(err))) continue;
+        q.side = 1;
+        plans[i] = q;
     }
     std::vector<int> seq(gc);
     std::iota(seq.begin(), seq.end(), 0);
-    plan_fused(n, dtype, std::min(b->major_f, n), seq, fwd, nullptr, &jp.pf, b->major_gates, false, kGroupBits, true);
-    std::reverse(seq.begin(), seq.end());
-    plan_fused(n, dtype, std::min(b->major_a, n), seq, adj, &slots, &jp.pa, b->major_gates, false, kGroupBitsAdjoint, true);
-    for (FusedProgram *p : {&jp.pf, &jp.pa})
-        for (size_t i = 0; i < p->gates.size(); ++i) {
-            RegGate &G = p->gates[i];
-            const qs_gate &src = gs[p->gate_src[i]];
-            const bool rot = src.kind == QS_GATE_RY || src.kind == QS_GATE_RZ;
-            G.pkind = rot ? src.kind : 0;
-            G.pidx = rot ? src.param : 0;
-            G.slot = rot && p == &jp.pa ? src.param : -1;
-        }
-    jp.gates = {};
-    jp.planned = true;
+    if (dir) std::reverse(seq.begin(), seq.end());
+    FusedProgram &prog = dir ? jp.pa : jp.pf;
+    plan_fused(n, dtype, std::min(dir ? b->major_a : b->major_f, n), seq, plans, dir ? &slots : nullptr, &prog, b->major_gates, false,
+               dir ? kGroupBitsAdjoint : kGroupBits, true);
+    for (size_t i = 0; i < prog.gates.size(); ++i) {
+        RegGate &G = prog.gates[i];
+        const qs_gate &src = gs[prog.gate_src[i]];
+        const bool rot = src.kind == QS_GATE_RY || src.kind == QS_GATE_RZ;
+        G.pkind = rot ? src.kind : 0;
+        G.pidx = rot ? src.param : 0;
+        G.slot = rot && dir ? src.param : -1;
+    }
 }
 
+// Plans every program of a batch on threads of their own, a program's two directions apart, while
+// qs_batch_create uploads the persistent kernel's tables (64 states of 13-15 qubits, 6 layers: create and first run 2.7 ms;
+// planned in the first run, on one thread per direction, 2.9).
+class MajorPlanner {
+  public:
+    explicit MajorPlanner(qs_batch *b) : b_(b), count_(2 * b->jprogs.size()) {
+        const size_t threads = std::min<size_t>(std::max(1u, std::thread::hardware_concurrency()), count_);
+        try {
+            th_.reserve(threads);
+            for (size_t w = 0; w < threads; ++w) th_.emplace_back([this] { work(); });
+        } catch (const std::exception &) {  // no more threads to be had: finish() does the rest
+        }
+    }
+    ~MajorPlanner() { join(); }
+    // Every program is planned on return (false: out of host memory).
+    bool finish() {
+        work();
+        join();
+        for (BatchJitProg &jp : b_->jprogs) jp.gates = {};
+        return !failed_;
+    }
+    void join() {
+        for (std::thread &t : th_) t.join();
+        th_.clear();
+    }
+
+  private:
+    void work() {
+        try {
+            for (size_t q; (q = next_.fetch_add(1)) < count_;) plan_major(b_, b_->jprogs[q / 2], (int)(q & 1));
+        } catch (const std::exception &) {
+            failed_ = true;
+        }
+    }
+    qs_batch *b_;
+    size_t count_;
+    std::atomic<size_t> next_{0};
+    std::atomic<bool> failed_{false};
+    std::vector<std::thread> th_;
+};
+
+// Compile the pass-major path's kernels and allocate its buffers (first QS_FLAG_JIT run).
 qs_status ensure_jit(qs_batch *b) {
     if (b->jit_ready) return QS_OK;
     const size_t es = elem_bytes(b->dtype), rs = es / 2;
     std::vector<JitRequest> reqs;
     for (BatchJitProg &jp : b->jprogs) {
-        plan_major(b, jp);
         reqs.push_back({&jp.pf, false, true, &jp.jf});
         reqs.push_back({&jp.pa, true, true, &jp.ja});
     }
@@ -553,30 +589,6 @@ qs_status qs_batch_create(int num_states, const int *n_qubits, const qs_gate *ga
     b->major_f = major_f;
     b->major_a = major_a;
     b->major_gates = major_gates;
-    qs_status st;
-    if ((st = upload(states, &b->d_states)) != QS_OK || (st = upload(order, &b->d_order)) != QS_OK ||
-        (st = upload(progs, &b->d_progs)) != QS_OK || (st = upload(passes, &b->d_passes)) != QS_OK ||
-        (st = upload(tgates, &b->d_gates)) != QS_OK || (st = upload(tgroups, &b->d_groups)) != QS_OK) {
-        free_batch(b);
-        return st;
-    }
-    const uint64_t ws_stride = max_large_n > 0 ? (1ull << max_large_n) : 0;
-    if (ws_stride) {
-        const size_t bytes = (size_t)grid * 2 * ws_stride * es;
-        cudaError_t e = cudaMalloc(&b->workspace, bytes);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            b->workspace = nullptr;
-            free_batch(b);
-            return set_error(QS_ENOMEM, "qs_batch_create: cannot allocate the large-state workspace");
-        }
-    }
-    if (cudaMalloc(&b->queue, sizeof(int)) != cudaSuccess) {
-        cudaGetLastError();
-        b->queue = nullptr;
-        free_batch(b);
-        return set_error(QS_ENOMEM, "qs_batch_create: cannot allocate the work queue");
-    }
     // the pass-major path's programs (states above small_bits), compiled on first use
     {
         std::vector<int> jp_of(progs.size(), -1);
@@ -599,6 +611,33 @@ qs_status qs_batch_create(int num_states, const int *n_qubits, const qs_gate *ga
         }
         b->param_off_host.assign(param_offsets, param_offsets + num_states + 1);
     }
+    MajorPlanner planner(b);
+    auto fail = [&](qs_status st, const char *what) {
+        planner.join();
+        free_batch(b);
+        return what ? set_error(st, what) : st;
+    };
+    qs_status st;
+    if ((st = upload(states, &b->d_states)) != QS_OK || (st = upload(order, &b->d_order)) != QS_OK ||
+        (st = upload(progs, &b->d_progs)) != QS_OK || (st = upload(passes, &b->d_passes)) != QS_OK ||
+        (st = upload(tgates, &b->d_gates)) != QS_OK || (st = upload(tgroups, &b->d_groups)) != QS_OK)
+        return fail(st, nullptr);
+    const uint64_t ws_stride = max_large_n > 0 ? (1ull << max_large_n) : 0;
+    if (ws_stride) {
+        const size_t bytes = (size_t)grid * 2 * ws_stride * es;
+        cudaError_t e = cudaMalloc(&b->workspace, bytes);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            b->workspace = nullptr;
+            return fail(QS_ENOMEM, "qs_batch_create: cannot allocate the large-state workspace");
+        }
+    }
+    if (cudaMalloc(&b->queue, sizeof(int)) != cudaSuccess) {
+        cudaGetLastError();
+        b->queue = nullptr;
+        return fail(QS_ENOMEM, "qs_batch_create: cannot allocate the work queue");
+    }
+    if (!planner.finish()) return fail(QS_ENOMEM, "qs_batch_create: no host memory for the pass-major programs");
     BatchArgs &a = b->args;
     a.states = static_cast<const BatchState *>(b->d_states);
     a.order = static_cast<const int32_t *>(b->d_order);
@@ -696,9 +735,7 @@ qs_status qs_batch_bytes(const qs_batch *b, double *algorithmic_bytes) {
     // writes lambda, every sweep pass reads and writes the selected tiles of psi and lambda
     double total = 0.0;
     const double es = (double)elem_bytes(b->dtype);
-    for (const BatchJitProg &cjp : b->jprogs) {
-        BatchJitProg &jp = const_cast<BatchJitProg &>(cjp);
-        plan_major(b, jp);
+    for (const BatchJitProg &jp : b->jprogs) {
         const double state = std::ldexp(es, jp.n);
         double per = 3.0 * state;
         for (size_t i = 0; i < jp.pf.passes.size(); ++i) per += 2.0 * state * pass_touched_fraction(jp.pf, (int)i);

@@ -316,7 +316,8 @@ int qs_get_l2_fetch_bytes(void);
  * not NULL, *out_norm2 = sum_k |psi_k|^2 -- all in one pass over the state. Complex64
  * states sum |psi_k|^2 in float32 within a tile of 8192 amplitudes, with a compensated
  * (Kahan) float32 running sum over a block's tiles and float64 across blocks; complex128
- * states sum in float64 throughout. Deterministic (fixed summation order).
+ * states sum each thread's amplitudes of a tile as 64-bit integers at a common scale (no worse
+ * than float64) and those sums in float64. Deterministic (fixed summation order).
  * With QS_FLAG_OUT_DEVICE in flags, out / out_norm2 are device pointers and the call is
  * asynchronous; otherwise they are host pointers and the call synchronises the stream. */
 qs_status qs_expect_z(const qs_state *s, double *out, double *out_norm2, int flags);

@@ -43,14 +43,18 @@ int occupancy_of(K kern) {
 template <typename Real, typename Idx, int NS, int LAY, int R, int OP, bool MASKED>
 cudaError_t go(void *psi, const GatePlan &p, const FxMat &fx, uint64_t cmask, uint64_t cvals, cudaStream_t st) {
     // units in flight per thread: complex64 2 with a vector on each side, 4 with one vector per unit.
-    // Exchanges have no arithmetic, and with 2 their loads and stores alternate at the memory: n = 28
-    // complex128, target 14, 1 / 2 / 4 / 8 units 1.33 / 1.55 / 1.33 / 1.30 ms; n = 29 complex64 1.35 /
-    // 1.43 / 1.34 / 1.32. complex128 arithmetic (one 16-byte vector per amplitude; n = 28, target 14, 1 / 2
-    // / 4 units): general 1.38 / 1.39 / 1.36 ms, real 1.40 / 1.39 / 1.35, unlike entries 1.43 / 1.46 /
-    // 1.49, diagonal 1.39 / 1.41 / 1.40, one-sided 0.67 / 0.72 / 0.72.
-    constexpr int UNR = OP == OP_SWAP ? 4
-                        : sizeof(Real) == 8 ? (OP == OP_GEN || OP == OP_REAL ? 4 : 1)
-                                            : (LAY == LAY_ADJ || OP == OP_SIDE) ? 4 : 2;
+    // Exchanges have no arithmetic, and with 2 units their loads and stores alternate at the memory: n = 29
+    // complex64, target 14, 1 / 2 / 4 / 8 units 1.35 / 1.43 / 1.34 / 1.32 ms. Single amplitudes (an inserted
+    // qubit 0: isolated 8 bytes) keep 2: X on q controlled by every lower qubit, q = 0..28, 1 / 2 / 4 units
+    // 7.10 / 7.14 / 7.60 ms (q = 1 alone 1.52 / 1.46 / 1.53). complex128 exchanges take 1: n = 28, target 14,
+    // 1 / 2 / 4 units 1.33 / 1.55 / 1.33 ms, X controlled by every lower qubit 5.56 / 5.86 / 5.64.
+    // complex128 arithmetic (one 16-byte vector per amplitude; n = 28, target 14, 1 / 2 / 4 units): general
+    // 1.38 / 1.39 / 1.36 ms, real 1.40 / 1.39 / 1.35, unlike entries 1.43 / 1.46 / 1.49, diagonal 1.39 / 1.41
+    // / 1.40, one-sided 0.67 / 0.72 / 0.72.
+    constexpr bool pair_unit = LAY == LAY_ADJ || OP == OP_SIDE;  // one vector per unit
+    constexpr int UNR = sizeof(Real) == 4 ? (pair_unit || (OP == OP_SWAP && R == 2) ? 4 : 2)
+                        : OP == OP_SWAP   ? (pair_unit ? 4 : 1)
+                                          : (OP == OP_GEN || OP == OP_REAL ? 4 : 1);
     auto kern = k_gate<Real, Idx, NS, LAY, R, OP, MASKED, UNR>;
     static const int occ = occupancy_of(kern);
     const uint64_t per_block = (uint64_t)kGateThreads * UNR;

@@ -7,8 +7,8 @@
 // register groups (row deposits, swizzled element offsets, folded exchanges), every gate's
 // operation, target place and control pattern become compile-time constants, so each gate is
 // straight-line code (its pair updates, predicated on row controls and guarded by its tile
-// predicate). Only the gate matrices (and, in the adjoint sweep, their derivatives) are kernel
-// parameters: they live in the constant bank, where the FMA instructions read them directly,
+// predicate). Only the gate matrices (and, in the adjoint sweep, the scales of the derivative
+// products) are kernel parameters: they live in the constant bank, where the FMA instructions read them directly,
 // and a circuit with the same structure but other angles reuses the compiled kernel.
 //
 // Sources are compiled with NVRTC for sm_103a into a cubin, cached by source text (a process-

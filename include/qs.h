@@ -249,8 +249,8 @@ qs_status qs_circuit_order(int n, qs_dtype dtype, const qs_gate *gates, size_t c
 /* Measured FMA rate of the current device in the arithmetic of `dtype` (QS_C64: float32,
  * QS_C128: float64), in flop/s (2 per FMA): one launch of independent FMA chains on every SM
  * for `iters` iterations (1 .. 2^24), timed with CUDA events on `stream`; synchronises the
- * stream. It is the denominator of the arithmetic rooflines (the complex128 path runs on the
- * FP64 pipe). Not part of the paper's method. */
+ * stream. It is the denominator of the arithmetic rooflines (complex128 tile passes run on
+ * the FP64 pipe). Not part of the paper's method. */
 qs_status qs_measure_fma_peak(qs_dtype dtype, int iters, void *stream, double *flops_per_s);
 
 /* Debug build (the library compiled with QS_DEBUG_CHECKS, libqs_debug.so): the gate,

@@ -1,8 +1,7 @@
 // k_peak.cu -- measured arithmetic peak of the device (the denominator of the ALU rooflines).
 //
-// complex128 gate updates and reductions run on the FP64 pipe, whose rate on this part is a
-// small fraction of the FP32 rate; their roofline is stated against a measured FMA rate, not a
-// datasheet figure. The kernel keeps 8 independent FMA chains per thread (enough to cover the
+// complex128 tile passes run on the FP64 pipe, whose rate on this part is a small fraction of the
+// FP32 rate; the arithmetic rooflines are stated against a measured FMA rate, not a datasheet figure. The kernel keeps 8 independent FMA chains per thread (enough to cover the
 // pipe latency) for `iters` iterations on every SM; flops = 2 per FMA.
 #include "qs_internal.cuh"
 

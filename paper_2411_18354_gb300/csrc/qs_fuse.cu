@@ -472,7 +472,7 @@ static void make_pass(int n, uint64_t Lmask, TilePass *P) {
 // whatever its kind (general 11.3, real 9.1, exchange 8.2 unless folded into a register
 // group's gather / scatter, diagonal about as much: the interpreter's per-gate work, not the
 // arithmetic, sets it), also for gates whose non-local controls select only some tiles;
-// 0.15 fits the measured plans best. complex128 gates are FP64-bound alone and inside a pass
+// 0.15 fits the measured plans best. complex128 gates are FP64-bound inside a pass
 // (a general 2x2 costs ~3 units there; alone, in fixed point, one), so only exchanges (no
 // arithmetic, ~0.33) gain from a pass.
 // A pass with fewer tiles than SMs leaves the rest idle, and its FP64 work takes as many times longer

@@ -157,7 +157,7 @@ __device__ __forceinline__ double to_f64(long long s, int sc) {
     return __hiloint2double(s ? __double2hiint(d) + (sc << 20) : 0, __double2loint(d));
 }
 
-// The same on the integer pipe (17 operations; ties away from zero), for forms whose conversions would
+// The same on the integer pipe (18 operations; ties away from zero), for forms whose conversions would
 // fill the FP64 pipe: a real update of psi and lambda with its derivative product, 2^23 pairs each:
 // all by conversion 206 us, half by integers 184, all by integers 207 (160 of memory time).
 __device__ __forceinline__ double to_f64_int(long long s, int sc) {
@@ -166,7 +166,10 @@ __device__ __forceinline__ double to_f64_int(long long s, int sc) {
     const unsigned uh = (unsigned)(u >> 32);
     const int lz = uh ? __clz((int)uh) : 32 + __clz((int)u);
     asm("shl.b64 %0, %0, %1;" : "+l"(u) : "r"(lz));
-    u = (u + 0x400) >> 11;  // the leading bit at bit 52: added to the exponent field below
+    // the leading bit at bit 52, added to the exponent field below. The rounding bit is added after the
+    // shift: before it the sum passes 64 bits for results just below a power of two (here it becomes 2^53,
+    // whose carry the exponent field takes).
+    u = (u >> 11) + ((u >> 10) & 1);
     const unsigned hi = (unsigned)(u >> 32) + ((unsigned)(1023 + 62 - lz + sc) << 20);
     return __hiloint2double(s ? (int)(hi | ((unsigned)sg & 0x80000000u)) : 0, (int)(unsigned)u);
 }

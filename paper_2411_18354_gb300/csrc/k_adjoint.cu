@@ -55,8 +55,8 @@ k_adj_step(typename CxT<Real>::T *__restrict__ psi, typename CxT<Real>::T *__res
                     acc = fma(a[i].x, x[i].y, acc);
                     acc = fma(-a[i].y, x[i].x, acc);
                 }
-                gate_side(x[i], g);
-                gate_side(a[i], g);
+                gate_side<true>(x[i], g);
+                gate_side<true>(a[i], g);
             }
             Vec<Real, R>::st(psi + k, x);
             Vec<Real, R>::st(lam + k, a);
@@ -161,8 +161,8 @@ k_adj_step_zy(typename CxT<Real>::T *__restrict__ psi, typename CxT<Real>::T *__
             T2 &b = (LAY == LAY_ADJ) ? lx[2 * i + 1] : ly[i];
             az = fma(b.y, y.x, az);  // -Im(conj(b) y): side 1 of a Z rotation (k_adj_step)
             az = fma(-b.x, y.y, az);
-            gate_side(y, gz);
-            gate_side(b, gz);
+            gate_side<true>(y, gz);
+            gate_side<true>(b, gz);
             ay = fma(b.x, x.x, ay);
             ay = fma(b.y, x.y, ay);
             ay = fma(-a.x, y.x, ay);
@@ -350,7 +350,7 @@ template <typename Real, typename Idx, int NS>
 cudaError_t by_shape(void *psi, void *lam, const GatePlan &p, const FxMat &fx, double *part, cudaStream_t st) {
     constexpr bool F = sizeof(Real) == 4;
     int op = p.op;
-    if (!F && op == OP_GEN && fx.form == FX_GENW) op = OP_GENW;
+    if (!F && op == OP_GEN && fx.form == FX_GENP) op = OP_GENP;
 #define QS_ADJ_OPS(LAY, R)                                                                                     \
     if (part) {                                                                                                \
         if (op == OP_DIAG) return go<Real, Idx, NS, LAY, R, OP_DIAG, PAULI_Z>(psi, lam, p, fx, part, st);       \
@@ -360,7 +360,7 @@ cudaError_t by_shape(void *psi, void *lam, const GatePlan &p, const FxMat &fx, d
     } else {                                                                                                   \
         if (op == OP_REAL) return go<Real, Idx, NS, LAY, R, OP_REAL, PAULI_NONE>(psi, lam, p, fx, part, st);    \
         if (op == OP_GEN) return go<Real, Idx, NS, LAY, R, OP_GEN, PAULI_NONE>(psi, lam, p, fx, part, st);      \
-        if (op == OP_GENW) return go<Real, Idx, NS, LAY, R, F ? OP_GEN : OP_GENW, PAULI_NONE>(psi, lam, p, fx, part, st); \
+        if (op == OP_GENP) return go<Real, Idx, NS, LAY, R, F ? OP_GEN : OP_GENP, PAULI_NONE>(psi, lam, p, fx, part, st); \
         if (op == OP_DIAG) return go<Real, Idx, NS, LAY, R, OP_DIAG, PAULI_NONE>(psi, lam, p, fx, part, st);    \
         if (op == OP_SWAP) return go<Real, Idx, NS, LAY, R, OP_SWAP, PAULI_NONE>(psi, lam, p, fx, part, st);    \
         if (op == OP_SIDE && LAY == LAY_SPLIT)                                                                 \

@@ -155,15 +155,15 @@ __device__ __forceinline__ void pair_update(T2 &x, T2 &y, const Real *m) {
 // (k_fx.cuh); a pair of zeros needs neither. G: a gate with its matrix m (and limbs fx).
 template <int OP, typename G>
 __device__ __forceinline__ void gate_pair(float2 &x, float2 &y, const G &g) {
-    pair_update<OP == OP_GENW ? (int)OP_GEN : OP, float2, float>(x, y, g.m);
+    pair_update<OP == OP_GENP ? (int)OP_GEN : OP, float2, float>(x, y, g.m);
 }
-template <typename G>
+template <bool INT = false, typename G>
 __device__ __forceinline__ void gate_side(float2 &x, const G &g) {
     x = cmul<float2, float>(g.m[0], g.m[1], x);
 }
-template <typename G>
+template <bool INT = false, typename G>
 __device__ __forceinline__ void gate_side(double2 &x, const G &g) {
-    if (!fx::mul<0>(x, g.fx) && (fx::nonzero(x.x) || fx::nonzero(x.y))) {
+    if (!fx::mul<0, INT>(x, g.fx) && (fx::nonzero(x.x) || fx::nonzero(x.y))) {
         fx::rare(x.x);
         x = cmul<double2, double>(g.m[0], g.m[1], x);
     }
@@ -181,8 +181,8 @@ template <int OP, typename G>
 __device__ __forceinline__ void gate_pair(double2 &x, double2 &y, const G &g) {
     if (OP == OP_SWAP) {
         pair_update<OP, double2, double>(x, y, g.m);
-    } else if (OP == OP_GEN || OP == OP_GENW) {
-        if (!(OP == OP_GEN ? fx::gen(x, y, g.fx) : fx::genw(x, y, g.fx)) &&
+    } else if (OP == OP_GEN || OP == OP_GENP) {
+        if (!(OP == OP_GEN ? fx::gen(x, y, g.fx) : fx::genp(x, y, g.fx)) &&
             (fx::nonzero(x.x) || fx::nonzero(x.y) || fx::nonzero(y.x) || fx::nonzero(y.y))) {
             fx::rare(x.x);
             pair_update<OP_GEN, double2, double>(x, y, g.m);
@@ -208,7 +208,7 @@ template <typename Idx>
 __device__ __forceinline__ void gate_pair_any(double2 &x, double2 &y, const DevGate<double, Idx> &g, int side) {
     switch (g.fx.form) {
     case FX_GEN: gate_pair<OP_GEN>(x, y, g); break;
-    case FX_GENW: gate_pair<OP_GENW>(x, y, g); break;
+    case FX_GENP: gate_pair<OP_GENP>(x, y, g); break;
     case FX_REAL: gate_pair<OP_REAL>(x, y, g); break;
     case FX_DIAG: gate_pair<OP_DIAG>(x, y, g); break;
     default: gate_side(side ? y : x, g); break;

@@ -49,8 +49,8 @@ cudaError_t go(void *psi, const GatePlan &p, const FxMat &fx, uint64_t cmask, ui
     // 7.10 / 7.14 / 7.60 ms (q = 1 alone 1.52 / 1.46 / 1.53). complex128 exchanges take 1: n = 28, target 14,
     // 1 / 2 / 4 units 1.33 / 1.55 / 1.33 ms, X controlled by every lower qubit 5.56 / 5.86 / 5.64.
     // complex128 arithmetic (one 16-byte vector per amplitude; n = 28, target 14, 1 / 2 / 4 units): general
-    // 1.38 / 1.39 / 1.36 ms, real 1.40 / 1.39 / 1.35, unlike entries 1.43 / 1.46 / 1.49, diagonal 1.39 / 1.41
-    // / 1.40, one-sided 0.67 / 0.72 / 0.72.
+    // 1.38 / 1.39 / 1.36 ms, real 1.40 / 1.39 / 1.35, parts of unlike size 1.97 / 1.90 / 1.94 (but n = 20: 9.1 /
+    // 10.0 / 10.3 us), diagonal 1.39 / 1.41 / 1.40, one-sided 0.67 / 0.72 / 0.72.
     constexpr bool pair_unit = LAY == LAY_ADJ || OP == OP_SIDE;  // one vector per unit
     constexpr int UNR = sizeof(Real) == 4 ? (pair_unit || (OP == OP_SWAP && R == 2) ? 4 : 2)
                         : OP == OP_SWAP   ? (pair_unit ? 4 : 1)
@@ -85,11 +85,11 @@ template <typename Real, typename Idx, int NS, bool MASKED>
 cudaError_t by_shape(void *psi, const GatePlan &p, const FxMat &fx, uint64_t cmask, uint64_t cvals, cudaStream_t st) {
     constexpr bool F = sizeof(Real) == 4;
     int op = MASKED ? (int)OP_GEN : p.op;
-    if (!F && !MASKED && op == OP_GEN && fx.form == FX_GENW) op = OP_GENW;
+    if (!F && !MASKED && op == OP_GEN && fx.form == FX_GENP) op = OP_GENP;
 #define QS_OPS(LAY, R)                                                                        \
     switch (op) {                                                                             \
         case OP_GEN: return go<Real, Idx, NS, LAY, R, OP_GEN, MASKED>(psi, p, fx, cmask, cvals, st); \
-        case OP_GENW: if (!MASKED && !F) return go<Real, Idx, NS, LAY, R, F ? OP_GEN : OP_GENW, false>(psi, p, fx, cmask, cvals, st); break; \
+        case OP_GENP: if (!MASKED && !F) return go<Real, Idx, NS, LAY, R, F ? OP_GEN : OP_GENP, false>(psi, p, fx, cmask, cvals, st); break; \
         case OP_REAL: if (!MASKED) return go<Real, Idx, NS, LAY, R, OP_REAL, false>(psi, p, fx, cmask, cvals, st); break; \
         case OP_SWAP: if (!MASKED) return go<Real, Idx, NS, LAY, R, OP_SWAP, false>(psi, p, fx, cmask, cvals, st); break; \
         case OP_DIAG: if (!MASKED) return go<Real, Idx, NS, LAY, R, OP_DIAG, false>(psi, p, fx, cmask, cvals, st); break; \

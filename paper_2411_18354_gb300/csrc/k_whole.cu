@@ -97,7 +97,7 @@ template <typename Real, typename T2>
 __device__ __forceinline__ void run_gate(T2 *sm, const WholeGate<Real> &g) {
     switch (g.op) {  // uniform
     case OP_GEN: run_op<OP_GEN, Real>(sm, g); break;
-    case OP_GENW: if (sizeof(Real) == 8) run_op<OP_GENW, Real>(sm, g); break;
+    case OP_GENP: if (sizeof(Real) == 8) run_op<OP_GENP, Real>(sm, g); break;
     case OP_REAL: run_op<OP_REAL, Real>(sm, g); break;
     case OP_SWAP: run_op<OP_SWAP, Real>(sm, g); break;
     case OP_DIAG: run_op<OP_DIAG, Real>(sm, g); break;
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(kWholeThreads) k_whole(typename CxT<Real>::T *
 inline void set_fx(WholeGate<float> &, const GatePlan &) {}
 inline void set_fx(WholeGate<double> &g, const GatePlan &p) {
     make_fx(p.U, p.op, &g.fx);
-    if (p.op == OP_GEN && g.fx.form == FX_GENW) g.op = OP_GENW;
+    if (p.op == OP_GEN && g.fx.form == FX_GENP) g.op = OP_GENP;
 }
 
 // Threads of the block. complex64: a gate is mostly issue (each thread's index and descriptor work, 16

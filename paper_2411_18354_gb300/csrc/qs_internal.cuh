@@ -22,7 +22,7 @@ enum GateOp : int {
     OP_DIAG = 2,  // (x, y) -> (a x, d y)
     OP_SIDE = 3,  // one side only: z -> s z on the amplitudes whose bit t equals `side`
     OP_REAL = 4,  // general 2x2 with real entries (e.g. RY, H): half the multiplications
-    OP_GENW = 5,  // kernels only: OP_GEN on complex128 with entries of unlike size (k_fx.cuh)
+    OP_GENP = 5,  // kernels only: OP_GEN on complex128 with parts of unlike size (k_fx.cuh)
 };
 
 // Layout classes of one work unit (see k_gate.cu).

@@ -199,10 +199,10 @@ int batch_grid(int dtype, size_t smem) {
     int occ = 0;
     cudaError_t e;
     if (dtype == QS_C64) {
-        e = cudaFuncSetAttribute(k_batch<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_smem(reinterpret_cast<const void *>(k_batch<float>), smem);
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch<float>, kBatchThreads, smem);
     } else {
-        e = cudaFuncSetAttribute(k_batch<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_smem(reinterpret_cast<const void *>(k_batch<double>), smem);
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch<double>, kBatchThreads, smem);
     }
     if (e != cudaSuccess) {

@@ -1,6 +1,5 @@
 // k_tile.cu -- fused tile-pass kernels (forward, and adjoint over psi and lambda).
 #include <algorithm>
-#include <atomic>
 
 #include "k_tile_dev.cuh"
 
@@ -63,16 +62,8 @@ cudaError_t go(void *psi, void *lam, const TilePass &p, const TileGroup *groups,
                size_t part_stride, cudaStream_t st) {
     auto kern = k_tile_pass<Real, ADJ>;
     const size_t smem = tile_smem_bytes(sizeof(Real) == 4 ? QS_C64 : QS_C128, p.k, ADJ, p.group_count, p.gate_count);
-    static std::atomic<size_t> configured[64];  // per device: dynamic shared memory allowed so far
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
-    if (smem > 48 * 1024 && smem > configured[dev].load()) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        size_t cur = configured[dev].load();
-        while (cur < smem && !configured[dev].compare_exchange_weak(cur, smem)) {
-        }
-    }
+    const cudaError_t allowed = allow_smem(reinterpret_cast<const void *>(kern), smem);
+    if (allowed != cudaSuccess) return allowed;
     int occ = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kTileThreads, smem) != cudaSuccess || occ < 1) occ = 1;
     uint64_t cap = (uint64_t)device_sm_count() * occ;

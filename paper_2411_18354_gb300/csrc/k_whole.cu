@@ -191,10 +191,8 @@ template <typename Real>
 cudaError_t go(void *psi, int n, const void *gates, int count, cudaStream_t st) {
     using T2 = typename CxT<Real>::T;
     const size_t smem = (sizeof(T2) << n) + kWholeChunk * sizeof(WholeGate<Real>);
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_whole<Real>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(reinterpret_cast<const void *>(k_whole<Real>), smem);
+    if (e != cudaSuccess) return e;
     // a gate has at most 8 block widths of pairs (run_op)
     static_assert(1 << (kWholeBitsC64 - 4) <= kWholeThreads && 1 << (kWholeBitsC128 - 4) <= 512, "more pairs per thread");
     k_whole<Real><<<1, whole_threads(n, sizeof(Real) == 8), smem, st>>>(static_cast<T2 *>(psi), n, static_cast<const WholeGate<Real> *>(gates), count);

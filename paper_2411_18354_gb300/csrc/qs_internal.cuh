@@ -76,6 +76,9 @@ void build_map(int n, const int *pos, int m, uint64_t ins, IndexMap *map);
 void plan_masked(const GatePlan &compact, GatePlan *out);
 
 int device_sm_count();
+// Raises a kernel's dynamic shared memory limit on the current device to `bytes` where it is lower. The
+// limit belongs to the kernel, so every caller of it on any thread shares it: it is never lowered.
+cudaError_t allow_smem(const void *kernel, size_t bytes);
 
 // Launchers (return the CUDA error of the launch).
 cudaError_t launch_gate(int dtype, void *psi, const GatePlan &p, cudaStream_t st);

@@ -5,6 +5,9 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <map>
+#include <mutex>
+#include <utility>
 
 #include "qs_internal.cuh"
 
@@ -26,6 +29,21 @@ int device_sm_count() {
         sms_of[dev].store(sms, std::memory_order_relaxed);
     }
     return sms;
+}
+
+cudaError_t allow_smem(const void *kernel, size_t bytes) {
+    if (bytes <= 48 * 1024) return cudaSuccess;  // allowed without asking
+    static std::mutex mu;
+    static std::map<std::pair<int, const void *>, size_t> allowed;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    size_t &now = allowed[{dev, kernel}];
+    if (now >= bytes) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) now = bytes;
+    return e;
 }
 
 static int ctz64(uint64_t v) { return __builtin_ctzll(v); }

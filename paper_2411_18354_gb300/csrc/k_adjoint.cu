@@ -250,11 +250,25 @@ __global__ void __launch_bounds__(256) k_obs_energy(const float2 *__restrict__ p
     }
 }
 
+// Sums of the first `rows` slot rows, each into its first element: a warp per row.
+__global__ void __launch_bounds__(256) k_slot_sums(double *__restrict__ part, int rows) {
+    const int s = (int)((blockIdx.x * 256 + threadIdx.x) >> 5);
+    const int lane = threadIdx.x & 31;
+    if (s >= rows) return;  // uniform over the warp
+    double *row = part + (size_t)s * kAdjMaxBlocks;
+    double v = 0.0;
+    for (int b = lane; b < kAdjMaxBlocks; b += 32) v += row[b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) row[0] = v;
+}
+
 // grad[p] = 2 * sum over the slots whose parameter is p, and over their blocks, of part[s][b]: a warp
-// per parameter, lane l looking at slots l, l + 32, ... and adding blocks l, l + 32, ... of each hit,
-// then a fixed-order shuffle reduction. Warp nparams (energy != nullptr): the energy from slot row
-// nslots. (Slot sums, a thread per parameter walking all slots, and the energy's own kernels were
-// four launches; the walk alone took 55 us at 960 slots.)
+// per parameter, lane l looking at slots l, l + 32, ... and adding blocks l, l + 32, ... of each hit
+// (SUMMED: the hit's sum, which k_slot_sums left in its first element), then a fixed-order shuffle
+// reduction. Warp nparams (energy != nullptr): the energy from slot row nslots. (A thread per parameter
+// walking all slots, and the energy's own kernels, were two more launches; the walk took 55 us at 960 slots.)
+template <bool SUMMED>
 __global__ void __launch_bounds__(256) k_grad_final(const double *__restrict__ part, const int *__restrict__ slot_param,
                                                     int nslots, double *__restrict__ grad, int nparams,
                                                     double *__restrict__ energy) {
@@ -263,14 +277,19 @@ __global__ void __launch_bounds__(256) k_grad_final(const double *__restrict__ p
     if (p > nparams || (p == nparams && !energy)) return;  // uniform over the warp
     double v = 0.0;
     auto add_row = [&](int s) {
-        for (int b = lane; b < kAdjMaxBlocks; b += 32) v += part[(size_t)s * kAdjMaxBlocks + b];
+        for (int b = lane; b < (SUMMED ? 1 : kAdjMaxBlocks); b += 32) v += part[(size_t)s * kAdjMaxBlocks + b];
     };
     if (p == nparams) {
         add_row(nslots);
     } else {
         for (int s0 = 0; s0 < nslots; s0 += 32) {
-            unsigned hits = __ballot_sync(0xffffffffu, s0 + lane < nslots && slot_param[s0 + lane] == p);
-            for (; hits; hits &= hits - 1) add_row(s0 + __ffs(hits) - 1);
+            const bool hit = s0 + lane < nslots && slot_param[s0 + lane] == p;
+            if (SUMMED) {
+                if (hit) v += part[(size_t)(s0 + lane) * kAdjMaxBlocks];
+            } else {
+                unsigned hits = __ballot_sync(0xffffffffu, hit);
+                for (; hits; hits &= hits - 1) add_row(s0 + __ffs(hits) - 1);
+            }
         }
     }
 #pragma unroll
@@ -434,12 +453,23 @@ cudaError_t launch_obs_energy(const void *psi, void *lam, int n, double *part, c
     return cudaGetLastError();
 }
 
-// energy (may be null): written from the partial sums in row nslots of part.
-cudaError_t launch_grad_final(const double *part, int nslots, const int *slot_param, double *grad, int nparams,
+// energy (may be null): written from the partial sums in row nslots of part. most: the most slots that
+// one parameter has. Its warp reads a row of 1024 partial sums in 1.8 us, and rows follow one another (one
+// parameter for all 320 slots of an n = 20 complex64 gradient: 1758 us, with the rows summed first 1188);
+// a launch of its own for the rows' sums takes about as long as two rows.
+cudaError_t launch_grad_final(double *part, int nslots, int most, const int *slot_param, double *grad, int nparams,
                               double *energy, cudaStream_t st) {
     if (nparams == 0 && !energy) return cudaSuccess;
-    const uint64_t warps = (uint64_t)nparams + 1;
-    k_grad_final<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(part, slot_param, nslots, grad, nparams, energy);
+    const unsigned grid = (unsigned)(((uint64_t)nparams + 1 + 7) / 8);
+    if (most > 2) {
+        const int rows = nslots + (energy ? 1 : 0);
+        k_slot_sums<<<(rows + 7) / 8, 256, 0, st>>>(part, rows);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        k_grad_final<true><<<grid, 256, 0, st>>>(part, slot_param, nslots, grad, nparams, energy);
+    } else {
+        k_grad_final<false><<<grid, 256, 0, st>>>(part, slot_param, nslots, grad, nparams, energy);
+    }
     return cudaGetLastError();
 }
 

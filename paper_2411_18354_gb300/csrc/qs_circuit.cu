@@ -27,7 +27,7 @@ cudaError_t launch_adj_step_zy(int dtype, void *psi, void *lam, const GatePlan &
 cudaError_t launch_obs_sumz(const void *psi, void *lam, int n, cudaStream_t st);
 cudaError_t launch_sum_vec(const double *z, int n, double *out, cudaStream_t st);
 cudaError_t launch_obs_energy(const void *psi, void *lam, int n, double *part, cudaStream_t st);
-cudaError_t launch_grad_final(const double *part, int nslots, const int *slot_param, double *grad, int nparams,
+cudaError_t launch_grad_final(double *part, int nslots, int most, const int *slot_param, double *grad, int nparams,
                               double *energy, cudaStream_t st);
 
 void release_state_buffers(qs_state *s) {
@@ -515,6 +515,17 @@ static void plan_adjoint_programs(const qs_state *s, int flags, AdjPlan *ap) {
     // (compiled passes too: with 4, their long straight-line groups spill registers)
     plan_fused(s->n, s->dtype, tile_bits(s->dtype, true, jit), seq, ap->adj, &ap->slot_of, &ap->pa,
                kPassMaxGates, true, 0, jit);
+}
+
+// How often the most used parameter occurs.
+static int most_uses(std::vector<int> params) {
+    std::sort(params.begin(), params.end());
+    int most = 0;
+    for (size_t i = 0, j; i < params.size(); i = j) {
+        for (j = i; j < params.size() && params[j] == params[i];) ++j;
+        most = std::max(most, (int)(j - i));
+    }
+    return most;
 }
 
 static bool plan_adjoint(const qs_state *s, const qs_gate *gates, size_t count, const double *theta, size_t n_theta,
@@ -1182,7 +1193,7 @@ qs_status qs_adjoint_grad(qs_state *s, const qs_gate *gates, size_t count, const
             if (e != cudaSuccess) return cuda_fail(e, "qs_adjoint_grad sweep launch");
         }
     }
-    e = launch_grad_final(part, nslots, slot_param_dev, on_dev ? grad : grad_dev, (int)n_theta,
+    e = launch_grad_final(part, nslots, most_uses(slot_param), slot_param_dev, on_dev ? grad : grad_dev, (int)n_theta,
                           s->dtype == QS_C64 ? energy_to : nullptr, stm);
     if (e != cudaSuccess) return cuda_fail(e, "qs_adjoint_grad final");
     if (!on_dev) {

@@ -574,11 +574,11 @@ def measure_batch(qs, W, peak):
                  {"small_bits": 12, "tile_bits": 11, "max_pass_gates": 64}):
         b = qs.Batch(ns, circuits, nparams, "c64", **jcfg)
         try:
-            jbytes = b.algorithmic_bytes()
             t0 = time.perf_counter()
             b.run(th, en, gr, qs.QS_FLAG_GRAPH | qs.QS_FLAG_JIT)
             torch.cuda.synchronize()
             first_s = time.perf_counter() - t0
+            jbytes = b.algorithmic_bytes()
             msj = _events_ms(lambda: b.run(th, en, gr, qs.QS_FLAG_GRAPH | qs.QS_FLAG_JIT), 3)
         finally:
             b.close()

@@ -402,7 +402,8 @@ qs_status qs_batch_info(const qs_batch *b, int *grid, int *small_bits, int *tile
 /* Bytes one run of the batch must move through device memory (its states above small_bits:
  * |0...0> written, each forward pass reading and writing the tiles its gates select, lambda =
  * O psi, each sweep pass reading and writing the selected tiles of psi and lambda; states in
- * shared memory move none): the numerator of the batch's roofline. Host only. */
+ * shared memory move none): the numerator of the batch's roofline. Of the passes of the last run's path
+ * (QS_FLAG_JIT or not), before the first run of the path without it. Host only. */
 qs_status qs_batch_bytes(const qs_batch *b, double *algorithmic_bytes);
 
 /* Release a batch (synchronises its stream first). NULL is accepted. */

@@ -44,7 +44,7 @@ constexpr int kSide = 3;  // parallel branches of a pass-major graph beside the 
 struct BatchJitProg {
     int n = 0, nparam = 0;
     std::vector<int> states;        // global state indices
-    std::vector<qs_gate> gates;     // of each state, until its programs are planned
+    std::vector<qs_gate> gates;     // of each state, until its programs are planned (first QS_FLAG_JIT run)
     qs::FusedProgram pf, pa;        // forward and sweep programs (rotation kinds / indices filled in)
     std::vector<qs::JitPass> jf, ja;
     void *psi = nullptr, *lam = nullptr;
@@ -90,7 +90,10 @@ struct qs_batch {
     int *d_small_order = nullptr;
     uint64_t *d_param_off = nullptr;
     std::vector<uint64_t> param_off_host;
-    bool jit_ready = false;
+    bool planned = false;     // the programs' passes
+    bool jit_ready = false;   // their kernels and buffers
+    bool last_jit = false;    // the path of the last run
+    double bytes = 0.0;       // what a run of the persistent kernel moves through device memory
     double jit_compile_s = 0.0;
 };
 
@@ -210,12 +213,13 @@ void plan_major(const qs_batch *b, BatchJitProg &jp, int dir) {
     }
 }
 
-// Plans every program of a batch on threads of their own, a program's two directions apart, while
-// qs_batch_create uploads the persistent kernel's tables (64 states of 13-15 qubits, 6 layers: the first
-// run takes 1.02 ms, with the planning in it 1.46).
+// Plans every program of a batch, its directions apart, on threads of their own, while the first
+// QS_FLAG_JIT run allocates what does not depend on the passes. (In qs_batch_create the planning cost
+// batches that never take the pass-major path 10 to 25 % of their creation: 512 states of 10-18 qubits 5.2 ms,
+// without 4.7; one program of 47 states 0.50, 0.43.)
 class MajorPlanner {
   public:
-    explicit MajorPlanner(qs_batch *b) : b_(b), count_(2 * b->jprogs.size()) {
+    explicit MajorPlanner(qs_batch *b) : b_(b), count_(b->planned ? 0 : 2 * b->jprogs.size()) {
         const size_t threads = std::min<size_t>(std::max(1u, std::thread::hardware_concurrency()), count_);
         try {
             th_.reserve(threads);
@@ -228,15 +232,17 @@ class MajorPlanner {
     bool finish() {
         work();
         join();
+        if (failed_) return false;
         for (BatchJitProg &jp : b_->jprogs) jp.gates = {};
-        return !failed_;
+        b_->planned = true;
+        return true;
     }
+
+  private:
     void join() {
         for (std::thread &t : th_) t.join();
         th_.clear();
     }
-
-  private:
     void work() {
         try {
             for (size_t q; (q = next_.fetch_add(1)) < count_;) plan_major(b_, b_->jprogs[q / 2], (int)(q & 1));
@@ -254,7 +260,27 @@ class MajorPlanner {
 // Compile the pass-major path's kernels and allocate its buffers (first QS_FLAG_JIT run).
 qs_status ensure_jit(qs_batch *b) {
     if (b->jit_ready) return QS_OK;
+    MajorPlanner planner(b);
     const size_t es = elem_bytes(b->dtype), rs = es / 2;
+    auto dev_alloc = [](void **p, size_t bytes) {
+        if (*p) return true;  // (left by a run that failed later)
+        cudaError_t e = cudaMalloc(p, std::max<size_t>(bytes, 16));
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            *p = nullptr;
+            return false;
+        }
+        return true;
+    };
+    const char *const no_memory = "qs_batch_run: cannot allocate the pass-major state buffers";
+    for (BatchJitProg &jp : b->jprogs) {
+        const size_t S = jp.states.size(), N = size_t(1) << jp.n;
+        if (!dev_alloc(&jp.psi, S * N * es) || !dev_alloc(&jp.lam, S * N * es) ||
+            !dev_alloc((void **)&jp.cs, S * std::max(1, jp.nparam) * 2 * sizeof(double)) ||
+            !dev_alloc((void **)&jp.obs, bm_obs_partials(jp.n, (int)S) * sizeof(double)))
+            return set_error(QS_ENOMEM, no_memory);
+    }
+    if (!planner.finish()) return set_error(QS_ENOMEM, "qs_batch_run: no host memory for the pass-major programs");
     std::vector<JitRequest> reqs;
     for (BatchJitProg &jp : b->jprogs) {
         reqs.push_back({&jp.pf, false, true, &jp.jf});
@@ -268,18 +294,8 @@ qs_status ensure_jit(qs_batch *b) {
         if (e == cudaSuccess) e = jit_load(jp.ja);
         if (e != cudaSuccess) return cuda_fail(e, "qs_batch_run: loading compiled passes");
     }
-    auto dev_alloc = [](void **p, size_t bytes) {
-        cudaError_t e = cudaMalloc(p, std::max<size_t>(bytes, 16));
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            *p = nullptr;
-            return false;
-        }
-        return true;
-    };
     for (BatchJitProg &jp : b->jprogs) {
         const int S = (int)jp.states.size();
-        const size_t N = size_t(1) << jp.n;
         jp.tiles = jp.pa.passes.empty() ? (jp.pf.passes.empty() ? 1u : (uint32_t)jp.pf.passes[0].ntiles)
                                         : (uint32_t)jp.pa.passes[0].ntiles;
         // sweep partials: per pass, [J][state][tile]; per parameter, the blocks of its gates
@@ -326,12 +342,8 @@ qs_status ensure_jit(qs_batch *b) {
             flat.insert(flat.end(), items[q].begin(), items[q].end());
         }
         csr[jp.nparam] = (int)flat.size();
-        if (!dev_alloc(&jp.psi, (size_t)S * N * es) || !dev_alloc(&jp.lam, (size_t)S * N * es) ||
-            !dev_alloc((void **)&jp.cs, (size_t)S * std::max(1, jp.nparam) * 2 * sizeof(double)) ||
-            !dev_alloc(&jp.mats, mat_reals * rs) ||
-            !dev_alloc((void **)&jp.part, total * sizeof(double)) ||
-            !dev_alloc((void **)&jp.obs, bm_obs_partials(jp.n, S) * sizeof(double)))
-            return set_error(QS_ENOMEM, "qs_batch_run: cannot allocate the pass-major state buffers");
+        if (!dev_alloc(&jp.mats, mat_reals * rs) || !dev_alloc((void **)&jp.part, total * sizeof(double)))
+            return set_error(QS_ENOMEM, no_memory);
         qs_status st;
         if ((st = upload(jp.states, (void **)&jp.d_states)) != QS_OK || (st = upload(csr, (void **)&jp.d_csr)) != QS_OK ||
             (st = upload(flat, (void **)&jp.d_items)) != QS_OK || (st = upload(mp, (void **)&jp.d_mpass)) != QS_OK ||
@@ -445,6 +457,7 @@ qs_status qs_batch_create(int num_states, const int *n_qubits, const qs_gate *ga
     std::vector<RegGate> tgates;
     std::vector<TileGroup> tgroups;
     std::map<std::string, int> prog_of;
+    std::vector<double> prog_bytes;
     int max_params = 1, max_large_n = 0, max_small_n = 0, smem_bits = 5;
     char err[256], e2[512];
     for (int s = 0; s < num_states; ++s) {
@@ -510,6 +523,14 @@ qs_status qs_batch_create(int num_states, const int *n_qubits, const qs_gate *ga
             plan_fused(n, dtype, k, seqf, fwdm, nullptr, &pf, max_pass_gates, false, kGroupBits);
             std::reverse(seq.begin(), seq.end());
             plan_fused(n, dtype, k, seq, adj, &slots, &pa, max_pass_gates, false, kGroupBitsAdjoint);
+            double bytes = 0.0;
+            if (!small) {
+                bytes = 3.0;
+                for (size_t i = 0; i < pf.passes.size(); ++i) bytes += 2.0 * pass_touched_fraction(pf, (int)i);
+                for (size_t i = 0; i < pa.passes.size(); ++i) bytes += 4.0 * pass_touched_fraction(pa, (int)i);
+                bytes *= std::ldexp((double)es, n);
+            }
+            prog_bytes.push_back(bytes);
             BatchProg bp{};
             bp.small = small;
             bp.n = n;
@@ -589,6 +610,7 @@ qs_status qs_batch_create(int num_states, const int *n_qubits, const qs_gate *ga
     b->major_f = major_f;
     b->major_a = major_a;
     b->major_gates = major_gates;
+    for (const BatchState &bs : states) b->bytes += prog_bytes[bs.prog];
     // the pass-major path's programs (states above small_bits), compiled on first use
     {
         std::vector<int> jp_of(progs.size(), -1);
@@ -611,9 +633,7 @@ qs_status qs_batch_create(int num_states, const int *n_qubits, const qs_gate *ga
         }
         b->param_off_host.assign(param_offsets, param_offsets + num_states + 1);
     }
-    MajorPlanner planner(b);
     auto fail = [&](qs_status st, const char *what) {
-        planner.join();
         free_batch(b);
         return what ? set_error(st, what) : st;
     };
@@ -637,7 +657,6 @@ qs_status qs_batch_create(int num_states, const int *n_qubits, const qs_gate *ga
         b->queue = nullptr;
         return fail(QS_ENOMEM, "qs_batch_create: cannot allocate the work queue");
     }
-    if (!planner.finish()) return fail(QS_ENOMEM, "qs_batch_create: no host memory for the pass-major programs");
     BatchArgs &a = b->args;
     a.states = static_cast<const BatchState *>(b->d_states);
     a.order = static_cast<const int32_t *>(b->d_order);
@@ -669,6 +688,7 @@ qs_status qs_batch_run(qs_batch *b, const double *theta, double *energy, double 
         qs_status st = ensure_jit(b);
         if (st != QS_OK) return st;
     }
+    b->last_jit = jit;
     auto enqueue = [&](cudaStream_t st) -> cudaError_t {
         if (jit) return enqueue_jit(b, a, st, (flags & QS_FLAG_GRAPH) != 0);
         cudaError_t e1 = cudaMemsetAsync(b->queue, 0, sizeof(int), st);
@@ -733,6 +753,10 @@ qs_status qs_batch_bytes(const qs_batch *b, double *algorithmic_bytes) {
     // states in shared memory move nothing through HBM; a larger state: |0...0> written, every
     // forward pass reads and writes the tiles its gates select, lambda = O psi reads psi and
     // writes lambda, every sweep pass reads and writes the selected tiles of psi and lambda
+    if (!b->last_jit) {
+        *algorithmic_bytes = b->bytes;
+        return QS_OK;
+    }
     double total = 0.0;
     const double es = (double)elem_bytes(b->dtype);
     for (const BatchJitProg &jp : b->jprogs) {

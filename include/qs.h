@@ -205,7 +205,7 @@ qs_status qs_apply_circuit(qs_state *s, const qs_gate *gates, size_t count,
  * register group's row copies. */
 typedef struct {
     int32_t launches;      /* kernel launches */
-    int32_t single_gates;  /* launches of one gate */
+    int32_t single_gates;  /* launches of one gate (sweep: or of a Z and a Y rotation joined) */
     int32_t tile_passes;   /* fused passes over shared-memory tiles */
     int32_t diag_runs;     /* passes that apply a run of diagonal gates */
     int32_t gates;         /* gates after same-target merging (identities included) */
@@ -221,10 +221,10 @@ typedef struct {
                                  matrix, 6 for a one-sided phase, 0 for an exchange; with
                                  QS_FLAG_ADJOINT also the sweep's un-apply of each gate on psi
                                  and on lambda, 8 per pair for each parameterised gate's
-                                 derivative product Im <lambda|P psi> / 2 (P = Y or Z), and 8
-                                 per amplitude for the energy and lambda = O psi. The same with
-                                 and without QS_FLAG_FUSE (the circuit's arithmetic, not a
-                                 kernel's). */
+                                 derivative product Im <lambda|P psi> / 2 (P = Y or Z; 4 where
+                                 one side of Z stands for both), and 8 per amplitude for the
+                                 energy and lambda = O psi. The same with and without
+                                 QS_FLAG_FUSE (the circuit's arithmetic, not a kernel's). */
 } qs_schedule;
 
 qs_status qs_circuit_schedule(int n, qs_dtype dtype, const qs_gate *gates, size_t count,

@@ -453,6 +453,8 @@ cudaError_t launch_obs_energy(const void *psi, void *lam, int n, double *part, c
     return cudaGetLastError();
 }
 
+int grad_final_launches(int most) { return most > 2 ? 2 : 1; }
+
 // energy (may be null): written from the partial sums in row nslots of part. most: the most slots that
 // one parameter has. Its warp reads a row of 1024 partial sums in 1.8 us, and rows follow one another (one
 // parameter for all 320 slots of an n = 20 complex64 gradient: 1758 us, with the rows summed first 1188);
@@ -461,7 +463,7 @@ cudaError_t launch_grad_final(double *part, int nslots, int most, const int *slo
                               double *energy, cudaStream_t st) {
     if (nparams == 0 && !energy) return cudaSuccess;
     const unsigned grid = (unsigned)(((uint64_t)nparams + 1 + 7) / 8);
-    if (most > 2) {
+    if (grad_final_launches(most) > 1) {
         const int rows = nslots + (energy ? 1 : 0);
         k_slot_sums<<<(rows + 7) / 8, 256, 0, st>>>(part, rows);
         const cudaError_t e = cudaGetLastError();

@@ -354,6 +354,8 @@ cudaError_t expect_z_impl(const void *psi, int n, double *scratch, double *out_z
 
 size_t reduce_scratch_doubles(int n) { return (size_t)kRedMaxBlocks * (size_t)(n + 1); }
 
+int expect_z_launches(int dtype, int n) { return n < (dtype == QS_C64 ? RedT<float>::TB : RedT<double>::TB) ? 1 : 2; }
+
 cudaError_t launch_expect_z(int dtype, const void *psi, int n, double *scratch, double *out_z,
                             double *out_norm2, cudaStream_t st) {
     if (dtype == QS_Q30) return launch_expect_z_q30(psi, n, scratch, out_z, out_norm2, st);

@@ -25,6 +25,7 @@ bool adj_steps_join(const GatePlan &z, const GatePlan &y);
 cudaError_t launch_adj_step_zy(int dtype, void *psi, void *lam, const GatePlan &z, const GatePlan &y, double *part_z,
                                double *part_y, cudaStream_t st);
 cudaError_t launch_obs_sumz(const void *psi, void *lam, int n, cudaStream_t st);
+int grad_final_launches(int most);
 cudaError_t launch_sum_vec(const double *z, int n, double *out, cudaStream_t st);
 cudaError_t launch_obs_energy(const void *psi, void *lam, int n, double *part, cudaStream_t st);
 cudaError_t launch_grad_final(double *part, int nslots, int most, const int *slot_param, double *grad, int nparams,
@@ -384,6 +385,14 @@ static qs_status ensure_device(void **buf, size_t *cap, size_t bytes, cudaStream
     return QS_OK;
 }
 
+// Sweep: the plan of the next op if one launch takes it with op `i`, a single parameterised step; else -1.
+static int joined_step(const FusedProgram &prog, size_t i, const std::vector<GatePlan> &plans, const std::vector<int> &slots) {
+    if (i + 1 >= prog.ops.size() || prog.ops[i + 1].pass >= 0 || prog.ops[i + 1].drun >= 0) return -1;
+    const int g = prog.ops[i].gate, next = prog.ops[i + 1].gate;
+    if (slots[g] < 0 || next < 0 || (size_t)next >= plans.size() || slots[next] < 0) return -1;
+    return adj_steps_join(plans[g], plans[next]) ? next : -1;
+}
+
 // Launch a fused program. Forward: `lam` == nullptr. Adjoint: single gates use the sweep
 // kernel with part + slot * P, passes use the adjoint tile kernel.
 static qs_status launch_program(qs_state *s, const FusedProgram &prog, const std::vector<GatePlan> &plans,
@@ -412,15 +421,13 @@ static qs_status launch_program(qs_state *s, const FusedProgram &prog, const std
             e = launch_gate(s->dtype, s->psi, plans[op.gate], st);
         } else {
             const int slot = (*slots)[op.gate];
-            if (slot >= 0 && oi + 1 < prog.ops.size() && prog.ops[oi + 1].pass < 0 && prog.ops[oi + 1].drun < 0) {
-                const int next = prog.ops[oi + 1].gate;
-                if (next >= 0 && (size_t)next < plans.size() && (*slots)[next] >= 0 && adj_steps_join(plans[op.gate], plans[next])) {
-                    e = launch_adj_step_zy(s->dtype, s->psi, lam, plans[op.gate], plans[next], part + (size_t)slot * P,
-                                           part + (size_t)(*slots)[next] * P, st);
-                    if (e != cudaSuccess) return cuda_fail(e, "fused program launch (joined sweep steps)");
-                    ++oi;
-                    continue;
-                }
+            const int next = joined_step(prog, oi, plans, *slots);
+            if (next >= 0) {
+                e = launch_adj_step_zy(s->dtype, s->psi, lam, plans[op.gate], plans[next], part + (size_t)slot * P,
+                                       part + (size_t)(*slots)[next] * P, st);
+                if (e != cudaSuccess) return cuda_fail(e, "fused program launch (joined sweep steps)");
+                ++oi;
+                continue;
             }
             e = launch_adj_step(s->dtype, s->psi, lam, plans[op.gate], slot >= 0 ? part + (size_t)slot * P : nullptr, st);
         }
@@ -674,9 +681,9 @@ qs_status qs_set_tile_bits(qs_dtype dtype, int adjoint, int bits) {
 
 int qs_get_tile_bits(qs_dtype dtype, int adjoint) { return tile_bits(dtype, adjoint != 0); }
 
-// The launches of qs_adjoint_grad: the forward program, the energy reduction and lambda = O psi
-// (one read of psi; one read of psi and a write of lambda), the reverse sweep over psi and lambda
-// (a sweep step or pass reads and writes both vectors), the gradient sums.
+// The launches of qs_adjoint_grad: the forward program, the energy and lambda = O psi (complex64: one read
+// of psi and a write of lambda; complex128: another read for the reduction), the reverse sweep over psi
+// and lambda (a sweep step or pass reads and writes both vectors, two joined steps once), the gradient sums.
 static qs_status adjoint_schedule(const qs_state *shape, const qs_gate *gates, size_t count, const double *theta,
                                   size_t n_theta, int flags, qs_schedule *out) {
     AdjPlan ap;
@@ -691,7 +698,8 @@ static qs_status adjoint_schedule(const qs_state *shape, const qs_gate *gates, s
     auto add_program = [&](const FusedProgram &prog, const std::vector<GatePlan> &plans, double vectors) {
         r.model_cost += prog.model_cost * vectors;
         for (const TilePass &P : prog.passes) r.pass_gates += P.gate_count;
-        for (const FusedOp &op : prog.ops) {
+        for (size_t i = 0; i < prog.ops.size(); ++i) {
+            const FusedOp &op = prog.ops[i];
             if (op.drun >= 0) {
                 ++r.diag_runs;
                 r.algorithmic_bytes += vectors * state_bytes * std::ldexp(2.0, -prog.druns[op.drun].nc.nfix);
@@ -699,8 +707,10 @@ static qs_status adjoint_schedule(const qs_state *shape, const qs_gate *gates, s
                 ++r.tile_passes;
                 r.algorithmic_bytes += vectors * 2.0 * state_bytes * pass_touched_fraction(prog, op.pass);
             } else {
+                const int next = vectors > 1.0 ? joined_step(prog, i, plans, ap.slot_of) : -1;
                 ++r.single_gates;
-                r.algorithmic_bytes += vectors * gate_algorithmic_bytes(plans[op.gate], dtype);
+                r.algorithmic_bytes += vectors * gate_algorithmic_bytes(plans[next >= 0 ? next : op.gate], dtype);
+                if (next >= 0) ++i;
             }
         }
     };
@@ -708,27 +718,31 @@ static qs_status adjoint_schedule(const qs_state *shape, const qs_gate *gates, s
     for (size_t i = 0; i < ap.adj.size(); ++i) {
         const GatePlan &p = ap.adj[i];
         r.algorithmic_flops += 2.0 * gate_algorithmic_flops(p);
-        if (ap.slot_of[i] >= 0) r.algorithmic_flops += 8.0 * std::ldexp(1.0, n - 1 - __builtin_popcountll(p.ctrl_mask));
+        if (ap.slot_of[i] >= 0)
+            r.algorithmic_flops += (p.op == OP_SIDE ? 4.0 : 8.0) * std::ldexp(1.0, n - 1 - __builtin_popcountll(p.ctrl_mask));
     }
     r.algorithmic_flops += 8.0 * std::ldexp(1.0, n);
     if (flags & QS_FLAG_FUSE) {
         add_program(ap.pf, ap.fwd, 1.0);
         add_program(ap.pa, ap.adj, 2.0);
     } else {
-        for (const auto *pl : {&ap.fwd, &ap.adj}) {
-            const double vectors = pl == &ap.adj ? 2.0 : 1.0;
-            for (const GatePlan &p : *pl) {
-                if (p.units == 0 && pl == &ap.fwd) continue;
-                ++r.single_gates;
-                const double b = p.op == OP_SIDE ? 0.5 : 1.0;
-                r.algorithmic_bytes += vectors * b * 2.0 * std::ldexp(dtype == QS_C64 ? 8.0 : 16.0,
-                                                                      n - __builtin_popcountll(p.ctrl_mask));
-                r.model_cost += vectors * (single_launch_cost(p, dtype) + launch_latency_cost(n, dtype));
-            }
+        auto add_step = [&](const GatePlan &p, double vectors) {
+            ++r.single_gates;
+            r.algorithmic_bytes += vectors * gate_algorithmic_bytes(p, dtype);
+            r.model_cost += vectors * (single_launch_cost(p, dtype) + launch_latency_cost(n, dtype));
+        };
+        for (const GatePlan &p : ap.fwd)
+            if (p.units != 0) add_step(p, 1.0);
+        for (size_t i = ap.adj.size(); i-- > 0;) {
+            if (ap.adj[i].units == 0) continue;
+            if (i > 0 && ap.slot_of[i] >= 0 && ap.slot_of[i - 1] >= 0 && adj_steps_join(ap.adj[i], ap.adj[i - 1])) --i;
+            add_step(ap.adj[i], 2.0);  // (joined: the second one's pairs)
         }
     }
-    r.algorithmic_bytes += 3.0 * state_bytes;  // energy: read psi; lambda = O psi: read psi, write lambda
-    r.launches = r.single_gates + r.tile_passes + r.diag_runs + 4;  // + reductions, lambda, gradient sums
+    r.algorithmic_bytes += (dtype == QS_C64 ? 2.0 : 3.0) * state_bytes;
+    r.launches = r.single_gates + r.tile_passes + r.diag_runs;
+    r.launches += dtype == QS_C64 ? 1 : expect_z_launches(dtype, n) + 2;  // energy and lambda
+    if (n_theta > 0 || dtype == QS_C64) r.launches += grad_final_launches(most_uses(ap.slot_param));
     *out = r;
     return QS_OK;
 }

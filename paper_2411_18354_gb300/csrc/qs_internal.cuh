@@ -95,6 +95,7 @@ cudaError_t launch_expect_z_q30(const void *psi, int n, double *scratch, double 
 // Reductions: partial sums per block, then a fixed-order final pass (deterministic).
 // `scratch` must hold reduce_scratch_doubles(n) doubles.
 size_t reduce_scratch_doubles(int n);
+int expect_z_launches(int dtype, int n);  // kernels of the next one
 cudaError_t launch_expect_z(int dtype, const void *psi, int n, double *scratch,
                             double *out_z /*device, n*/, double *out_norm2 /*device, 1*/,
                             cudaStream_t st);

@@ -477,7 +477,7 @@ static void make_pass(int n, uint64_t Lmask, TilePass *P) {
 // arithmetic, ~0.33) gain from a pass.
 // A pass with fewer tiles than SMs leaves the rest idle, and its FP64 work takes as many times longer
 // (13 qubits, 200 gates with 0-3 controls: planned into passes 875 us, apart 465).
-static double pass_gate_cost(int n, int dtype, int k, const GatePlan &p, bool jit) {
+static double pass_gate_cost(int n, int dtype, int k, const GatePlan &p, bool jit, double sms) {
     if (dtype == QS_C64 && !jit) return 0.15;
     if (dtype == QS_C64) {
         // passes compiled for their shape (QS_FLAG_JIT), measured at n = 24 in units of one
@@ -487,7 +487,7 @@ static double pass_gate_cost(int n, int dtype, int k, const GatePlan &p, bool ji
         double c = p.op == OP_GEN ? 0.13 : p.op == OP_REAL ? 0.065 : p.op == OP_SWAP ? 0.04 : 0.035;
         return c * std::max(std::ldexp(1.0, -popc(p.ctrl_mask)), 0.125);
     }
-    return p.op == OP_SWAP ? 0.33 : 3.0 * std::max(1.0, 152.0 * std::ldexp(1.0, -std::max(0, n - k)));
+    return p.op == OP_SWAP ? 0.33 : 3.0 * std::max(1.0, sms * std::ldexp(1.0, -std::max(0, n - k)));
 }
 
 // Compute cost of one diagonal gate inside a k_diag_run launch (its factor is formed once per
@@ -496,10 +496,12 @@ static double pass_gate_cost(int n, int dtype, int k, const GatePlan &p, bool ji
 // point at memory speed: QFT at n = 22, one run per qubit 3.18 ms (144 us each, 6.5 units), every gate
 // alone 1.98 ms.
 // (its blocks hold 2048 amplitudes: below 2^18 amplitudes SMs idle)
-static double diag_run_gate_cost(int n, int dtype) {
-    return dtype == QS_C64 ? 0.005 : 0.35 * std::max(1.0, 152.0 * std::ldexp(1.0, -std::max(0, n - 11)));
+static double diag_run_gate_cost(int n, int dtype, double sms) {
+    return dtype == QS_C64 ? 0.005 : 0.35 * std::max(1.0, sms * std::ldexp(1.0, -std::max(0, n - 11)));
 }
-static double diag_run_lead_cost(int n, int dtype) { return dtype == QS_C64 ? 0.0 : 3.0 * diag_run_gate_cost(n, dtype); }
+static double diag_run_lead_cost(int n, int dtype, double sms) {
+    return dtype == QS_C64 ? 0.0 : 3.0 * diag_run_gate_cost(n, dtype, sms);
+}
 
 enum { SEG_SINGLE, SEG_PASS, SEG_DIAG, SEG_LEAD_DIAG, SEG_NONE };
 
@@ -536,6 +538,8 @@ static void plan_in_order(int n, int dtype, int k, const std::vector<int> &seq, 
     const int b = std::min(k, b0);
     const uint64_t low = (b >= 64) ? ~0ull : ((1ull << b) - 1ull);
     const bool adjoint = gslots != nullptr;
+    const int found = device_sm_count();
+    const double sms = found > 1 ? found : 152;  // (planning on a host without a device: as on a GB300)
     const bool diag_runs = !adjoint && allow_single && n >= kDiagChunkBits;
     auto is_param = [&](int g) { return adjoint && (*gslots)[g] >= 0; };
     const size_t N = seq.size();
@@ -550,7 +554,7 @@ static void plan_in_order(int n, int dtype, int k, const std::vector<int> &seq, 
         tbit_of[j] = real ? (1ull << p.t) : 0ull;
         ctrl_of[j] = p.ctrl_mask;
         param_of[j] = param;
-        cost_of[j] = real ? pass_gate_cost(n, dtype, k, p, jit) * (param && jit ? 1.5 : 1.0) : 0.0;
+        cost_of[j] = real ? pass_gate_cost(n, dtype, k, p, jit, sms) * (param && jit ? 1.5 : 1.0) : 0.0;
     }
     // Take gates seq[i], seq[i + 1], ... (before `end`) into one pass while its targets fit in
     // k local qubits and the gate and parameter limits allow; visit(j, frac, compute, real)
@@ -742,7 +746,7 @@ static void plan_in_order(int n, int dtype, int k, const std::vector<int> &seq, 
         if (diag_runs && p0.units != 0 && is_diag(g0)) {
             diag_span(j, N, false, [&](size_t e, double frac, int real) {
                 if (real < 2) return;
-                const double v = launch_cost + frac + real * diag_run_gate_cost(n, dtype) + best[e + 1];
+                const double v = launch_cost + frac + real * diag_run_gate_cost(n, dtype, sms) + best[e + 1];
                 if (v < bv - 1e-9) {
                     bv = v;
                     bc = e + 1;
@@ -754,7 +758,7 @@ static void plan_in_order(int n, int dtype, int k, const std::vector<int> &seq, 
             !is_diag(g0) && j + 1 < N) {
             diag_span(j + 1, N, true, [&](size_t e, double frac, int real) {
                 if (real < 1) return;
-                const double v = launch_cost + frac + diag_run_lead_cost(n, dtype) + real * diag_run_gate_cost(n, dtype) + best[e + 1];
+                const double v = launch_cost + frac + diag_run_lead_cost(n, dtype, sms) + real * diag_run_gate_cost(n, dtype, sms) + best[e + 1];
                 if (v < bv - 1e-9) {
                     bv = v;
                     bc = e + 1;

@@ -148,7 +148,7 @@ class ClockSampler:
 
 def kernel_source_hash() -> str:
     h = hashlib.sha1()
-    for name in ("k_gate.cuh", "k_gate_dispatch.cuh", "qs_plan.cu", "qs_api.cu"):
+    for name in ("k_gate.cuh", "k_fx.cuh", "k_gate_dispatch.cuh", "qs_internal.cuh", "qs_plan.cu", "qs_api.cu"):
         with open(os.path.join(ROOT, "paper_2411_18354_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:12]

@@ -39,9 +39,9 @@
 // RY 1.1e-16 (2.2e-16), RZ RY 1.2e-16 (3.8e-16).
 //
 // Measured, uncontrolled gate at n = 28 on target 14 (8.6 GB moved, a copy of the same bytes 1.35 ms;
-// float64 form: general 4.3 ms, diagonal 2.2, one-sided 1.1): FX_GEN 1.41 ms, FX_GENP 1.97, with the
-// one-scale test on random amplitudes 1.56, RX 1.51; real 1.36; diagonal 1.43 (own scales 1.43);
-// one-sided 0.67 (own scales 0.70). FX_GENP is bound by the integer pipe (16 shifts of 64 bits more).
+// float64 form: general 4.3 ms, diagonal 2.2, one-sided 1.1): FX_GEN 1.41 ms, FX_GENP 1.87, with the
+// one-scale test on random amplitudes 1.44, RX 1.46; real 1.36; diagonal 1.43 (own scales 1.43);
+// one-sided 0.67 (own scales 0.70). FX_GENP has 16 shifts of 64 bits more than FX_GEN.
 #pragma once
 
 #include <algorithm>

@@ -47,10 +47,11 @@ cudaError_t go(void *psi, const GatePlan &p, const FxMat &fx, uint64_t cmask, ui
     // complex64, target 14, 1 / 2 / 4 / 8 units 1.35 / 1.43 / 1.34 / 1.32 ms. Single amplitudes (an inserted
     // qubit 0: isolated 8 bytes) keep 2: X on q controlled by every lower qubit, q = 0..28, 1 / 2 / 4 units
     // 7.10 / 7.14 / 7.60 ms (q = 1 alone 1.52 / 1.46 / 1.53). complex128 exchanges take 1: n = 28, target 14,
-    // 1 / 2 / 4 units 1.33 / 1.55 / 1.33 ms, X controlled by every lower qubit 5.56 / 5.86 / 5.64.
+    // 1 / 2 / 4 units 1.33 / 1.55 / 1.33 ms, X controlled by every lower qubit 5.56 / 5.86 / 5.64 (slower with 1
+    // are targets 1 to 3 and 5 with a control: 0.69 / 0.67 / 0.67; adjacent pairs take 4).
     // complex128 arithmetic (one 16-byte vector per amplitude; n = 28, target 14, 1 / 2 / 4 units): general
-    // 1.38 / 1.39 / 1.36 ms, real 1.40 / 1.39 / 1.35, parts of unlike size 1.97 / 1.90 / 1.94 (but n = 20: 9.1 /
-    // 10.0 / 10.3 us), diagonal 1.39 / 1.41 / 1.40, one-sided 0.67 / 0.72 / 0.72.
+    // 1.38 / 1.39 / 1.36 ms, real 1.40 / 1.39 / 1.35, parts of unlike size 1.97 / 1.90 / 1.94 (at five blocks
+    // per SM; n = 20: 9.1 / 10.0 / 10.3 us), diagonal 1.39 / 1.41 / 1.40, one-sided 0.67 / 0.72 / 0.72.
     constexpr bool pair_unit = LAY == LAY_ADJ || OP == OP_SIDE;  // one vector per unit
     constexpr int UNR = sizeof(Real) == 4 ? (pair_unit || (OP == OP_SWAP && R == 2) ? 4 : 2)
                         : OP == OP_SWAP   ? (pair_unit ? 4 : 1)

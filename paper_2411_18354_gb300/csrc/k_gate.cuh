@@ -251,9 +251,9 @@ template <> struct Log2<4> { static constexpr int v = 2; };
 //             amplitude fails the control test return without touching memory.
 // complex128 matrices with parts of unlike size wait on chains of shifts, not on one pipe (ALU 60 % busy, 5
 // blocks of 42 registers per SM): eight blocks of 32 registers, n = 28, target 14, near-diagonal 1.97 -> 1.87 ms, a
-// Haar matrix with a small part 1.56 -> 1.44, rotation about X 1.51 -> 1.46.
+// Haar matrix with a small part 1.56 -> 1.44, rotation about X 1.51 -> 1.46. (0: no bound for the others.)
 template <typename Real, typename Idx, int NS, int LAY, int R, int OP, bool MASKED, int UNR>
-__global__ void __launch_bounds__(kGateThreads, sizeof(Real) == 8 && OP == OP_GENP ? 8 : 1)
+__global__ void __launch_bounds__(kGateThreads, sizeof(Real) == 8 && OP == OP_GENP ? 8 : 0)
 k_gate(typename CxT<Real>::T *__restrict__ psi, const DevGate<Real, Idx> g, Idx units, int side) {
     using T2 = typename CxT<Real>::T;
     constexpr int r = Log2<R>::v;

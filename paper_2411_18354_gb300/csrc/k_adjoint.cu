@@ -127,7 +127,8 @@ k_adj_step(typename CxT<Real>::T *__restrict__ psi, typename CxT<Real>::T *__res
 // gz), then a Y rotation (g); one read and write of psi and lambda and one launch instead of two (an
 // ansatz layer applies RY and RZ to every qubit). n = 20 complex128,
 // 8-layer gradient: 7.27 -> 5.81 ms (with half of the real update's conversions on the integer pipe
-// and two blocks per SM for the tile sweep).
+// and two blocks per SM for the tile sweep); 5.94 with a scale of its own for every part of small phases.
+// Bound by the FP64 pipe (77 % busy): six multiply-adds of the derivative products and the other conversions.
 template <typename Real, typename Idx, int NS, int LAY, int R>
 __global__ void __launch_bounds__(kGateThreads)
 k_adj_step_zy(typename CxT<Real>::T *__restrict__ psi, typename CxT<Real>::T *__restrict__ lam,

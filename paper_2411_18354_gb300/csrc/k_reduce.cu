@@ -25,7 +25,8 @@
 // sums per 16 values become float64 and are added there. The warp-level sums are formed once per
 // run of 2^m consecutive tiles (the low m tile bits have per-thread sums of their own). n = 28:
 // 2.72 -> 0.80 ms (5.4 TB/s), error against exact arithmetic as before (1-2 units in the last place);
-// a basis state, whose zeros add nothing, 2.74 -> 0.63.
+// a basis state, whose zeros add nothing, 2.74 -> 0.63. What is left in float64 keeps that pipe 61 % busy, with
+// two blocks of 126 registers per SM.
 #include <algorithm>
 
 #include "k_gate.cuh"

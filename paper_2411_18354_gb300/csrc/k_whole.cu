@@ -8,8 +8,8 @@
 // a gate with nothing else on the SM to hide it. Here a gate is a few dozen instructions that stay in
 // the cache, its descriptor was read while the previous gate ran, and a gate with c controls touches 2^-c of the state; what is left is the shared-memory
 // traffic (4096 amplitudes read and written: 512 clocks) and a barrier per gate.
-// 200 gates with 0-3 controls, complex64: 12 qubits 129 -> 87 us, 10 qubits 110 -> 57; complex128, 10
-// qubits: 705 -> 157.
+// 200 gates with 0-3 controls, complex64: 12 qubits 129 -> 87 us, 10 qubits 110 -> 56; complex128, 10
+// qubits: 705 -> 160.
 #include <algorithm>
 #include <cstring>
 

@@ -40,8 +40,10 @@ class AdjointEnergy(torch.autograd.Function):
         # the gate matrices are built on the host from theta: this copy is the call's only
         # host round trip; energy and gradient are written to device tensors on torch's current
         # stream without waiting
-        # (converted by torch, after the copy: numpy has no bfloat16)
-        th = theta.detach().cpu().to(torch.float64).numpy()
+        th = theta.detach().cpu()
+        if th.dtype not in (torch.float64, torch.float32):  # numpy has no bfloat16
+            th = th.to(torch.float64)
+        th = th.numpy().astype(np.float64, copy=False)
         st = _state(n, dtype, theta.device)
         _lib.qs_state_set_stream(st.h, int(torch.cuda.current_stream(theta.device).cuda_stream))
         st.set_basis(0)

@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <mutex>
 #include <vector>
 
@@ -525,7 +526,10 @@ static void plan_adjoint_programs(const qs_state *s, int flags, AdjPlan *ap) {
 }
 
 // How often the most used parameter occurs.
-static int most_uses(std::vector<int> params) {
+static int most_uses(const std::vector<int> &slot_param) {
+    if (std::adjacent_find(slot_param.begin(), slot_param.end(), std::greater_equal<int>()) == slot_param.end())
+        return slot_param.empty() ? 0 : 1;  // ascending: each its own
+    std::vector<int> params = slot_param;
     std::sort(params.begin(), params.end());
     int most = 0;
     for (size_t i = 0, j; i < params.size(); i = j) {

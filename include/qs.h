@@ -153,7 +153,9 @@ qs_status qs_state_synchronize(const qs_state *s);
  * target is out of range, the mask holds the target or bits >= n, ctrl_vals has bits
  * outside the mask, or U holds a NaN/Inf. Exact structure in U is used: [[0,1],[1,0]]
  * runs the exchange path (bit-exact), b = c = 0 runs a diagonal path, and a diagonal with
- * a == 1 (or d == 1) touches only the amplitudes it changes. */
+ * a == 1 (or d == 1) touches only the amplitudes it changes. complex128 results: each real or
+ * imaginary part within 2^-50 of the sum of the magnitudes of its four real products, as in
+ * float64 arithmetic (which is used, per pair, where exponents leave fixed point no room). */
 qs_status qs_apply_gate(qs_state *s, int target, uint64_t ctrl_mask, uint64_t ctrl_vals,
                         const double U[8]);
 
